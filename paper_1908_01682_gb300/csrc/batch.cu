@@ -55,8 +55,7 @@ template <class T> struct BInst {
     Geo<T> G;          // geometry of the instance (its own cell grid)
     Phys<T> Ph;
     T hi[3];           // upper box corner, for the input check
-    double tau;        // step of the instance
-    double g[3];
+    StepVals step;     // tau and g of the instance
     uint32_t coff;     // first cell in the batch key space
     uint32_t goff, ng; // gas slots [goff, goff + ng)
     uint32_t doff, nd; // dust slots
@@ -464,15 +463,12 @@ __device__ void ph_update(const BatchArgs<T> &B, int q, BInst<T> &si, unsigned c
         __syncthreads();
         load_inst(&B.inst[ch.inst], si);
         __syncthreads();
-        const A tau = A(si.tau);
-        const A gv[3] = {A(si.g[0]), A(si.g[1]), A(si.g[2])};
         const uint32_t cell = ch.begin + threadIdx.x;
         int drag = 0;
         if (cell < ch.end) {
             T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
-            drag = cell_drag_solve<T, A, DIM>(si.Ph, tau, gv, B.harmonic, si.has_frozen, gvel, gid, B.acc,
-                                              B.gstart[cell], B.gstart[cell + 1], dvel, B.dstart[cell],
-                                              B.dstart[cell + 1], un, vn, ig, id);
+            drag = cell_drag<T, A, DIM>(si.Ph, si.step, B.harmonic, si.has_frozen, gvel, gid, B.acc, B.gstart[cell],
+                                        B.gstart[cell + 1], dvel, B.dstart[cell], B.dstart[cell + 1], un, vn, ig, id);
             if (drag) {
 #pragma unroll
                 for (int k = 0; k < DIM; ++k) {
@@ -486,8 +482,9 @@ __device__ void ph_update(const BatchArgs<T> &B, int q, BInst<T> &si, unsigned c
         s_drag[threadIdx.x] = drag;
         __syncthreads();
         const uint32_t c0 = ch.begin - si.coff, ncc = ch.end - ch.begin;
-        const T tau_t = T(tau);
-        const T gt[3] = {T(gv[0]), T(gv[1]), T(gv[2])};
+        const T tau_t = step_val<T>(si.step.tau, si.step.dtau);
+        const T gt[3] = {step_val<T>(si.step.g[0], si.step.dg[0]), step_val<T>(si.step.g[1], si.step.dg[1]),
+                         step_val<T>(si.step.g[2], si.step.dg[2])};
         const int adiabatic = si.Ph.eos == TFSPH_EOS_ADIABATIC;
         for (uint32_t a = B.gstart[ch.begin] + threadIdx.x; a < B.gstart[ch.end]; a += bd) {
             V4<T> p = gpos[a];
@@ -610,9 +607,9 @@ void *pick_persistent(int dim, bool fp64_cells, bool full)
 #define TF_P(A, D)                                                                         \
     return full ? persistent_fn<A, D, 3>() : persistent_fn<A, D, 2>();
     if (fp64_cells) {
-        if (dim == 1) { TF_P(double, 1) }
-        if (dim == 2) { TF_P(double, 2) }
-        TF_P(double, 3)
+        if (dim == 1) { TF_P(df, 1) }
+        if (dim == 2) { TF_P(df, 2) }
+        TF_P(df, 3)
     }
     if (dim == 1) { TF_P(float, 1) }
     if (dim == 2) { TF_P(float, 2) }
@@ -852,9 +849,9 @@ cudaError_t launch_update(const tfsph_batch *b, const BatchArgs<Tf> &B, cudaStre
     const size_t sm = update_smem(b->block);
     if (b->fp64_cells) {
         switch (b->dim) {
-            case 1: k_b_update<double, 1><<<B.ncch, b->block, sm, s>>>(B); break;
-            case 2: k_b_update<double, 2><<<B.ncch, b->block, sm, s>>>(B); break;
-            default: k_b_update<double, 3><<<B.ncch, b->block, sm, s>>>(B); break;
+            case 1: k_b_update<df, 1><<<B.ncch, b->block, sm, s>>>(B); break;
+            case 2: k_b_update<df, 2><<<B.ncch, b->block, sm, s>>>(B); break;
+            default: k_b_update<df, 3><<<B.ncch, b->block, sm, s>>>(B); break;
         }
     } else {
         switch (b->dim) {
@@ -1113,7 +1110,6 @@ int tfsph_batch_init(tfsph_batch **out, const tfsph_params *params, const int64_
         const uint32_t nc = cell_grid(p, nc3);
         make_geo_phys<Tf>(p, nc3, nc, I.G, I.Ph);
         for (int d = 0; d < 3; ++d) I.hi[d] = d < p.dim ? (Tf)p.hi[d] : Tf(1);
-        I.tau = 0.0;
         I.coff = coff;
         I.goff = goff;
         I.ng = (uint32_t)n_gas[i];
@@ -1276,16 +1272,18 @@ int tfsph_batch_step(tfsph_batch *b, const double *tau, const double *g, int32_t
     bool changed = false;
     for (int i = 0; i < b->n_inst; ++i) {
         BInst<Tf> &I = b->hinst[i];
+        double t = I.step.dtau, gi[3] = {I.step.dg[0], I.step.dg[1], I.step.dg[2]};
         if (tau) {
             if (!std::isfinite(tau[i]) || !(tau[i] > 0)) return bfail(b, TFSPH_E_INVALID_ARG, "tau must be finite and > 0");
-            if (I.tau != tau[i]) { I.tau = tau[i]; changed = true; }
+            if (I.step.dtau != tau[i]) { t = tau[i]; changed = true; }
         }
         if (g)
             for (int k = 0; k < 3; ++k) {
                 const double v = k < b->dim ? g[3 * i + k] : 0.0;
                 if (!std::isfinite(v)) return bfail(b, TFSPH_E_NONFINITE, "non-finite gravity");
-                if (I.g[k] != v) { I.g[k] = v; changed = true; }
+                if (gi[k] != v) { gi[k] = v; changed = true; }
             }
+        I.step = step_vals(t, gi);
     }
     b->tau_set = true;
     if (changed) {

@@ -3,7 +3,8 @@
 //
 // One CTA owns kCellsPerCta consecutive cells and, because particles are
 // stored in cell order, the contiguous gas and dust ranges of those cells.
-//   Phase 1 (thread per cell, accumulator type A): N, L, sum v, sum u,
+//   Phase 1 (thread per cell, accumulator type A: float, double, or df, the
+//   two-float form of double that the FP32 state takes): N, L, sum v, sum u,
 //     sum A, sum t_j (or sum 1/t_j) in storage order, then
 //       eps* = m_d L / (m_g N)                                (Eq. 17)
 //       t*   = sum t_j / L   (or L / sum 1/t_j)               (Eq. 18)
@@ -25,9 +26,11 @@
 namespace tfsph {
 namespace {
 
+// (FP32 state, 101^3 cells: 66 us with df against 202 us in binary64, whose
+// pipe was 84 % busy.)
 template <class T, class A, int DIM, bool EST>
-__global__ void __launch_bounds__(kCellsPerCta, (sizeof(T) == 4 && sizeof(A) == 4) ? 12 : 1)
-k_cell_update(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int has_frozen, int adiabatic,
+__global__ void __launch_bounds__(kCellsPerCta, (sizeof(T) == 4 && sizeof(A) == 4) ? 12 : (sizeof(T) == 4 ? 8 : 1))
+k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, int adiabatic,
               V4<T> *__restrict__ gpos, V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
               uint32_t *__restrict__ gkey, const uint32_t *__restrict__ gstart, const V4<T> *__restrict__ acc,
               V4<T> *__restrict__ dpos, V4<T> *__restrict__ dvel, uint32_t *__restrict__ dkey,
@@ -42,14 +45,13 @@ k_cell_update(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int h
     const uint32_t ncells = G.ncells;
     const uint32_t c0 = blockIdx.x * kCellsPerCta;
     const uint32_t c = c0 + threadIdx.x;
-    const A gv[3] = {g0, g1, g2};
 
     // ---- phase 1: per-cell sums and the implicit solve ----
     int drag = 0;
     if (c < ncells) {
         T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
-        drag = cell_drag_solve<T, A, DIM>(Ph, tau, gv, harmonic, has_frozen, gvel, gid, acc, gstart[c],
-                                          gstart[c + 1], dvel, dstart[c], dstart[c + 1], un, vn, ig, id);
+        drag = cell_drag<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gstart[c], gstart[c + 1], dvel,
+                                    dstart[c], dstart[c + 1], un, vn, ig, id);
         if (drag) {
 #pragma unroll
             for (int k = 0; k < DIM; ++k) {
@@ -65,8 +67,8 @@ k_cell_update(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int h
 
     // ---- phase 2: particle updates over the CTA's storage ranges ----
     const uint32_t c1 = min(c0 + (uint32_t)kCellsPerCta, ncells);
-    const T tau_t = T(tau);
-    const T gt[3] = {T(g0), T(g1), T(g2)};
+    const T tau_t = step_val<T>(S.tau, S.dtau);
+    const T gt[3] = {step_val<T>(S.g[0], S.dg[0]), step_val<T>(S.g[1], S.dg[1]), step_val<T>(S.g[2], S.dg[2])};
     {
         const uint32_t a0 = gstart[c0], a1 = gstart[c1];
         for (uint32_t a = a0 + threadIdx.x; a < a1; a += blockDim.x) {
@@ -122,14 +124,151 @@ k_cell_update(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int h
 //   u_j' = v*' + (u_j + tau g - v*') id              id = 1/(1 + rt)
 //   v*' = u*' + w',  u*' = ubar + tau g + rt w',  w' = (vbar - ubar + tau Abar)/den,
 //   den = 1 + rt (1 + eps),  rt = tau / t*,  t* = mean (or harmonic mean) of t_j.
+struct CellRange {
+    uint32_t gs, ge, ds, de;  // the cell's gas and dust slots
+};
+// What a cell hands its particles: ig, id, lambda_t*, t*, L, then per axis
+// the lambdas of vbar, Abar (per gas particle) and ubar (per dust particle).
+template <class T> struct CellLam {
+    T ig, id, lt, tst, L, lv[3], lA[3], lu[3];
+};
+
+// One cell's reverse solve with accumulator A; 0 without drag, 2 when df's
+// range may not hold it (the bounds of cell_drag_solve, on the lambdas too).
+template <class T, class A, int DIM>
+__device__ __forceinline__ int cell_adjoint_solve(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
+                                                  const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                                  const V4<T> *__restrict__ acc, const V4<T> *__restrict__ dvel,
+                                                  const V4<T> *__restrict__ lgx, const V4<T> *lgv,
+                                                  const V4<T> *__restrict__ ldx, const V4<T> *ldu, const CellRange &R,
+                                                  CellLam<T> &O)
+{
+    constexpr bool kPair = std::is_same<A, df>::value;
+    const A one = A(1.0f), zero = A(0.0f);
+    const A tau = step_val<A>(S.tau, S.dtau);
+    A gv[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) gv[k] = step_val<A>(S.g[k], S.dg[k]);
+    uint32_t ng = 0, nd = 0;
+    A st = zero;
+    A sv[3] = {zero, zero, zero}, sa[3] = {zero, zero, zero}, su[3] = {zero, zero, zero};
+    auto add = [](A &s, T x) {
+        if constexpr (kPair) s += (float)x;
+        else s += A(x);
+    };
+    for (uint32_t a = R.gs; a < R.ge; ++a) {
+        if (has_frozen && (gid[a] & kFrozenBit)) continue;
+        const V4<T> v = gvel[a];
+        const V4<T> ac = acc[a];
+        ++ng;
+        add(sv[0], v.x);
+        add(sa[0], ac.x);
+        if (DIM > 1) { add(sv[1], v.y); add(sa[1], ac.y); }
+        if (DIM > 2) { add(sv[2], v.z); add(sa[2], ac.z); }
+    }
+    for (uint32_t j = R.ds; j < R.de; ++j) {
+        const V4<T> u = dvel[j];
+        ++nd;
+        add(su[0], u.x);
+        if (DIM > 1) add(su[1], u.y);
+        if (DIM > 2) add(su[2], u.z);
+        if (harmonic) st += one / A(u.w);
+        else add(st, u.w);
+    }
+    if (ng == 0 || nd == 0) return 0;
+    const A N = A(ng), L = A(nd);
+    const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
+    const A tst = harmonic ? L / st : st / L;
+    const A rt = tau / tst;
+    const A den = one + rt * (one + eps);
+    const A ig = one / (one + rt * eps), id = one / (one + rt);
+    bool fits = true;
+    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    A wn[3] = {zero, zero, zero}, un[3] = {zero, zero, zero}, vn[3] = {zero, zero, zero};
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        wn[k] = ((sv[k] / N - su[k] / L) + tau * (sa[k] / N)) / den;
+        un[k] = su[k] / L + tau * gv[k] + rt * wn[k];
+        vn[k] = un[k] + wn[k];
+        if constexpr (kPair)
+            fits = fits && !df_small(wn[k]) && !df_small(un[k]) && !df_small(vn[k]) &&
+                   df_in(un[k], -0x1p60f, 0x1p60f) && df_in(vn[k], -0x1p60f, 0x1p60f);
+    }
+    // sums over the cell's particles of the lambdas reaching u*', v*', ig, id
+    A S_un[3] = {zero, zero, zero}, S_vn[3] = {zero, zero, zero}, S_ig = zero, S_id = zero;
+    for (uint32_t a = R.gs; a < R.ge; ++a) {
+        if (has_frozen && (gid[a] & kFrozenBit)) continue;
+        const V4<T> v = gvel[a], ac = acc[a], lx = lgx[a], lv = lgv[a];
+        const T vv[3] = {v.x, v.y, v.z}, aa[3] = {ac.x, ac.y, ac.z}, xx[3] = {lx.x, lx.y, lx.z},
+                ll[3] = {lv.x, lv.y, lv.z};
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            const A l = A(ll[k]) + tau * A(xx[k]);
+            S_un[k] += (one - ig) * l;
+            S_ig += (A(vv[k]) + tau * (A(aa[k]) + gv[k]) - un[k]) * l;
+        }
+    }
+    for (uint32_t j = R.ds; j < R.de; ++j) {
+        const V4<T> u = dvel[j], lx = ldx[j], lu = ldu[j];
+        const T uu[3] = {u.x, u.y, u.z}, xx[3] = {lx.x, lx.y, lx.z}, ll[3] = {lu.x, lu.y, lu.z};
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) {
+            const A l = A(ll[k]) + tau * A(xx[k]);
+            S_vn[k] += (one - id) * l;
+            S_id += (A(uu[k]) + tau * gv[k] - vn[k]) * l;
+        }
+    }
+    A l_rt = zero, l_den = zero;
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        const A l_vn = S_vn[k];
+        const A l_un = S_un[k] + l_vn;
+        const A l_wn = l_vn + rt * l_un;
+        l_rt += wn[k] * l_un;
+        const A l_w = l_wn / den;
+        l_den -= wn[k] * l_wn / den;
+        O.lv[k] = T(l_w / N);               // lambda of vbar, per gas particle
+        O.lA[k] = T(tau * l_wn / den / N);  // lambda of Abar, per gas particle
+        O.lu[k] = T((l_un - l_w) / L);      // lambda of ubar, per dust particle
+        if constexpr (kPair)
+            fits = fits && !df_small(l_vn) && !df_small(l_un) && !df_small(l_wn) && df_in(l_un, -0x1p60f, 0x1p60f) &&
+                   df_in(l_wn, -0x1p60f, 0x1p60f);
+    }
+    l_rt += (one + eps) * l_den;
+    l_rt -= eps * ig * ig * S_ig;
+    l_rt -= id * id * S_id;
+    const A lt = -(rt / tst) * l_rt;
+    if constexpr (kPair)
+        fits = fits && !df_small(S_ig) && !df_small(S_id) && !df_small(l_rt) && df_in(l_rt, -0x1p60f, 0x1p60f) &&
+               df_in(lt, -0x1p100f, 0x1p100f);
+    O.lt = T(lt);  // lambda of t*
+    O.ig = T(ig);
+    O.id = T(id);
+    O.tst = T(tst);
+    O.L = T(L);
+    return fits ? 1 : 2;
+}
+
+// Its binary64 form for the cells outside df's range, out of line.
+template <class T, int DIM>
+__device__ __noinline__ int cell_adjoint_wide(const Phys<T> Ph, const StepVals S, int harmonic, int has_frozen,
+                                              const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                              const V4<T> *__restrict__ acc, const V4<T> *__restrict__ dvel,
+                                              const V4<T> *__restrict__ lgx, const V4<T> *lgv,
+                                              const V4<T> *__restrict__ ldx, const V4<T> *ldu, const CellRange R,
+                                              CellLam<T> *O)
+{
+    return cell_adjoint_solve<T, double, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu, R,
+                                              *O);
+}
+
 template <class T, class A, int DIM>
 __global__ void __launch_bounds__(kCellsPerCta)
-k_cell_adjoint(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int has_frozen,
+k_cell_adjoint(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen,
                const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid, const uint32_t *__restrict__ gstart,
                const V4<T> *__restrict__ acc, const V4<T> *__restrict__ gpos, const V4<T> *__restrict__ dvel,
                const V4<T> *__restrict__ dpos, const uint32_t *__restrict__ dstart, const V4<T> *__restrict__ lgx,
-               V4<T> *__restrict__ lgv, const V4<T> *__restrict__ ldx, V4<T> *__restrict__ ldu,
-               V4<T> *__restrict__ lA, T *__restrict__ lts)
+               V4<T> *lgv, const V4<T> *__restrict__ ldx, V4<T> *ldu, V4<T> *__restrict__ lA, T *__restrict__ lts)
 {
     __shared__ T s_ig[kCellsPerCta], s_id[kCellsPerCta], s_lt[kCellsPerCta], s_tst[kCellsPerCta], s_L[kCellsPerCta];
     __shared__ T s_lv[3][kCellsPerCta], s_lA[3][kCellsPerCta], s_lu[3][kCellsPerCta];
@@ -138,91 +277,39 @@ k_cell_adjoint(Geo<T> G, Phys<T> Ph, A tau, A g0, A g1, A g2, int harmonic, int 
     const uint32_t ncells = G.ncells;
     const uint32_t c0 = blockIdx.x * kCellsPerCta;
     const uint32_t c = c0 + threadIdx.x;
-    const A gv[3] = {g0, g1, g2};
     int drag = 0;
     if (c < ncells) {
-        const uint32_t gs = gstart[c], ge = gstart[c + 1];
-        const uint32_t ds = dstart[c], de = dstart[c + 1];
-        A N = A(0), L = A(0), st = A(0);
-        A sv[3] = {A(0), A(0), A(0)}, sa[3] = {A(0), A(0), A(0)}, su[3] = {A(0), A(0), A(0)};
-        for (uint32_t a = gs; a < ge; ++a) {
-            if (has_frozen && (gid[a] & kFrozenBit)) continue;
-            const V4<T> v = gvel[a];
-            const V4<T> ac = acc[a];
-            N += A(1);
-            sv[0] += A(v.x); sa[0] += A(ac.x);
-            if (DIM > 1) { sv[1] += A(v.y); sa[1] += A(ac.y); }
-            if (DIM > 2) { sv[2] += A(v.z); sa[2] += A(ac.z); }
+        const CellRange R{gstart[c], gstart[c + 1], dstart[c], dstart[c + 1]};
+        CellLam<T> O;
+        drag = cell_adjoint_solve<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu, R,
+                                             O);
+        if constexpr (std::is_same<A, df>::value) {
+            if (drag == 2) {
+                CellLam<T> W;
+                drag = cell_adjoint_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu,
+                                                 R, &W);
+                O = W;
+            }
         }
-        for (uint32_t j = ds; j < de; ++j) {
-            const V4<T> u = dvel[j];
-            L += A(1);
-            su[0] += A(u.x);
-            if (DIM > 1) su[1] += A(u.y);
-            if (DIM > 2) su[2] += A(u.z);
-            st += harmonic ? A(1) / A(u.w) : A(u.w);
-        }
-        drag = (N > A(0) && L > A(0)) ? 1 : 0;
         if (drag) {
-            const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
-            const A tst = harmonic ? L / st : st / L;
-            const A rt = tau / tst;
-            const A den = A(1) + rt * (A(1) + eps);
-            const A ig = A(1) / (A(1) + rt * eps), id = A(1) / (A(1) + rt);
-            A wn[3] = {A(0), A(0), A(0)}, un[3] = {A(0), A(0), A(0)}, vn[3] = {A(0), A(0), A(0)};
+#pragma unroll
             for (int k = 0; k < DIM; ++k) {
-                wn[k] = ((sv[k] / N - su[k] / L) + tau * (sa[k] / N)) / den;
-                un[k] = su[k] / L + tau * gv[k] + rt * wn[k];
-                vn[k] = un[k] + wn[k];
+                s_lv[k][threadIdx.x] = O.lv[k];
+                s_lA[k][threadIdx.x] = O.lA[k];
+                s_lu[k][threadIdx.x] = O.lu[k];
             }
-            // sums over the cell's particles of the lambdas reaching u*', v*', ig, id
-            A S_un[3] = {A(0), A(0), A(0)}, S_vn[3] = {A(0), A(0), A(0)}, S_ig = A(0), S_id = A(0);
-            for (uint32_t a = gs; a < ge; ++a) {
-                if (has_frozen && (gid[a] & kFrozenBit)) continue;
-                const V4<T> v = gvel[a], ac = acc[a], lx = lgx[a], lv = lgv[a];
-                const A l[3] = {A(lv.x) + tau * A(lx.x), A(lv.y) + tau * A(lx.y), A(lv.z) + tau * A(lx.z)};
-                const A vv[3] = {A(v.x), A(v.y), A(v.z)}, aa[3] = {A(ac.x), A(ac.y), A(ac.z)};
-                for (int k = 0; k < DIM; ++k) {
-                    S_un[k] += (A(1) - ig) * l[k];
-                    S_ig += (vv[k] + tau * (aa[k] + gv[k]) - un[k]) * l[k];
-                }
-            }
-            for (uint32_t j = ds; j < de; ++j) {
-                const V4<T> u = dvel[j], lx = ldx[j], lu = ldu[j];
-                const A l[3] = {A(lu.x) + tau * A(lx.x), A(lu.y) + tau * A(lx.y), A(lu.z) + tau * A(lx.z)};
-                const A uu[3] = {A(u.x), A(u.y), A(u.z)};
-                for (int k = 0; k < DIM; ++k) {
-                    S_vn[k] += (A(1) - id) * l[k];
-                    S_id += (uu[k] + tau * gv[k] - vn[k]) * l[k];
-                }
-            }
-            A l_rt = A(0), l_den = A(0);
-            for (int k = 0; k < DIM; ++k) {
-                const A l_vn = S_vn[k];
-                const A l_un = S_un[k] + l_vn;
-                const A l_wn = l_vn + rt * l_un;
-                l_rt += wn[k] * l_un;
-                const A l_w = l_wn / den;
-                l_den -= wn[k] * l_wn / den;
-                s_lv[k][threadIdx.x] = T(l_w / N);                 // lambda of vbar, per gas particle
-                s_lA[k][threadIdx.x] = T(tau * l_wn / den / N);    // lambda of Abar, per gas particle
-                s_lu[k][threadIdx.x] = T((l_un - l_w) / L);        // lambda of ubar, per dust particle
-            }
-            l_rt += (A(1) + eps) * l_den;
-            l_rt -= eps * ig * ig * S_ig;
-            l_rt -= id * id * S_id;
-            s_lt[threadIdx.x] = T(-(rt / tst) * l_rt);             // lambda of t*
-            s_ig[threadIdx.x] = T(ig);
-            s_id[threadIdx.x] = T(id);
-            s_tst[threadIdx.x] = T(tst);
-            s_L[threadIdx.x] = T(L);
+            s_lt[threadIdx.x] = O.lt;
+            s_ig[threadIdx.x] = O.ig;
+            s_id[threadIdx.x] = O.id;
+            s_tst[threadIdx.x] = O.tst;
+            s_L[threadIdx.x] = O.L;
         }
     }
     s_drag[threadIdx.x] = drag;
     __syncthreads();
 
     const uint32_t c1 = min(c0 + (uint32_t)kCellsPerCta, ncells);
-    const T tau_t = T(tau);
+    const T tau_t = step_val<T>(S.tau, S.dtau);
     for (uint32_t a = gstart[c0] + threadIdx.x; a < gstart[c1]; a += blockDim.x) {
         V4<T> la;
         la.x = la.y = la.z = la.w = T(0);
@@ -282,7 +369,7 @@ cudaError_t cell_adjoint_t(const LaunchCtx &L, const void *geo, const void *phys
     const Phys<T> &Ph = *static_cast<const Phys<T> *>(phys);
     const uint32_t blocks = (Gg.ncells + kCellsPerCta - 1) / kCellsPerCta;
     k_cell_adjoint<T, A, DIM><<<blocks, kCellsPerCta, 0, L.stream>>>(
-        Gg, Ph, A(S.tau), A(S.g[0]), A(S.g[1]), A(S.g[2]), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
+        Gg, Ph, step_vals(S.tau, S.g), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
         static_cast<const V4<T> *>(G.vel[G.cur]), G.id[G.cur], G.start, static_cast<const V4<T> *>(acc),
         static_cast<const V4<T> *>(G.pos[G.cur]), static_cast<const V4<T> *>(D.vel[D.cur]),
         static_cast<const V4<T> *>(D.pos[D.cur]), D.start, static_cast<const V4<T> *>(lgx), static_cast<V4<T> *>(lgv),
@@ -313,7 +400,7 @@ cudaError_t cell_update_t(const LaunchCtx &L, const void *geo, const void *phys,
     for (int d = 0; d < DIM; ++d) est = est && Gg.est_exact[d];
     auto kern = est ? k_cell_update<T, A, DIM, true> : k_cell_update<T, A, DIM, false>;
     kern<<<blocks, kCellsPerCta, 0, L.stream>>>(
-        Gg, Ph, A(S.tau), A(S.g[0]), A(S.g[1]), A(S.g[2]), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
+        Gg, Ph, step_vals(S.tau, S.g), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
         Ph.eos == TFSPH_EOS_ADIABATIC, static_cast<V4<T> *>(G.pos[G.cur]), static_cast<V4<T> *>(G.vel[G.cur]),
         G.id[G.cur], G.key, G.start, static_cast<const V4<T> *>(acc), static_cast<V4<T> *>(D.pos[D.cur]),
         static_cast<V4<T> *>(D.vel[D.cur]), D.key, D.start);
@@ -340,7 +427,7 @@ cudaError_t launch_cell_adjoint(const LaunchCtx &L, const void *geo, const void 
     if (L.precision == TFSPH_FP64)
         return cell_adjoint_dim<double, double>(L, geo, phys, G, D, acc, S, lgx, lgv, ldx, ldu, lA, lts);
     if (S.cell_acc == TFSPH_CELL_ACC_FP64)
-        return cell_adjoint_dim<float, double>(L, geo, phys, G, D, acc, S, lgx, lgv, ldx, ldu, lA, lts);
+        return cell_adjoint_dim<float, df>(L, geo, phys, G, D, acc, S, lgx, lgv, ldx, ldu, lA, lts);
     return cell_adjoint_dim<float, float>(L, geo, phys, G, D, acc, S, lgx, lgv, ldx, ldu, lA, lts);
 }
 
@@ -348,7 +435,7 @@ cudaError_t launch_cell_update(const LaunchCtx &L, const void *geo, const void *
                                PhaseBufs &D, const void *acc, const StepArgs &S)
 {
     if (L.precision == TFSPH_FP64) return cell_update_dim<double, double>(L, geo, phys, G, D, acc, S);
-    if (S.cell_acc == TFSPH_CELL_ACC_FP64) return cell_update_dim<float, double>(L, geo, phys, G, D, acc, S);
+    if (S.cell_acc == TFSPH_CELL_ACC_FP64) return cell_update_dim<float, df>(L, geo, phys, G, D, acc, S);
     return cell_update_dim<float, float>(L, geo, phys, G, D, acc, S);
 }
 

@@ -3,12 +3,40 @@
 // implicit solve, and the per-particle update of each phase.
 #pragma once
 
+#include <type_traits>
+
+#include "dfloat.cuh"
 #include "tfsph_internal.cuh"
 
 namespace tfsph {
 
+// tau and g of a step for every accumulator type: float takes the leading
+// parts, df the pairs, double the binary64 values. Filled on the host, so no
+// kernel converts them.
+struct StepVals {
+    df tau, g[3];
+    double dtau, dg[3];
+};
+inline StepVals step_vals(double tau, const double g[3])
+{
+    StepVals v;
+    v.tau = df(tau);
+    v.dtau = tau;
+    for (int k = 0; k < 3; ++k) {
+        v.g[k] = df(g[k]);
+        v.dg[k] = g[k];
+    }
+    return v;
+}
+template <class A> __device__ __forceinline__ A step_val(df pair, double wide)
+{
+    if constexpr (std::is_same<A, df>::value) return pair;
+    else if constexpr (sizeof(A) == 4) return pair.h;
+    else return A(wide);
+}
+
 // One cell: N, L, sum v, sum u, sum A, sum t_j (or sum 1/t_j) in storage
-// order, with accumulator type A, then
+// order, with accumulator type A (float, df or double), then
 //   eps* = m_d L / (m_g N)                                (Eq. 17)
 //   t*   = sum t_j / L   (or L / sum 1/t_j)               (Eq. 18)
 //   w    = v_* - u_*                                      (Eq. 21)
@@ -16,30 +44,42 @@ namespace tfsph {
 //   u_*' = u_* + tau g + (tau/t*) w',  v_*' = u_*' + w'
 // which is the cell average of the implicit Eqs. 19-20. Returns 1 when the
 // cell holds moving gas and dust (drag applies) and then sets un = u_*',
-// vn = v_*', ig = 1/(1 + tau eps*/t*) and id = 1/(1 + tau/t*).
+// vn = v_*', ig = 1/(1 + tau eps*/t*) and id = 1/(1 + tau/t*). With A = df it
+// returns 2 where the binary32 exponent range may not hold the solve: tau/t*
+// outside [2^-60, 2^24], eps* outside [2^-40, 2^40], or a velocity so small
+// (nonzero, below 2^-80) or so large that low parts are lost.
 template <class T, class A, int DIM>
-__device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, A tau, const A gv[3], int harmonic, int has_frozen,
+__device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
                                                const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
                                                const V4<T> *__restrict__ acc, uint32_t gs, uint32_t ge,
                                                const V4<T> *__restrict__ dvel, uint32_t ds, uint32_t de, T un_out[3],
                                                T vn_out[3], T &ig_out, T &id_out)
 {
-    A N = A(0), L = A(0), st = A(0);
-    A sv[3] = {A(0), A(0), A(0)}, sa[3] = {A(0), A(0), A(0)}, su[3] = {A(0), A(0), A(0)};
+    constexpr bool kPair = std::is_same<A, df>::value;
+    const A one = A(1.0f), zero = A(0.0f);
+    uint32_t ng = 0, nd = 0;
+    A st = zero;
+    A sv[3] = {zero, zero, zero}, sa[3] = {zero, zero, zero}, su[3] = {zero, zero, zero};
+    // a particle's component into a sum (df: value + float)
+    auto add = [](A &s, T x) {
+        if constexpr (kPair) s += (float)x;
+        else s += A(x);
+    };
     auto add_gas = [&](uint32_t idv, const V4<T> &v, const V4<T> &ac) {
         if (has_frozen && (idv & kFrozenBit)) return;
-        N += A(1);
-        sv[0] += A(v.x);
-        sa[0] += A(ac.x);
-        if (DIM > 1) { sv[1] += A(v.y); sa[1] += A(ac.y); }
-        if (DIM > 2) { sv[2] += A(v.z); sa[2] += A(ac.z); }
+        ++ng;
+        add(sv[0], v.x);
+        add(sa[0], ac.x);
+        if (DIM > 1) { add(sv[1], v.y); add(sa[1], ac.y); }
+        if (DIM > 2) { add(sv[2], v.z); add(sa[2], ac.z); }
     };
     auto add_dust = [&](const V4<T> &u) {
-        L += A(1);
-        su[0] += A(u.x);
-        if (DIM > 1) su[1] += A(u.y);
-        if (DIM > 2) su[2] += A(u.z);
-        st += harmonic ? A(1) / A(u.w) : A(u.w);
+        ++nd;
+        add(su[0], u.x);
+        if (DIM > 1) add(su[1], u.y);
+        if (DIM > 2) add(su[2], u.z);
+        if (harmonic) st += one / A(u.w);
+        else add(st, u.w);
     };
     // the first gas and dust particles are loaded together (the usual cell
     // holds one or a few of each), the rest in storage order
@@ -55,31 +95,86 @@ __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, A tau, const A
     for (uint32_t a = gs + 1; a < ge; ++a) add_gas(has_frozen ? gid[a] : 0u, gvel[a], acc[a]);
     if (ds < de) add_dust(u0);
     for (uint32_t j = ds + 1; j < de; ++j) add_dust(dvel[j]);
-    if (!(N > A(0) && L > A(0))) return 0;
+    if (ng == 0 || nd == 0) return 0;
+    const A tau = step_val<A>(S.tau, S.dtau);
+    const A N = A(ng), L = A(nd);
     const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
     // 1/N and 1/L from one division (N L is an exact product of counts)
-    const A invNL = A(1) / (N * L);
+    const A invNL = one / (N * L);
     const A invN = L * invNL, invL = N * invNL;
     // rt = tau / t*, with t* = st / L (mean) or L / st (harmonic mean)
     const A rt = harmonic ? tau * st * invL : tau * L / st;
-    const A den = A(1) + rt * (A(1) + eps);
-    const A invden = A(1) / den;  // one division for the DIM components
+    const A den = one + rt * (one + eps);
+    const A invden = one / den;  // one division for the DIM components
+    bool fits = true;
+    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
         const A vs = sv[k] * invN;
         const A us = su[k] * invL;
         const A ab = sa[k] * invN;
         const A wn = ((vs - us) + tau * ab) * invden;
-        const A un = us + tau * gv[k] + rt * wn;
+        const A un = us + tau * step_val<A>(S.g[k], S.dg[k]) + rt * wn;
+        const A vn = un + wn;
         un_out[k] = T(un);
-        vn_out[k] = T(un + wn);
+        vn_out[k] = T(vn);
+        if constexpr (kPair)
+            fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p100f, 0x1p100f) &&
+                   df_in(vn, -0x1p100f, 0x1p100f);
     }
     // 1/(1 + rt eps) and 1/(1 + rt) from one division
-    const A dg = A(1) + rt * eps, dd = A(1) + rt;
-    const A invgd = A(1) / (dg * dd);
+    const A dg = one + rt * eps, dd = one + rt;
+    const A invgd = one / (dg * dd);
     ig_out = T(dd * invgd);
     id_out = T(dg * invgd);
-    return 1;
+    return fits ? 1 : 2;
+}
+
+// The binary64 solve of a cell outside df's range (see above): rare, so out of
+// line and off the register allocation of the common path.
+template <class T, int DIM>
+__device__ __noinline__ int cell_drag_wide(const Phys<T> Ph, const StepVals S, int harmonic, int has_frozen,
+                                           const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                           const V4<T> *__restrict__ acc, uint32_t gs, uint32_t ge,
+                                           const V4<T> *__restrict__ dvel, uint32_t ds, uint32_t de, T *out)
+{
+    T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
+    const int r = cell_drag_solve<T, double, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de,
+                                                  un, vn, ig, id);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) {
+        out[k] = un[k];
+        out[3 + k] = vn[k];
+    }
+    out[6] = ig;
+    out[7] = id;
+    return r;
+}
+
+// cell_drag_solve with df's rare cells taken in binary64.
+template <class T, class A, int DIM>
+__device__ __forceinline__ int cell_drag(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
+                                         const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                         const V4<T> *__restrict__ acc, uint32_t gs, uint32_t ge,
+                                         const V4<T> *__restrict__ dvel, uint32_t ds, uint32_t de, T un[3], T vn[3],
+                                         T &ig, T &id)
+{
+    int r = cell_drag_solve<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, un, vn, ig,
+                                       id);
+    if constexpr (std::is_same<A, df>::value) {
+        if (r == 2) {
+            T o[8];
+            r = cell_drag_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, o);
+#pragma unroll
+            for (int k = 0; k < DIM; ++k) {
+                un[k] = o[k];
+                vn[k] = o[3 + k];
+            }
+            ig = o[6];
+            id = o[7];
+        }
+    }
+    return r;
 }
 
 // Gas particle (Eq. 19 solved for v'): v' = u_*' + (v + tau (A + g) - u_*') ig
