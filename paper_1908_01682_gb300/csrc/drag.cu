@@ -1,8 +1,9 @@
 // Implicit drag in cell (Sec. 2.3, Eqs. 17-21) fused with the particle
 // update and the next step's cell keys.
 //
-// One CTA owns kCellsPerCta consecutive cells and, because particles are
-// stored in cell order, the contiguous gas and dust ranges of those cells.
+// One CTA owns kCellsPerCta (or fewer) consecutive cells and, because
+// particles are stored in cell order, the contiguous gas and dust ranges of
+// those cells.
 //   Phase 1 (thread per cell, accumulator type A: float, double, or df, the
 //   two-float form of double that the FP32 state takes): N, L, sum v, sum u,
 //     sum A, sum t_j (or sum 1/t_j) in storage order, then
@@ -21,14 +22,17 @@
 //     next cell key.
 // The per-cell results live in shared memory only; nothing per cell is
 // written to global memory.
+#include <algorithm>
+
 #include "drag_ops.cuh"
 
 namespace tfsph {
 namespace {
 
-// (FP32 state, 101^3 cells: 66 us with df against 202 us in binary64, whose
-// pipe was 84 % busy.)
-template <class T, class A, int DIM, bool EST>
+// LANES: 1, a thread per cell in phase 1, or 4, four lanes per cell (cells of
+// several particles, whose serial sums otherwise wait on one load at a time).
+// The CTA owns blockDim.x / LANES cells.
+template <class T, class A, int DIM, bool EST, int LANES>
 __global__ void __launch_bounds__(kCellsPerCta, (sizeof(T) == 4 && sizeof(A) == 4) ? 12 : (sizeof(T) == 4 ? 8 : 1))
 k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, int adiabatic,
               V4<T> *__restrict__ gpos, V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
@@ -43,30 +47,61 @@ k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, in
     __shared__ int s_drag[kCellsPerCta];
 
     const uint32_t ncells = G.ncells;
-    const uint32_t c0 = blockIdx.x * kCellsPerCta;
-    const uint32_t c = c0 + threadIdx.x;
+    const uint32_t cpc = blockDim.x / LANES;
+    const uint32_t c0 = blockIdx.x * cpc;
+    const uint32_t lc0 = threadIdx.x / LANES;
+    const uint32_t c = c0 + lc0;
 
     // ---- phase 1: per-cell sums and the implicit solve ----
     int drag = 0;
     if (c < ncells) {
+        const uint32_t gs = gstart[c], ge = gstart[c + 1], ds = dstart[c], de = dstart[c + 1];
         T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
-        drag = cell_drag<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gstart[c], gstart[c + 1], dvel,
-                                    dstart[c], dstart[c + 1], un, vn, ig, id);
-        if (drag) {
+        if constexpr (LANES == 1) {
+            drag = cell_drag<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, un, vn, ig,
+                                        id);
+            if (drag) {
 #pragma unroll
-            for (int k = 0; k < DIM; ++k) {
-                s_us[k][threadIdx.x] = un[k];
-                s_vs[k][threadIdx.x] = vn[k];
+                for (int k = 0; k < DIM; ++k) {
+                    s_us[k][lc0] = un[k];
+                    s_vs[k][lc0] = vn[k];
+                }
+                s_ig[lc0] = ig;
+                s_id[lc0] = id;
             }
-            s_ig[threadIdx.x] = ig;
-            s_id[threadIdx.x] = id;
+        } else {
+            const int k = threadIdx.x & 3;
+            const unsigned mask = 0xfu << (threadIdx.x & 28);
+            drag = cell_drag_lanes<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, mask,
+                                              un[0], vn[0], ig, id);
+            if (drag == 1) {
+                if (k < DIM) {
+                    s_us[k][lc0] = un[0];
+                    s_vs[k][lc0] = vn[0];
+                }
+                if (k == 0) {
+                    s_ig[lc0] = ig;
+                    s_id[lc0] = id;
+                }
+            } else if (drag == 2) {
+                if (k == 0) {
+                    T o[8];
+                    cell_drag_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, o);
+                    for (int m = 0; m < DIM; ++m) {
+                        s_us[m][lc0] = o[m];
+                        s_vs[m][lc0] = o[3 + m];
+                    }
+                    s_ig[lc0] = o[6];
+                    s_id[lc0] = o[7];
+                }
+            }
         }
     }
-    s_drag[threadIdx.x] = drag;
+    if (LANES == 1 || (threadIdx.x & 3) == 0) s_drag[lc0] = drag;
     __syncthreads();
 
     // ---- phase 2: particle updates over the CTA's storage ranges ----
-    const uint32_t c1 = min(c0 + (uint32_t)kCellsPerCta, ncells);
+    const uint32_t c1 = min(c0 + cpc, ncells);
     const T tau_t = step_val<T>(S.tau, S.dtau);
     const T gt[3] = {step_val<T>(S.g[0], S.dg[0]), step_val<T>(S.g[1], S.dg[1]), step_val<T>(S.g[2], S.dg[2])};
     {
@@ -80,7 +115,7 @@ k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, in
             V4<T> v = gvel[a];
             const V4<T> ac = acc[a];
             const uint32_t lc = cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
-            const bool dr = lc < (uint32_t)kCellsPerCta && s_drag[lc];
+            const bool dr = lc < cpc && s_drag[lc];
             T us[3] = {T(0), T(0), T(0)}, ig = T(0);
             if (dr) {
                 ig = s_ig[lc];
@@ -99,7 +134,7 @@ k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, in
             V4<T> p = dpos[j];
             V4<T> u = dvel[j];
             const uint32_t lc = cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
-            const bool dr = lc < (uint32_t)kCellsPerCta && s_drag[lc];
+            const bool dr = lc < cpc && s_drag[lc];
             T vs[3] = {T(0), T(0), T(0)}, id = T(0);
             if (dr) {
                 id = s_id[lc];
@@ -395,11 +430,22 @@ cudaError_t cell_update_t(const LaunchCtx &L, const void *geo, const void *phys,
 {
     const Geo<T> &Gg = *static_cast<const Geo<T> *>(geo);
     const Phys<T> &Ph = *static_cast<const Phys<T> *>(phys);
-    const uint32_t blocks = (Gg.ncells + kCellsPerCta - 1) / kCellsPerCta;
     bool est = true;
     for (int d = 0; d < DIM; ++d) est = est && Gg.est_exact[d];
-    auto kern = est ? k_cell_update<T, A, DIM, true> : k_cell_update<T, A, DIM, false>;
-    kern<<<blocks, kCellsPerCta, 0, L.stream>>>(
+    // Four lanes per cell where cells hold several particles of a phase; with
+    // binary64 sums only while the chip is not full of warps anyway (the lanes
+    // repeat the scalar part of the solve on the 2-lane pipe).
+    // Fewer cells per CTA, down to one warp, until every SM has two CTAs.
+    const double mean = (double)std::max(G.n, D.n) / (double)Gg.ncells;
+    const bool lanes = mean >= 1.5 && (sizeof(A) == 4 || std::is_same<A, df>::value || Gg.ncells < 4096u);
+    const int per = lanes ? 4 : 1;
+    int threads = kCellsPerCta;
+    while (threads > 32 && (int64_t)Gg.ncells * per < (int64_t)threads * 2 * kSmCount) threads /= 2;
+    const uint32_t cpc = (uint32_t)(threads / per);
+    const uint32_t blocks = (Gg.ncells + cpc - 1) / cpc;
+    auto kern = lanes ? (est ? k_cell_update<T, A, DIM, true, 4> : k_cell_update<T, A, DIM, false, 4>)
+                      : (est ? k_cell_update<T, A, DIM, true, 1> : k_cell_update<T, A, DIM, false, 1>);
+    kern<<<blocks, threads, 0, L.stream>>>(
         Gg, Ph, step_vals(S.tau, S.g), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
         Ph.eos == TFSPH_EOS_ADIABATIC, static_cast<V4<T> *>(G.pos[G.cur]), static_cast<V4<T> *>(G.vel[G.cur]),
         G.id[G.cur], G.key, G.start, static_cast<const V4<T> *>(acc), static_cast<V4<T> *>(D.pos[D.cur]),

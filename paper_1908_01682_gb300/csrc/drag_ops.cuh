@@ -91,9 +91,13 @@ __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals
         if (has_frozen) id0 = gid[gs];
     }
     if (ds < de) u0 = dvel[ds];
+    // not unrolled: with a particle or two per cell the unrolled bodies only
+    // cost registers and branches (128^3 box: 67 us against 82 unrolled)
     if (gs < ge) add_gas(id0, v0, a0);
+#pragma unroll 1
     for (uint32_t a = gs + 1; a < ge; ++a) add_gas(has_frozen ? gid[a] : 0u, gvel[a], acc[a]);
     if (ds < de) add_dust(u0);
+#pragma unroll 1
     for (uint32_t j = ds + 1; j < de; ++j) add_dust(dvel[j]);
     if (ng == 0 || nd == 0) return 0;
     const A tau = step_val<A>(S.tau, S.dtau);
@@ -175,6 +179,105 @@ __device__ __forceinline__ int cell_drag(const Phys<T> &Ph, const StepVals &S, i
         }
     }
     return r;
+}
+
+// A value of lane src of the warp (df, float or double).
+template <class A> __device__ __forceinline__ A lane_value(unsigned mask, A v, int src)
+{
+    if constexpr (std::is_same<A, df>::value)
+        return df(__shfl_sync(mask, v.h, src), __shfl_sync(mask, v.l, src));
+    else return __shfl_sync(mask, v, src);
+}
+
+// The same solve by four consecutive lanes of a warp, lane k of them on
+// component k (lane 3 on the stopping times), for cells holding several
+// particles: four times the threads of the form above, loads of a component
+// by consecutive lanes, four particles in flight per lane, and the terms of
+// every sum still added in storage order by one lane, so both forms round
+// alike. Lane k returns un[k], vn[k] in un, vn; ig and id come back in every
+// lane. mask: the four lanes, which call it together.
+template <class T, class A, int DIM>
+__device__ __forceinline__ int cell_drag_lanes(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
+                                               const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                               const V4<T> *__restrict__ acc, uint32_t gs, uint32_t ge,
+                                               const V4<T> *__restrict__ dvel, uint32_t ds, uint32_t de,
+                                               unsigned mask, T &un_out, T &vn_out, T &ig_out, T &id_out)
+{
+    constexpr bool kPair = std::is_same<A, df>::value;
+    const int k = threadIdx.x & 3;
+    const A one = A(1.0f), zero = A(0.0f);
+    auto add = [](A &s, T x) {
+        if constexpr (kPair) s += (float)x;
+        else s += A(x);
+    };
+    const T *gv = reinterpret_cast<const T *>(gvel) + k, *ga = reinterpret_cast<const T *>(acc) + k;
+    const T *dv = reinterpret_cast<const T *>(dvel) + k;
+    const bool axis = k < DIM, last = k == 3;
+    uint32_t ng = 0, nd = de - ds;
+    A sv = zero, sa = zero, su = zero;  // lane 3: su is the sum over the stopping times
+    constexpr int kAhead = 4;
+    for (uint32_t a = gs; a < ge; a += kAhead) {
+        T v[kAhead], ac[kAhead];
+        uint32_t fz[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const bool in = a + u < ge;
+            v[u] = in && axis ? gv[4 * (size_t)(a + u)] : T(0);
+            ac[u] = in && axis ? ga[4 * (size_t)(a + u)] : T(0);
+            fz[u] = in ? (has_frozen ? gid[a + u] & kFrozenBit : 0u) : 1u;
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            if (!fz[u]) {
+                ++ng;
+                add(sv, v[u]);
+                add(sa, ac[u]);
+            }
+    }
+    for (uint32_t j = ds; j < de; j += kAhead) {
+        T w[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) w[u] = j + u < de && (axis || last) ? dv[4 * (size_t)(j + u)] : T(1);
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u)
+            if (j + u < de) {
+                if (harmonic && last) su += one / A(w[u]);
+                else add(su, w[u]);
+            }
+    }
+    if (ng == 0 || nd == 0) return 0;
+    const A st = lane_value(mask, su, (threadIdx.x & 31) | 3);
+    const A tau = step_val<A>(S.tau, S.dtau);
+    const A N = A(ng), L = A(nd);
+    const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
+    const A invNL = one / (N * L);
+    const A invN = L * invNL, invL = N * invNL;
+    const A rt = harmonic ? tau * st * invL : tau * L / st;
+    const A den = one + rt * (one + eps);
+    const A invden = one / den;
+    const A dg = one + rt * eps, dd = one + rt;
+    const A invgd = one / (dg * dd);
+    ig_out = T(dd * invgd);
+    id_out = T(dg * invgd);
+    bool fits = true;
+    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    if (axis) {
+        const A g = k == 0 ? step_val<A>(S.g[0], S.dg[0])
+                           : (k == 1 ? step_val<A>(S.g[1], S.dg[1]) : step_val<A>(S.g[2], S.dg[2]));
+        const A us = su * invL;
+        const A wn = ((sv * invN - us) + tau * (sa * invN)) * invden;
+        const A un = us + tau * g + rt * wn;
+        const A vn = un + wn;
+        un_out = T(un);
+        vn_out = T(vn);
+        if constexpr (kPair)
+            fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p100f, 0x1p100f) &&
+                   df_in(vn, -0x1p100f, 0x1p100f);
+    }
+    if constexpr (kPair) {
+        if (!__all_sync(mask, fits)) return 2;
+    }
+    return 1;
 }
 
 // Gas particle (Eq. 19 solved for v'): v' = u_*' + (v + tau (A + g) - u_*') ig

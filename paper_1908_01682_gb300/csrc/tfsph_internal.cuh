@@ -139,8 +139,11 @@ constexpr int kScanThreads = 256;
 constexpr int kScanItems = 8;  // the scan kernels move them as two 16-byte words
 constexpr int kScanTile = kScanThreads * kScanItems;
 
-// Cell-update CTA: one thread per cell in phase 1.
+// Cell-update CTA: most cells (one thread per cell in phase 1).
 constexpr int kCellsPerCta = 128;
+
+// SMs of the chip the kernels are written for; grids are cut to fill them.
+constexpr int kSmCount = 152;
 
 // ---------------------------------------------------------------------------
 // Launchers (host functions), grouped by translation unit.
@@ -359,11 +362,12 @@ template <class T> __device__ __forceinline__ T min_image(T d, int per, T L, T h
     return d;
 }
 
-// Periodic image of x in [lo, lo + L).
+// Periodic image of x in [lo, lo + L). The division is skipped where its
+// floor is known to be 0 (0 <= y < L: y / L rounds to less than 1).
 template <class T> __device__ __forceinline__ T wrap_periodic(T x, T lo, T L)
 {
     T y = x - lo;
-    y -= L * floor(y / L);
+    if (!(y >= T(0) && y < L)) y -= L * floor(y / L);
     T r = lo + y;
     if (r >= lo + L) r = lo;
     if (r < lo) r = lo;
