@@ -50,7 +50,7 @@ extern "C" {
 #define TFSPH_E_CUDA          4  /* a CUDA runtime call failed */
 #define TFSPH_E_OOM           5  /* device or host allocation failed */
 #define TFSPH_E_INTERNAL      6  /* a device-side consistency check failed */
-#define TFSPH_E_TIMEOUT       7  /* a bounded device-side wait ran out (batched persistent step) */
+#define TFSPH_E_TIMEOUT       7  /* a bounded device-side wait ran out (a one-launch step) */
 
 #define TFSPH_MEM_HOST   0
 #define TFSPH_MEM_DEVICE 1

@@ -30,6 +30,7 @@
 #include <vector>
 
 #include "drag_ops.cuh"
+#include "grid_barrier.cuh"
 #include "pair.cuh"
 #include "sort_ops.cuh"
 
@@ -39,11 +40,6 @@ namespace {
 
 constexpr int kItems = 8;              // scan items per thread
 constexpr int kMaxBlock = 512;
-
-struct GridBar {
-    unsigned int count;
-    unsigned int gen;
-};
 
 // [begin, end): storage slots (particle chunks) or global cells (cell
 // chunks) of instance inst; end - begin <= the CTA size.
@@ -85,47 +81,11 @@ template <class T> struct BatchArgs {
 __device__ __forceinline__ uint32_t thread_rank() { return blockIdx.x * blockDim.x + threadIdx.x; }
 __device__ __forceinline__ uint32_t thread_count() { return gridDim.x * blockDim.x; }
 
-__device__ __forceinline__ unsigned int ld_acquire(const unsigned int *p)
-{
-    unsigned int v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 __device__ __forceinline__ int ld_parity(const int *p) { return *reinterpret_cast<const volatile int *>(p); }
 
-// Grid-wide barrier of a cooperative launch. The last CTA to arrive resets
-// the count and advances the generation; the others wait for the generation
-// to change, at most spin_limit clock cycles. Returns false (after flagging
-// kErrTimeout) when the wait ran out; the caller then returns at once.
-template <class T> __device__ bool grid_barrier(const BatchArgs<T> &B)
+template <class T> __device__ __forceinline__ bool grid_barrier(const BatchArgs<T> &B)
 {
-    __shared__ int s_ok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        const unsigned int g = ld_acquire(&B.bar->gen);
-        __threadfence();
-        if (atomicAdd(&B.bar->count, 1u) == gridDim.x - 1) {
-            atomicExch(&B.bar->count, 0u);
-            __threadfence();
-            atomicAdd(&B.bar->gen, 1u);
-        } else {
-            const long long t0 = clock64();
-            while (ld_acquire(&B.bar->gen) == g) {
-                if (clock64() - t0 > B.spin_limit) {
-                    atomicOr(B.err, kErrTimeout);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
-            }
-        }
-        __threadfence();
-        s_ok = ok;
-    }
-    __syncthreads();
-    return s_ok != 0;
+    return tfsph::grid_barrier(B.bar, B.spin_limit, B.err, 64u);
 }
 
 // Copies an instance record into shared memory (the whole CTA takes part).
@@ -415,7 +375,7 @@ __device__ void ph_pair_tiled(const BatchArgs<T> &B, int q, BInst<T> &si, unsign
                 T t;
                 const int ca = axis_cell(pa.x, G.lo[0], G.inv_w[0], n, t);
                 int olo, ohi;
-                x_window(G, t - T(ca), G.lim2, olo, ohi);
+                x_window<T, 1>(G, t - T(ca), G.lim2, olo, ohi);
                 const int hl = max(ca + olo - w0, 0), hh = min(ca + ohi - w0, nwc - 1) + 1;  // window cells [hl, hh)
                 // cells h < s0 lie across the low seam, h >= s1 across the high one
                 const int s0 = per ? min(max(-w0, 0), nwc) : 0;
@@ -425,7 +385,7 @@ __device__ void ph_pair_tiled(const BatchArgs<T> &B, int q, BInst<T> &si, unsign
                         const V4<T> pb = sp[j];
                         T d[3];
                         const T r2 = pair_r2<T, 1, decltype(seam)::value>(G, pa, pb, d);
-                        A.add(G, si.Ph, pb, nullptr, T(1), 0u, r2, d);
+                        A.template add<1>(G, si.Ph, pb, nullptr, T(1), 0u, r2, d);
                     }
                 };
                 // the global walk's order: wrapped from below, wrapped from above, then the rest,

@@ -417,7 +417,8 @@ cudaError_t keys_t(const LaunchCtx &L, const void *geo, const PhaseBufs &P)
 }
 
 template <class T>
-cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D, uint32_t *bsum, int64_t nblk)
+cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D, uint32_t *bsum, int64_t nblk,
+                  bool counted)
 {
     const Geo<T> &Gm = *static_cast<const Geo<T> *>(geo);
     const int ng = (int)G.n, nd = (int)D.n;
@@ -425,7 +426,7 @@ cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &
     const uint32_t ncells = Gm.ncells;
     // combined atomics pay when a phase has on average more than one particle per cell
     const bool agg = (double)std::max(ng, nd) >= 1.5 * (double)ncells;
-    if (ntot > 0) {
+    if (ntot > 0 && !counted) {
         if (agg) k_count<true><<<grid_for(ntot, 256), 256, 0, L.stream>>>(G.key, ng, G.count, D.key, nd, D.count);
         else k_count<false><<<grid_for(ntot, 256), 256, 0, L.stream>>>(G.key, ng, G.count, D.key, nd, D.count);
     }
@@ -519,10 +520,10 @@ cudaError_t launch_keys(const LaunchCtx &L, const void *geo, const PhaseBufs &P)
 }
 
 cudaError_t launch_bin(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D, uint32_t *bsum,
-                       int64_t nblk)
+                       int64_t nblk, bool counted)
 {
-    return L.precision == TFSPH_FP64 ? bin_t<double>(L, geo, G, D, bsum, nblk)
-                                     : bin_t<float>(L, geo, G, D, bsum, nblk);
+    return L.precision == TFSPH_FP64 ? bin_t<double>(L, geo, G, D, bsum, nblk, counted)
+                                     : bin_t<float>(L, geo, G, D, bsum, nblk, counted);
 }
 
 cudaError_t launch_pack(const LaunchCtx &L, PhaseBufs &P, const void *const *src, int ncomp_v,

@@ -40,113 +40,10 @@ k_cell_update(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen, in
               V4<T> *__restrict__ dpos, V4<T> *__restrict__ dvel, uint32_t *__restrict__ dkey,
               const uint32_t *__restrict__ dstart)
 {
-    __shared__ T s_us[3][kCellsPerCta];
-    __shared__ T s_vs[3][kCellsPerCta];
-    __shared__ T s_ig[kCellsPerCta];
-    __shared__ T s_id[kCellsPerCta];
-    __shared__ int s_drag[kCellsPerCta];
-
-    const uint32_t ncells = G.ncells;
+    __shared__ CellShared<T> s;
     const uint32_t cpc = blockDim.x / LANES;
-    const uint32_t c0 = blockIdx.x * cpc;
-    const uint32_t lc0 = threadIdx.x / LANES;
-    const uint32_t c = c0 + lc0;
-
-    // ---- phase 1: per-cell sums and the implicit solve ----
-    int drag = 0;
-    if (c < ncells) {
-        const uint32_t gs = gstart[c], ge = gstart[c + 1], ds = dstart[c], de = dstart[c + 1];
-        T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
-        if constexpr (LANES == 1) {
-            drag = cell_drag<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, un, vn, ig,
-                                        id);
-            if (drag) {
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) {
-                    s_us[k][lc0] = un[k];
-                    s_vs[k][lc0] = vn[k];
-                }
-                s_ig[lc0] = ig;
-                s_id[lc0] = id;
-            }
-        } else {
-            const int k = threadIdx.x & 3;
-            const unsigned mask = 0xfu << (threadIdx.x & 28);
-            drag = cell_drag_lanes<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, mask,
-                                              un[0], vn[0], ig, id);
-            if (drag == 1) {
-                if (k < DIM) {
-                    s_us[k][lc0] = un[0];
-                    s_vs[k][lc0] = vn[0];
-                }
-                if (k == 0) {
-                    s_ig[lc0] = ig;
-                    s_id[lc0] = id;
-                }
-            } else if (drag == 2) {
-                if (k == 0) {
-                    T o[8];
-                    cell_drag_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, o);
-                    for (int m = 0; m < DIM; ++m) {
-                        s_us[m][lc0] = o[m];
-                        s_vs[m][lc0] = o[3 + m];
-                    }
-                    s_ig[lc0] = o[6];
-                    s_id[lc0] = o[7];
-                }
-            }
-        }
-    }
-    if (LANES == 1 || (threadIdx.x & 3) == 0) s_drag[lc0] = drag;
-    __syncthreads();
-
-    // ---- phase 2: particle updates over the CTA's storage ranges ----
-    const uint32_t c1 = min(c0 + cpc, ncells);
-    const T tau_t = step_val<T>(S.tau, S.dtau);
-    const T gt[3] = {step_val<T>(S.g[0], S.dg[0]), step_val<T>(S.g[1], S.dg[1]), step_val<T>(S.g[2], S.dg[2])};
-    {
-        const uint32_t a0 = gstart[c0], a1 = gstart[c1];
-        for (uint32_t a = a0 + threadIdx.x; a < a1; a += blockDim.x) {
-            V4<T> p = gpos[a];
-            if (has_frozen && (gid[a] & kFrozenBit)) {
-                gkey[a] = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
-                continue;
-            }
-            V4<T> v = gvel[a];
-            const V4<T> ac = acc[a];
-            const uint32_t lc = cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
-            const bool dr = lc < cpc && s_drag[lc];
-            T us[3] = {T(0), T(0), T(0)}, ig = T(0);
-            if (dr) {
-                ig = s_ig[lc];
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) us[k] = s_us[k][lc];
-            }
-            gas_particle_update<T, DIM>(G, tau_t, gt, adiabatic, p, v, ac, dr, us, ig);
-            gpos[a] = p;
-            gvel[a] = v;
-            gkey[a] = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
-        }
-    }
-    {
-        const uint32_t j0 = dstart[c0], j1 = dstart[c1];
-        for (uint32_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
-            V4<T> p = dpos[j];
-            V4<T> u = dvel[j];
-            const uint32_t lc = cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
-            const bool dr = lc < cpc && s_drag[lc];
-            T vs[3] = {T(0), T(0), T(0)}, id = T(0);
-            if (dr) {
-                id = s_id[lc];
-#pragma unroll
-                for (int k = 0; k < DIM; ++k) vs[k] = s_vs[k][lc];
-            }
-            dust_particle_update<T, DIM>(G, tau_t, gt, p, u, dr, vs, id);
-            dpos[j] = p;
-            dvel[j] = u;
-            dkey[j] = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
-        }
-    }
+    cell_update_cta<T, A, DIM, EST, LANES>(s, G, Ph, S, harmonic, has_frozen, adiabatic, blockIdx.x * cpc, cpc,
+                                           threadIdx.x, gpos, gvel, gid, gkey, gstart, acc, dpos, dvel, dkey, dstart);
 }
 
 // Reverse mode of the cell drag and the particle update (isothermal gas,

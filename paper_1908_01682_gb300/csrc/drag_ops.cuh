@@ -341,4 +341,150 @@ __device__ __forceinline__ void dust_particle_update(const Geo<T> &G, T tau_t, c
     }
 }
 
+// The cells [c0, c0 + cpc) and their particles, by one CTA (see drag.cu):
+// phase 1 with LANES threads per cell, then the particle updates and the next
+// cell keys; the dust loop starts at thread dust_tid. With COUNT and gcnt the
+// next keys are counted too (gcnt, dcnt: all zero before). The caller syncs before it
+// reuses the shared arrays.
+template <class T> struct CellShared {
+    T us[3][kCellsPerCta], vs[3][kCellsPerCta], ig[kCellsPerCta], id[kCellsPerCta];
+    int drag[kCellsPerCta];
+    // binary64: the cells' first slots, by which a particle finds its cell
+    // without the key's binary64 arithmetic
+    uint32_t first[sizeof(T) == 8 ? 2 : 1][sizeof(T) == 8 ? kCellsPerCta : 1];
+};
+// The last of n cells whose first slot is at or before i.
+__device__ __forceinline__ uint32_t slot_cell(const uint32_t *first, uint32_t n, uint32_t i)
+{
+    uint32_t lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi + 1) >> 1;
+        if (first[mid] <= i) lo = mid;
+        else hi = mid - 1;
+    }
+    return lo;
+}
+template <class T, class A, int DIM, bool EST, int LANES, bool COUNT = false>
+__device__ __forceinline__ void
+cell_update_cta(CellShared<T> &s, const Geo<T> &G, const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
+                int adiabatic, uint32_t c0, uint32_t cpc, uint32_t dust_tid, V4<T> *__restrict__ gpos,
+                V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid, uint32_t *__restrict__ gkey,
+                const uint32_t *__restrict__ gstart, const V4<T> *__restrict__ acc, V4<T> *__restrict__ dpos,
+                V4<T> *__restrict__ dvel, uint32_t *__restrict__ dkey, const uint32_t *__restrict__ dstart,
+                uint32_t *__restrict__ gcnt = nullptr, uint32_t *__restrict__ dcnt = nullptr)
+{
+    constexpr bool kWide = sizeof(T) == 8;
+    const uint32_t ncells = G.ncells;
+    const uint32_t lc0 = threadIdx.x / LANES;
+    const uint32_t c = c0 + lc0;
+
+    // ---- phase 1: per-cell sums and the implicit solve ----
+    int drag = 0;
+    if (lc0 < cpc && c < ncells) {
+        const uint32_t gs = gstart[c], ge = gstart[c + 1], ds = dstart[c], de = dstart[c + 1];
+        if (kWide && (LANES == 1 || (threadIdx.x & 3) == 0)) {
+            s.first[0][lc0] = gs;
+            s.first[kWide ? 1 : 0][lc0] = ds;
+        }
+        T un[3] = {T(0), T(0), T(0)}, vn[3] = {T(0), T(0), T(0)}, ig = T(0), id = T(0);
+        if constexpr (LANES == 1) {
+            drag = cell_drag<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, un, vn, ig,
+                                        id);
+            if (drag) {
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) {
+                    s.us[k][lc0] = un[k];
+                    s.vs[k][lc0] = vn[k];
+                }
+                s.ig[lc0] = ig;
+                s.id[lc0] = id;
+            }
+        } else {
+            const int k = threadIdx.x & 3;
+            const unsigned mask = 0xfu << (threadIdx.x & 28);
+            drag = cell_drag_lanes<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, mask,
+                                              un[0], vn[0], ig, id);
+            if (drag == 1) {
+                if (k < DIM) {
+                    s.us[k][lc0] = un[0];
+                    s.vs[k][lc0] = vn[0];
+                }
+                if (k == 0) {
+                    s.ig[lc0] = ig;
+                    s.id[lc0] = id;
+                }
+            } else if (drag == 2) {
+                if (k == 0) {
+                    T o[8];
+                    cell_drag_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, gs, ge, dvel, ds, de, o);
+                    for (int m = 0; m < DIM; ++m) {
+                        s.us[m][lc0] = o[m];
+                        s.vs[m][lc0] = o[3 + m];
+                    }
+                    s.ig[lc0] = o[6];
+                    s.id[lc0] = o[7];
+                }
+            }
+        }
+    }
+    if (lc0 < cpc && (LANES == 1 || (threadIdx.x & 3) == 0)) s.drag[lc0] = drag;
+    __syncthreads();
+
+    // ---- phase 2: particle updates over the CTA's storage ranges ----
+    const uint32_t c1 = min(c0 + cpc, ncells);
+    const T tau_t = step_val<T>(S.tau, S.dtau);
+    const T gt[3] = {step_val<T>(S.g[0], S.dg[0]), step_val<T>(S.g[1], S.dg[1]), step_val<T>(S.g[2], S.dg[2])};
+    {
+        const uint32_t a0 = gstart[c0], a1 = gstart[c1];
+        for (uint32_t a = a0 + threadIdx.x; a < a1; a += blockDim.x) {
+            V4<T> p = gpos[a];
+            if (has_frozen && (gid[a] & kFrozenBit)) {
+                const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
+                gkey[a] = key;
+                if (COUNT && gcnt) atomicAdd(&gcnt[key], 1u);
+                continue;
+            }
+            V4<T> v = gvel[a];
+            const V4<T> ac = acc[a];
+            const uint32_t lc = kWide ? slot_cell(s.first[0], c1 - c0, a)
+                                      : cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
+            const bool dr = lc < cpc && s.drag[lc];
+            T us[3] = {T(0), T(0), T(0)}, ig = T(0);
+            if (dr) {
+                ig = s.ig[lc];
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) us[k] = s.us[k][lc];
+            }
+            gas_particle_update<T, DIM>(G, tau_t, gt, adiabatic, p, v, ac, dr, us, ig);
+            gpos[a] = p;
+            gvel[a] = v;
+            const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
+            gkey[a] = key;
+            if (COUNT && gcnt) atomicAdd(&gcnt[key], 1u);
+        }
+    }
+    {
+        const uint32_t j0 = dstart[c0], j1 = dstart[c1];
+        for (uint32_t j = j0 + dust_tid; j < j1; j += blockDim.x) {
+            V4<T> p = dpos[j];
+            V4<T> u = dvel[j];
+            const uint32_t lc = kWide ? slot_cell(s.first[kWide ? 1 : 0], c1 - c0, j)
+                                      : cell_key<T, DIM, EST>(G, p.x, p.y, p.z) - c0;
+            const bool dr = lc < cpc && s.drag[lc];
+            T vs[3] = {T(0), T(0), T(0)}, id = T(0);
+            if (dr) {
+                id = s.id[lc];
+#pragma unroll
+                for (int k = 0; k < DIM; ++k) vs[k] = s.vs[k][lc];
+            }
+            dust_particle_update<T, DIM>(G, tau_t, gt, p, u, dr, vs, id);
+            dpos[j] = p;
+            dvel[j] = u;
+            const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
+            dkey[j] = key;
+            if (COUNT && gcnt) atomicAdd(&dcnt[key], 1u);
+        }
+    }
+}
+
 }  // namespace tfsph

@@ -73,6 +73,20 @@ template <int MODE> struct ModeUses {
     static constexpr bool rho = MODE == 3 || MODE == 5;
 };
 
+// Distance of a pair from r^2 and its displacement. In 1D binary64 it is |d|,
+// which is what the rounded square root of the rounded square returns (away
+// from underflow), without the square root's chain on the binary64 pipe.
+template <class T, int DIM> __device__ __forceinline__ T pair_dist(T r2, const T d[3])
+{
+    if (DIM == 1 && sizeof(T) == 8) return fabs(d[0]);
+    return pair_sqrt(r2);
+}
+template <class T, int DIM> __device__ __forceinline__ T pair_inv_dist(T r2, const T d[3])
+{
+    if (DIM == 1 && sizeof(T) == 8) return T(1) / fabs(d[0]);
+    return pair_rsqrt(r2);
+}
+
 // ---------------------------------------------------------------------------
 // Per-pair work. MODE 0: density, 1: density + neighbour statistics,
 // 2: isothermal force without viscosity, 3: force with viscosity and/or
@@ -103,7 +117,7 @@ template <class T, int MODE> struct PairAcc {
     // candidate b: position (with p_b/rho_b^2 in .w), velocity, density, id,
     // squared distance r2 and displacement d = x_a - x_b (LISTED: b comes from
     // the neighbour list, whose entries passed the same r2 < 4h^2 test)
-    template <bool LISTED = false>
+    template <int DIM, bool LISTED = false>
     __device__ __forceinline__ void add(const Geo<T> &G, const Phys<T> &Ph, const V4<T> &pb, const V4<T> *vb,
                                         T rhob, uint32_t idb, T r2, const T d[3])
     {
@@ -132,7 +146,7 @@ template <class T, int MODE> struct PairAcc {
             return;
         }
         if (MODE <= 1) {
-            sum += kernel_w4(pair_sqrt(r2) * G.inv_h);
+            sum += kernel_w4(pair_dist<T, DIM>(r2, d) * G.inv_h);
             if (MODE == 1) {
                 ++cnt;
                 fp += (uint64_t)((idb & kIdMask) + 1u) * 0x9E3779B97F4A7C15ull;
@@ -142,7 +156,7 @@ template <class T, int MODE> struct PairAcc {
             // which acc_store applies once together with m_g
             // self or coincident particle (r^2 below the smallest normal):
             // 1/r taken as 0, so q = 0, g is finite and s d = 0 (no branch)
-            const T inv_r = r2 >= pair_r2_min<T>() ? pair_rsqrt(r2) : T(0);
+            const T inv_r = r2 >= pair_r2_min<T>() ? pair_inv_dist<T, DIM>(r2, d) : T(0);
             const T q = r2 * inv_r * G.inv_h;
             const T a = fmax(T(2) - q, T(0));
             const T g = q < T(1) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
@@ -152,7 +166,7 @@ template <class T, int MODE> struct PairAcc {
             az -= s * d[2];
         } else {
             if (!(r2 >= pair_r2_min<T>())) return;  // self or coincident particle: zero gradient
-            const T inv_r = pair_rsqrt(r2);
+            const T inv_r = pair_inv_dist<T, DIM>(r2, d);
             const T F = kernel_f(G, r2 * inv_r * G.inv_h, G.h * inv_r);  // (1/r) dW/dr
             T coef = qa + pb.w;
             if (MODE == 3) {
@@ -272,21 +286,55 @@ __device__ __forceinline__ int floor_int(double x) { return __double2int_rd(x); 
 // the squared radius rem of a particle at fractional position fx (the
 // closed form of the tile walk's x window; at most one cell wider than the
 // exact slab test at its ends).
-template <class T>
+template <class T, int DIM>
 __device__ __forceinline__ void x_window(const Geo<T> &G, T fx, T rem, int &olo, int &ohi)
 {
-    const T t = approx_sqrt(fmax(rem, T(0))) * G.inv_w[0];
+    // in 1D the radius is the whole reach: its square root is a constant
+    const T t = DIM == 1 ? G.reach0 : approx_sqrt(fmax(rem, T(0))) * G.inv_w[0];
     ohi = min(G.R[0], max(0, floor_int(fx + t)));
     olo = -min(G.R[0], max(0, floor_int(t - fx + T(1))));
+}
+
+// A neighbour's term apart from its addition, without a branch on membership
+// (zero for candidates outside, which leaves the sums as they are), for walks
+// that evaluate several candidates at once and add them in order. MODE 0: the
+// kernel value; MODE 2: the factor s of the displacement. With add_term the
+// same sums as add(), bit for bit.
+template <class T, int DIM, int MODE>
+__device__ __forceinline__ T pair_term(const PairAcc<T, MODE> &A, const Geo<T> &G, const Phys<T> &Ph, const V4<T> &pb,
+                                       T r2, const T d[3], bool in)
+{
+    static_assert(MODE == 0 || MODE == 2, "density and isothermal force");
+    if (MODE == 0) {
+        const T w = kernel_w4(pair_dist<T, DIM>(r2, d) * G.inv_h);
+        return in ? w : T(0);
+    }
+    const T inv_r = r2 >= pair_r2_min<T>() ? pair_inv_dist<T, DIM>(r2, d) : T(0);
+    const T q = r2 * inv_r * G.inv_h;
+    const T a = fmax(T(2) - q, T(0));
+    const T g = q < T(1) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
+    return in ? (A.qa + pb.w) * g : T(0);
+}
+template <class T, int DIM, int MODE>
+__device__ __forceinline__ void add_term(PairAcc<T, MODE> &A, T s, const T d[3])
+{
+    if (MODE == 0) {
+        A.sum += s;
+    } else {
+        A.ax -= s * d[0];
+        if (DIM > 1) A.ay -= s * d[1];
+        if (DIM > 2) A.az -= s * d[2];
+    }
 }
 
 // Calls f(b, n, seam) for every contiguous storage range [b, b + n) of cells
 // that may hold neighbours of a particle at (px, py, pz): per row of cells
 // (fixed y, z), the part of its x window wrapped below 0, the part wrapped
-// above n - 1, then the main part. seam is true when the range lies across a
+// above n - 1, then the main part (TILE_ORDER: the main part before the one
+// wrapped above, the order of the tiled walks). seam is true when the range lies across a
 // periodic seam from the particle, so its displacements need the periodic
 // image; within the particle's own image the plain difference is exact.
-template <class T, int DIM, class F>
+template <class T, int DIM, bool TILE_ORDER = false, class F>
 __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *__restrict__ start,
                                                T px, T py, T pz, F &&f)
 {
@@ -367,8 +415,9 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                 f(b, start[row + nx] - b, row_seam);
             } else {
                 int olo, ohi;
-                x_window(G, fx, G.lim2 - dz2 - dy2, olo, ohi);
+                x_window<T, DIM>(G, fx, G.lim2 - dz2 - dy2, olo, ohi);
                 int x0 = cx + olo, x1 = cx + ohi;
+                uint32_t hb = 0, hn = 0;  // the part wrapped above, kept for last in TILE_ORDER
                 if (G.per[0]) {
                     if (x0 < 0) {
                         const uint32_t b = start[row + x0 + nx];
@@ -376,8 +425,9 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                         x0 = 0;
                     }
                     if (x1 >= nx) {
-                        const uint32_t b = start[row];
-                        f(b, start[row + (x1 - nx) + 1] - b, true);
+                        hb = start[row];
+                        hn = start[row + (x1 - nx) + 1] - hb;
+                        if (!TILE_ORDER) f(hb, hn, true);
                         x1 = nx - 1;
                     }
                 } else {
@@ -386,6 +436,7 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                 }
                 const uint32_t b = start[row + x0];
                 f(b, start[row + x1 + 1] - b, row_seam);
+                if (TILE_ORDER && hn) f(hb, hn, true);
             }
         }
     }
@@ -408,7 +459,7 @@ __device__ __forceinline__ void walk_global(PairAcc<T, MODE> &A, const Geo<T> &G
                 if (ModeUses<MODE>::vel) vb = vel[b];
                 if (ModeUses<MODE>::rho) rhob = rho[b];
             }
-            A.add(G, Ph, pb, &vb, rhob, MODE == 1 ? id[b] : 0u, r2, d);
+            A.template add<DIM>(G, Ph, pb, &vb, rhob, MODE == 1 ? id[b] : 0u, r2, d);
         }
     };
     for_each_range<T, DIM>(G, start, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {

@@ -169,15 +169,15 @@ __device__ __forceinline__ void walk_smem_range(PairAcc<T, MODE> &A, const Geo<T
         const T r2 = pair_r2<T, DIM, SEAM>(G, pa, pb, d);
         if (REC) {
             if (r2 < G.h2x4) {
-                A.add(G, Ph, pb, nullptr, T(1), 0u, r2, d);
+                A.template add<DIM>(G, Ph, pb, nullptr, T(1), 0u, r2, d);
                 rec->push(j, SEAM);
             }
         } else if (ModeUses<MODE>::vel || ModeUses<MODE>::rho) {
             if (r2 < G.h2x4)
-                A.add(G, Ph, pb, ModeUses<MODE>::vel ? &svel[j] : nullptr, ModeUses<MODE>::rho ? srho[j] : T(1), 0u,
-                      r2, d);
+                A.template add<DIM>(G, Ph, pb, ModeUses<MODE>::vel ? &svel[j] : nullptr,
+                                    ModeUses<MODE>::rho ? srho[j] : T(1), 0u, r2, d);
         } else {
-            A.add(G, Ph, pb, nullptr, T(1), MODE == 1 ? sid[j] : 0u, r2, d);
+            A.template add<DIM>(G, Ph, pb, nullptr, T(1), MODE == 1 ? sid[j] : 0u, r2, d);
         }
     }
 }
@@ -326,7 +326,7 @@ __device__ __forceinline__ void read_list(PairAcc<T, MODE> &A, const Geo<T> &G, 
         T d[3];
         const T r2 = (!SEAMLESS && (cur & kNbSeam)) ? pair_r2<T, DIM, true>(G, pa, pb, d)
                                                     : pair_r2<T, DIM, false>(G, pa, pb, d);
-        A.template add<true>(G, Ph, pb, nullptr, T(1), 0u, r2, d);
+        A.template add<DIM, true>(G, Ph, pb, nullptr, T(1), 0u, r2, d);
     };
     auto quad = [&](unsigned long long w) {
         const uint32_t l = (uint32_t)w, h = (uint32_t)(w >> 32);

@@ -50,10 +50,13 @@ struct tfsph_ctx {
     alignas(64) unsigned char phys[sizeof(Phys<double>)];
     NbList nbl;                 // gas neighbour list of the density pass (nbl.idx null: none)
     XDragBufs xb;               // per-particle scratch of the ISPH / MK drag
+    SmallPlan small;            // the one-launch step of a small context (fn null: not taken)
+    void *bar = nullptr;        // its grid barrier
     bool nbl_valid = false;     // nbl belongs to the current binning
     bool prepared = false;      // binning and density of the current state are done
     bool forced = false;        // ... and acc holds its pressure acceleration
     bool counts_dirty = false;  // a binning did not finish: zero the cell counts first
+    bool counted = false;       // the cell counts are those of the current keys (else zero)
     bool has_frozen = false;
     int64_t steps = 0;
     int64_t device_bytes = 0;
@@ -250,6 +253,8 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
         }
     }
     c->has_frozen = any_frozen;
+    c->counts_dirty = c->counts_dirty || c->counted;  // counts of the replaced keys
+    c->counted = false;
     c->prepared = false;
     c->forced = false;
     c->nbl_valid = false;
@@ -291,6 +296,32 @@ int next_events(tfsph_ctx *c, cudaEvent_t **out)
     return TFSPH_OK;
 }
 
+// Whether the context's stream is being captured into a graph. Only contexts
+// of the one-launch step ask: a captured step leaves no counts for the next
+// one, so that a graph of steps can be replayed.
+bool capturing(const tfsph_ctx *c)
+{
+    if (!c->small.fn) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
+}
+
+// Zeroes the cell counts after a binning that did not finish, or where a
+// capture meets counts left by the step before it.
+int clear_counts(tfsph_ctx *c, bool cap)
+{
+    if (c->counts_dirty || (cap && c->counted)) {
+        TF_CUDA(c, cudaMemsetAsync(c->G.count, 0, (size_t)c->ncells * 4, c->stream));
+        TF_CUDA(c, cudaMemsetAsync(c->D.count, 0, (size_t)c->ncells * 4, c->stream));
+        c->counted = false;
+    }
+    return TFSPH_OK;
+}
+
 int prepare(tfsph_ctx *c, cudaEvent_t *ev = nullptr)
 {
     if (c->prepared) {
@@ -300,14 +331,13 @@ int prepare(tfsph_ctx *c, cudaEvent_t *ev = nullptr)
     }
     LaunchCtx L = lctx(c);
     L.ev = ev;
-    if (c->counts_dirty) {
-        TF_CUDA(c, cudaMemsetAsync(c->G.count, 0, (size_t)c->ncells * 4, c->stream));
-        TF_CUDA(c, cudaMemsetAsync(c->D.count, 0, (size_t)c->ncells * 4, c->stream));
-    }
+    const bool cap = capturing(c);
+    if (int rc = clear_counts(c, cap)) return rc;
     c->counts_dirty = true;
-    TF_CUDA(c, launch_bin(L, c->geo, c->G, c->D, c->bsum, c->nblk));
-    c->counts_dirty = false;
-    c->launches += (c->G.n + c->D.n > 0) ? 6 : 3;
+    TF_CUDA(c, launch_bin(L, c->geo, c->G, c->D, c->bsum, c->nblk, c->counted));
+    c->counts_dirty = cap;  // the memset of a capture has not run yet
+    c->launches += (c->G.n + c->D.n > 0) ? (c->counted ? 5 : 6) : 3;
+    c->counted = false;
     TF_CUDA(c, launch_density(L, c->geo, c->phys, c->G, c->rho_g, true, nullptr, nullptr,
                               c->nbl.idx ? &c->nbl : nullptr));
     c->nbl_valid = c->nbl.idx != nullptr;
@@ -486,6 +516,9 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
     c->d_flags = static_cast<int *>(tmp);
     e = cudaMemset(c->d_err, 0, 64);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
+    if (p->drag == TFSPH_DRAG_IDIC)
+        small_plan(c->geo, c->phys, c->precision, c->cell_acc, c->dim, n_gas, n_dust, &c->small);
+    c->bar = c->d_err + 8;  // in the error word's block
     // staging for host I/O: the larger phase's input arrays (+ frozen flags), or a field export
     const int64_t nmax = std::max<int64_t>(n_gas, n_dust);
     const size_t stage = std::max<size_t>((size_t)(2 * p->dim + 1) * (size_t)nmax * c->tsize + (size_t)n_gas + 256,
@@ -551,9 +584,6 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
     cudaEvent_t *ev = nullptr;
     int rc = next_events(c, &ev);
     if (rc) return rc;
-    if (ev) TF_CUDA(c, cudaEventRecord(ev[0], c->stream));
-    rc = forward_quantities(c, ev);
-    if (rc) return rc;
     StepArgs S;
     S.tau = tau;
     S.g[0] = gg[0];
@@ -562,6 +592,25 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
     S.tstar_mode = c->p.tstar_mode;
     S.cell_acc = c->cell_acc;
     S.has_frozen = c->has_frozen ? 1 : 0;
+    // a small context steps in one launch, unless its phases are being timed
+    // or a field export or snapshot has already done the first of them
+    if (c->small.fn && !ev && !c->prepared) {
+        const bool cap = capturing(c);
+        if ((rc = clear_counts(c, cap))) return rc;
+        c->counts_dirty = true;
+        TF_CUDA(c, launch_step_small(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->acc, S, c->small, c->bar, c->counted,
+                                     !cap));
+        c->counts_dirty = cap;
+        c->counted = !cap;
+        c->launches += 1;
+        c->forced = false;
+        c->nbl_valid = false;
+        c->steps += 1;
+        return TFSPH_OK;
+    }
+    if (ev) TF_CUDA(c, cudaEventRecord(ev[0], c->stream));
+    rc = forward_quantities(c, ev);
+    if (rc) return rc;
     if (c->p.drag == TFSPH_DRAG_IDIC) {
         TF_CUDA(c, launch_cell_update(L, c->geo, c->phys, c->G, c->D, c->acc, S));
         c->launches += 1;
@@ -884,6 +933,7 @@ int tfsph_load_state(tfsph_ctx *c, const void *buf, int mem_kind)
     c->forced = true;
     c->nbl_valid = false;  // the neighbour list is not part of a snapshot
     c->counts_dirty = true;
+    c->counted = false;
     if (h.steps >= 0) c->steps = h.steps;
     return TFSPH_OK;
 }
@@ -1056,6 +1106,12 @@ int tfsph_sync(tfsph_ctx *c)
     TF_CUDA(c, cudaMemcpy(&err, c->d_err, sizeof(int), cudaMemcpyDeviceToHost));
     if (err) {
         TF_CUDA(c, cudaMemset(c->d_err, 0, sizeof(int)));
+        if (err & kErrTimeout) {
+            // the barrier and the counts were left as the wait found them
+            TF_CUDA(c, cudaMemset(c->bar, 0, 32));
+            c->counts_dirty = true;
+            return fail(c, TFSPH_E_TIMEOUT, "a grid barrier of the one-launch step waited too long");
+        }
         if (err & kErrBadTstop) return fail(c, TFSPH_E_NONFINITE, "a t_stop value was <= 0 or not finite");
         return fail(c, TFSPH_E_INTERNAL, "device-side consistency check failed");
     }

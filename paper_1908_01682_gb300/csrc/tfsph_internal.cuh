@@ -65,6 +65,7 @@ template <class T> struct Geo {
     T halfL[3];
     T h2x4;        // (T)(4 h^2): neighbour iff r^2 < h2x4
     T lim2;        // squared pruning radius for candidate cells (2h plus margin)
+    T reach0;      // that radius in cells along x, rounded up (the 1D window)
     T wnorm;       // sigma_d / h^d
     T fnorm;       // sigma_d / h^(d+2): (1/r) dW/dr = fnorm * g(q)
     T inv_h;
@@ -158,8 +159,9 @@ struct LaunchCtx {
 
 // bin.cu
 cudaError_t launch_keys(const LaunchCtx &L, const void *geo, const PhaseBufs &P);
+// counted: the cell counts of the current keys are there already.
 cudaError_t launch_bin(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D,
-                       uint32_t *bsum, int64_t nblk);
+                       uint32_t *bsum, int64_t nblk, bool counted);
 cudaError_t launch_pack(const LaunchCtx &L, PhaseBufs &P, const void *const *src, int ncomp_v,
                         const uint8_t *frozen, bool is_gas);
 cudaError_t launch_unpack(const LaunchCtx &L, const PhaseBufs &P, int what, void *out, int order,
@@ -253,6 +255,7 @@ void make_geo_phys(const tfsph_params &p, const int ncell[3], uint32_t ncells, G
     }
     G.h2x4 = T(4.0 * p.h * p.h);
     G.lim2 = T(reach * reach * (1.0 + 16.0 * u));
+    G.reach0 = T(reach * (1.0 + 16.0 * u) * ((double)ncell[0] / (p.hi[0] - p.lo[0])) * (1.0 + 4.0 * u));
     const double sigma = p.dim == 1 ? 2.0 / 3.0 : (p.dim == 2 ? 10.0 / (7.0 * M_PI) : 1.0 / M_PI);
     G.wnorm = T(sigma / pow(p.h, p.dim));
     G.fnorm = T(sigma / pow(p.h, p.dim + 2));
@@ -288,6 +291,23 @@ struct StepArgs {
 };
 cudaError_t launch_cell_update(const LaunchCtx &L, const void *geo, const void *phys,
                                PhaseBufs &G, PhaseBufs &D, const void *acc, const StepArgs &S);
+// small.cu: the whole IDIC step of a small context in one cooperative launch.
+// small_plan decides once per context whether it takes it (up to
+// kSmallParticles particles of both phases and kSmallCells cells). counted:
+// the cell counts are those of the current keys; count: leave those of the
+// next keys.
+constexpr int64_t kSmallParticles = 65536;
+constexpr uint32_t kSmallCells = 32768;
+struct SmallPlan {
+    void *fn = nullptr;  // NULL: not taken
+    int grid = 0, threads = 128, lanes = 1;
+    bool cluster = false;
+};
+bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, int dim, int64_t ng, int64_t nd,
+                SmallPlan *P);
+cudaError_t launch_step_small(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
+                              void *rho, void *acc, const StepArgs &S, const SmallPlan &P, void *bar, bool counted, bool count);
+
 // xdrag.cu: the ISPH or MK drag and particle update (scheme TFSPH_DRAG_ISPH |
 // TFSPH_DRAG_MK) after binning, gas and dust densities and the gas pressure
 // force. Scratch per particle: g4, d4, d4b (V4) and g1 (T).
