@@ -371,6 +371,11 @@ def _is_torch(a) -> bool:
     return type(a).__module__.startswith("torch")
 
 
+def _rows_contiguous(a, dim: int) -> bool:
+    """A plain (>= dim, n) torch tensor whose rows are contiguous (a view a[k] then has its data where it lies)."""
+    return _is_torch(a) and a.dim() == 2 and a.shape[0] >= dim and (a.shape[1] <= 1 or a.stride(1) == 1)
+
+
 class Context:
     """Owns one tfsph context. Inputs are either all numpy arrays (host) or all
     torch CUDA tensors (device), in the context's precision, component-major."""
@@ -400,6 +405,15 @@ class Context:
             mem = TFSPH_MEM_HOST
             conv = lambda a: np.ascontiguousarray(a, dtype=self.dtype)
             ptr = lambda a: a.ctypes.data
+        if mem == TFSPH_MEM_DEVICE and all(_rows_contiguous(a, d) for a in (gx, gv, dx, du)):
+            # (dim, n) tensors with contiguous rows: the rows' addresses, without a view per component
+            rows = lambda a: [a.data_ptr() + k * a.stride(0) * a.element_size() for k in range(d)]
+            tail = [conv(ge)] if self.params.eos == TFSPH_EOS_ADIABATIC else []
+            last = conv(tstop)
+            fz = None if frozen is None else frozen.contiguous()
+            self._keep = [gx, gv, dx, du, last, fz] + tail
+            return (rows(gx) + rows(gv) + [ptr(a) for a in tail], rows(dx) + rows(du) + [ptr(last)],
+                    None if fz is None else ptr(fz), mem)
         comps = [conv(gx[k]) for k in range(d)] + [conv(gv[k]) for k in range(d)]
         if self.params.eos == TFSPH_EOS_ADIABATIC:
             comps.append(conv(ge))

@@ -219,27 +219,31 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     const int ngas_arr = 2 * d + (c->p.eos == TFSPH_EOS_ADIABATIC ? 1 : 0);
     const int ndust_arr = 2 * d + 1;
     LaunchCtx L = lctx(c);
-    std::vector<const void *> dv;
-    const uint8_t *dfz = nullptr;
+    std::vector<const void *> gv, dv;
+    const uint8_t *dfz = nullptr, *none = nullptr;
+    const int gas_w = c->p.eos == TFSPH_EOS_ADIABATIC;
     bool staged = false;
-    int rc = stage_inputs(c, gas, ngas_arr, c->G.n, frozen, mem_kind, dv, &dfz, &staged);
+    int rc = stage_inputs(c, gas, ngas_arr, c->G.n, frozen, mem_kind, gv, &dfz, &staged);
     if (rc) return rc;
     c->G.cur = 0;
-    TF_CUDA(c, launch_pack(L, c->G, dv.data(), c->p.eos == TFSPH_EOS_ADIABATIC, dfz, true));
-    // the gas staging area is reused for dust only after the pack has consumed it
-    if (staged) TF_CUDA(c, cudaStreamSynchronize(c->stream));
-    rc = stage_inputs(c, dust, ndust_arr, c->D.n, nullptr, mem_kind, dv, &dfz);
-    if (rc) return rc;
     c->D.cur = 0;
-    TF_CUDA(c, launch_pack(L, c->D, dv.data(), 1, nullptr, false));
-    TF_CUDA(c, launch_keys(L, c->geo, c->G));
-    TF_CUDA(c, launch_keys(L, c->geo, c->D));
-    TF_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
-    TF_CUDA(c, launch_check(L, c->geo, c->G, 1, c->d_flags));
-    TF_CUDA(c, launch_check(L, c->geo, c->D, 0, c->d_flags));
+    PhaseBufs G = c->G;
+    if (staged) {
+        // the staging area is reused for dust only after the gas is packed
+        PhaseBufs no_dust = c->D;
+        no_dust.n = 0;
+        TF_CUDA(c, launch_load(L, c->geo, G, no_dust, gv.data(), gas_w, dfz, nullptr, c->d_flags));
+        TF_CUDA(c, cudaStreamSynchronize(c->stream));
+        G.n = 0;
+    }
+    rc = stage_inputs(c, dust, ndust_arr, c->D.n, nullptr, mem_kind, dv, &none);
+    if (rc) return rc;
+    TF_CUDA(c, launch_load(L, c->geo, G, c->D, gv.data(), gas_w, dfz, dv.data(), c->d_flags));
     int flags = 0;
     TF_CUDA(c, cudaMemcpyAsync(&flags, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     TF_CUDA(c, cudaStreamSynchronize(c->stream));
+    // the flags are zero between loads
+    if (flags) TF_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
     if (flags & 1) return fail(c, TFSPH_E_NONFINITE, "non-finite position, velocity or energy in the input");
     if (flags & 4) return fail(c, TFSPH_E_NONFINITE, "dust t_stop must be finite and > 0");
     if (flags & 2) return fail(c, TFSPH_E_OUT_OF_DOMAIN, "a moving particle lies outside [lo, hi)");
@@ -512,8 +516,7 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
     if ((rc = dalloc(c, &c->scalar, 64))) return bail(rc);
     if ((rc = dalloc(c, &tmp, 64))) return bail(rc);
     c->d_err = static_cast<int *>(tmp);
-    if ((rc = dalloc(c, &tmp, 64))) return bail(rc);
-    c->d_flags = static_cast<int *>(tmp);
+    c->d_flags = c->d_err + 4;  // in the error word's block, zeroed below
     e = cudaMemset(c->d_err, 0, 64);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
     if (p->drag == TFSPH_DRAG_IDIC)

@@ -167,8 +167,10 @@ cudaError_t launch_pack(const LaunchCtx &L, PhaseBufs &P, const void *const *src
 cudaError_t launch_unpack(const LaunchCtx &L, const PhaseBufs &P, int what, void *out, int order,
                           const void *aux);
 cudaError_t launch_set_tstop(const LaunchCtx &L, PhaseBufs &D, const void *t_stop);
-cudaError_t launch_check(const LaunchCtx &L, const void *geo, const PhaseBufs &P, int is_gas,
-                         int *flags);
+// Pack, keys and input check of a single context's state (device-visible
+// component arrays in id order; a phase of zero particles is skipped).
+cudaError_t launch_load(const LaunchCtx &L, const void *geo, const PhaseBufs &G, const PhaseBufs &D,
+                        const void *const *gas, int gas_w, const uint8_t *frozen, const void *const *dust, int *flags);
 cudaError_t launch_max_speed(const LaunchCtx &L, const void *phys, const PhaseBufs &G,
                              void *partials, int nblk, void *result);
 cudaError_t launch_debug_keys(const LaunchCtx &L, const void *geo, const PhaseBufs &P, uint32_t *out);
