@@ -73,6 +73,22 @@ template <int MODE> struct ModeUses {
     static constexpr bool rho = MODE == 3 || MODE == 5;
 };
 
+// 1 / sqrt(x) in binary64 by one third-order step from the hardware's
+// approximation y0 (relative error e / 2 with e = 1 - x y0^2 about 2^-19):
+// y = y0 (1 + e / 2 + 3 e^2 / 8), the binomial series of (1 - e)^(-1/2) up to
+// e^2, so its truncation is below 2^-57. Five operations on the binary64 pipe,
+// which bounds the 3D force in FP64, where a square root and a division take
+// about twenty. Below 2^-1000 it gives 0: a zero displacement, whose kernel
+// terms vanish.
+__device__ __forceinline__ double rsqrt_wide(double x)
+{
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(x));
+    const double e = __fma_rn(-(x * y0), y0, 1.0);
+    const double y = __fma_rn(y0 * e, __fma_rn(0.375, e, 0.5), y0);
+    return x >= 0x1p-1000 ? y : 0.0;
+}
+
 // Distance of a pair from r^2 and its displacement. In 1D binary64 it is |d|,
 // which is what the rounded square root of the rounded square returns (away
 // from underflow), without the square root's chain on the binary64 pipe.
@@ -84,7 +100,19 @@ template <class T, int DIM> __device__ __forceinline__ T pair_dist(T r2, const T
 template <class T, int DIM> __device__ __forceinline__ T pair_inv_dist(T r2, const T d[3])
 {
     if (DIM == 1 && sizeof(T) == 8) return T(1) / fabs(d[0]);
+    if constexpr (DIM == 3 && sizeof(T) == 8) return rsqrt_wide(r2);
     return pair_rsqrt(r2);
+}
+
+// 1/r, and 0 for a zero displacement.
+template <class T, int DIM> __device__ __forceinline__ T pair_inv_dist0(T r2, const T d[3])
+{
+    if constexpr (sizeof(T) == 8) {
+        if (DIM == 3) return pair_inv_dist<T, DIM>(r2, d);
+        const T inv = pair_inv_dist<T, DIM>(r2, d);
+        return __double_as_longlong(r2) != 0 ? inv : T(0);
+    }
+    return r2 >= pair_r2_min<T>() ? pair_inv_dist<T, DIM>(r2, d) : T(0);
 }
 
 // ---------------------------------------------------------------------------
@@ -156,10 +184,10 @@ template <class T, int MODE> struct PairAcc {
             // which acc_store applies once together with m_g
             // self or coincident particle (r^2 below the smallest normal):
             // 1/r taken as 0, so q = 0, g is finite and s d = 0 (no branch)
-            const T inv_r = r2 >= pair_r2_min<T>() ? pair_inv_dist<T, DIM>(r2, d) : T(0);
+            const T inv_r = pair_inv_dist0<T, DIM>(r2, d);
             const T q = r2 * inv_r * G.inv_h;
-            const T a = fmax(T(2) - q, T(0));
-            const T g = q < T(1) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
+            const T a = positive_part(T(2) - q);
+            const T g = below_one(q) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
             const T s = (qa + pb.w) * g;
             ax -= s * d[0];
             ay -= s * d[1];
@@ -309,10 +337,10 @@ __device__ __forceinline__ T pair_term(const PairAcc<T, MODE> &A, const Geo<T> &
         const T w = kernel_w4(pair_dist<T, DIM>(r2, d) * G.inv_h);
         return in ? w : T(0);
     }
-    const T inv_r = r2 >= pair_r2_min<T>() ? pair_inv_dist<T, DIM>(r2, d) : T(0);
+    const T inv_r = pair_inv_dist0<T, DIM>(r2, d);
     const T q = r2 * inv_r * G.inv_h;
-    const T a = fmax(T(2) - q, T(0));
-    const T g = q < T(1) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
+    const T a = positive_part(T(2) - q);
+    const T g = below_one(q) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
     return in ? (A.qa + pb.w) * g : T(0);
 }
 template <class T, int DIM, int MODE>

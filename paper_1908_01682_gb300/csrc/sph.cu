@@ -29,6 +29,11 @@ constexpr int kTileThreads = 256;
 // force): 4 CTAs per SM, each with its static arrays and the 1 KB the
 // hardware reserves, within the SM's 228 KB (4 x (56832 + 64 + 1024) bytes).
 constexpr int kTileSmemPos = 56832;
+// The same for the binary64 state in 3D, whose tiles also hold a binary32 copy
+// of the positions: 2 CTAs per SM. They are bound by the binary64 pipe, which
+// a few warps fill.
+constexpr int kTileSmemWide = 112 * 1024;
+template <class T, int DIM> constexpr bool kPrefilter = sizeof(T) == 8 && DIM == 3;
 
 // One thread per particle, candidates from global memory.
 template <class T, int DIM, int MODE>
@@ -314,13 +319,51 @@ __device__ __noinline__ void particle_tile(const Geo<T> G, const Phys<T> Ph, con
     acc_store(A, Ph, a, mass, vel, out_rho, pr_out, out_acc, nullptr, nullptr);
 }
 
+// The recording walk of a binary64 particle in 3D (seamless tiles): rows and
+// candidates are taken in binary32 from a copy of the staged positions
+// relative to the tile, in units of h (sf; pf the particle's own), so that the binary64 pipe,
+// at 2 lanes per SM and clock the bound of these sums, only sees the listed
+// pairs. thr and reach2 carry margins over 4h^2 and the pruning radius that
+// cover the rounding of the relative coordinates, of the cell fractions f and
+// of the arithmetic here; a pair between 4h^2 and thr lies where the kernel is
+// zero (its (2 - q) is clamped) and adds nothing.
+__device__ __forceinline__ void record_walk_f32(const int R[3], const float w[3], const float inv_w[3], float reach2,
+                                                float thr, const TileCfg &C, const int h[3], const float f[3],
+                                                const float4 pf, const uint16_t *lstart, const float4 *sf, NbRec &rec)
+{
+    const float tz = approx_sqrt(reach2) * inv_w[2];
+    const int oz1 = min(R[2], max(0, floor_int(f[2] + tz))), oz0 = -min(R[2], max(0, floor_int(tz - f[2] + 1.0f)));
+#pragma unroll 1
+    for (int oz = oz0; oz <= oz1; ++oz) {
+        const float sz = slab_dist(oz, f[2]) * w[2], dz2 = sz * sz;
+        const float ty = approx_sqrt(fmaxf(reach2 - dz2, 0.0f)) * inv_w[1];
+        const int oy1 = min(R[1], max(0, floor_int(f[1] + ty))), oy0 = -min(R[1], max(0, floor_int(ty - f[1] + 1.0f)));
+#pragma unroll 1
+        for (int oy = oy0; oy <= oy1; ++oy) {
+            const float sy = slab_dist(oy, f[1]) * w[1];
+            const float tx = approx_sqrt(fmaxf(reach2 - dz2 - sy * sy, 0.0f)) * inv_w[0];
+            const int ohi = min(R[0], max(0, floor_int(f[0] + tx)));
+            const int olo = -min(R[0], max(0, floor_int(tx - f[0] + 1.0f)));
+            const int hrow = C.H[0] * ((h[1] + oy) + C.H[1] * (h[2] + oz)) + h[0];
+            const int j1 = lstart[hrow + ohi + 1];
+#pragma unroll 1
+            for (int j = lstart[hrow + olo]; j < j1; ++j) {
+                const float4 q = sf[j];
+                const float dx = pf.x - q.x, dy = pf.y - q.y, dz = pf.z - q.z;
+                if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < thr) rec.push(j, false);
+            }
+        }
+    }
+}
+
 // Pair sums over a particle's recorded list (groups `e[g * st]` of four
 // 16-bit entries, n entries), in the recorded order (SEAMLESS: the tile
-// recorded no seam flags).
-template <class T, int DIM, int MODE, bool SEAMLESS>
+// recorded no seam flags; RO: the list was written by an earlier kernel).
+template <class T, int DIM, int MODE, bool SEAMLESS, bool RO = true>
 __device__ __forceinline__ void read_list(PairAcc<T, MODE> &A, const Geo<T> &G, const Phys<T> &Ph, const V4<T> &pa,
                                           const V4<T> *spos, const unsigned long long *e, size_t st, int n)
 {
+    auto load = [](const unsigned long long *q) { return RO ? __ldg(q) : *q; };
     auto pair = [&](uint32_t cur) {
         const V4<T> pb = spos[cur & 0x7FFFu];
         T d[3];
@@ -341,29 +384,30 @@ __device__ __forceinline__ void read_list(PairAcc<T, MODE> &A, const Geo<T> &G, 
     int g = 0;
     unsigned long long c0, c1, n0 = 0, n1 = 0;
     if (ng >= 2) {
-        n0 = __ldg(&e[0]);
-        n1 = __ldg(&e[st]);
+        n0 = load(&e[0]);
+        n1 = load(&e[st]);
     }
     for (; g + 2 <= ng; g += 2) {
         c0 = n0;
         c1 = n1;
         if (g + 4 <= ng) {
-            n0 = __ldg(&e[(size_t)(g + 2) * st]);
-            n1 = __ldg(&e[(size_t)(g + 3) * st]);
+            n0 = load(&e[(size_t)(g + 2) * st]);
+            n1 = load(&e[(size_t)(g + 3) * st]);
         }
         quad(c0);
         quad(c1);
     }
-    if (g < ng) quad(__ldg(&e[(size_t)g++ * st]));
+    if (g < ng) quad(load(&e[(size_t)g++ * st]));
     const int m = n & 3;
     if (m) {
-        const unsigned long long w = __ldg(&e[(size_t)g * st]);
+        const unsigned long long w = load(&e[(size_t)g * st]);
         for (int u = 0; u < m; ++u) pair((uint32_t)(w >> (16 * u)) & 0xFFFFu);
     }
 }
 
 template <class T, int DIM, int MODE>
-__global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? ((MODE == 0 || MODE == 2) ? 4 : 3) : 1)
+__global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? ((MODE == 0 || MODE == 2) ? 4 : 3)
+                                                         : (kPrefilter<T, DIM> && (MODE == 0 || MODE == 2) ? 2 : 1))
 k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, const V4<T> *__restrict__ vel,
             const T *__restrict__ rho, const uint32_t *__restrict__ id, const uint32_t *__restrict__ start, T mass,
             T *__restrict__ out_rho, T *pr_out, V4<T> *__restrict__ out_acc, int32_t *__restrict__ cnt,
@@ -383,6 +427,8 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
     V4<T> *svel = spos + C.cap;                        // modes staging a second V4
     T *srho = reinterpret_cast<T *>(svel + (ModeUses<MODE>::vel ? C.cap : 0));  // modes staging a scalar
     uint32_t *sid = reinterpret_cast<uint32_t *>(spos + C.cap);  // MODE 1
+    float4 *sf = reinterpret_cast<float4 *>(spos + C.cap);       // binary32 copy (kPrefilter, MODE 0)
+    constexpr bool kPre = kPrefilter<T, DIM> && MODE == 0;
 
     const int tid = threadIdx.x;
     int b = blockIdx.x;
@@ -430,6 +476,17 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
             }
         }
     }
+
+    // origin of the binary32 copy: the tile's corner, in staged coordinates
+    T org[3] = {T(0), T(0), T(0)};
+    if constexpr (kPre) {
+#pragma unroll
+        for (int k = 0; k < DIM; ++k) org[k] = G.lo[k] + T(c0[k]) * G.w[k] - orig[k];
+    }
+    auto copy32 = [&](int j, const V4<T> &q) {
+        if constexpr (kPre) sf[j] = make_float4((float)((q.x - org[0]) * G.inv_h), (float)((q.y - org[1]) * G.inv_h),
+                                (float)((q.z - org[2]) * G.inv_h), 0.0f);
+    };
 
     // owned rows: global start and particle count
     for (int r = tid; r < C.nrows; r += blockDim.x) {
@@ -491,7 +548,9 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                 const uint32_t g0 = (uint32_t)hr_first[r];
                 for (int u = lane; u < m; u += 16) {
                     const uint32_t gi = g0 + (uint32_t)u;
-                    spos[j0 + u] = pos[gi];
+                    const V4<T> q = pos[gi];
+                    spos[j0 + u] = q;
+                    copy32(j0 + u, q);
                     if (ModeUses<MODE>::vel) svel[j0 + u] = vel[gi];
                     if (ModeUses<MODE>::rho) srho[j0 + u] = rho[gi];
                     if (MODE == 1) sid[j0 + u] = id[gi];
@@ -548,6 +607,7 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                     if (DIM > 1) q.y = sub_rn(q.y, sh[1]);
                     if (DIM > 2) q.z = sub_rn(q.z, sh[2]);
                     spos[j] = q;
+                    copy32(j, q);
                     if (ModeUses<MODE>::vel) svel[j] = vel[gi];
                     if (ModeUses<MODE>::rho) srho[j] = rho[gi];
                     if (MODE == 1) sid[j] = id[gi];
@@ -590,7 +650,37 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
             const bool listed = nbl.idx && p < nbl.owned_cap;
             const size_t oc = (size_t)nbl.owned_cap;
             const size_t lbase = (size_t)blockIdx.x * (size_t)(nbl.cap / 4 + 1) * oc + (size_t)p;
-            if (MODE == 0 && listed) {
+            if (kPre && listed && seamless) {
+                if constexpr (kPre) {
+                    NbRec rec{nbl.idx + lbase, (uint32_t)oc, nbl.cap / 4, 0};
+                    const int ja = lstart[hrow + G.R[0]] + k;
+                    T t[3];
+                    const int h[3] = {axis_cell(pc.x, G.lo[0], G.inv_w[0], G.n[0], t[0]) - c0[0] + G.R[0],
+                                      axis_cell(pc.y, G.lo[1], G.inv_w[1], G.n[1], t[1]) - c0[1] + G.R[1],
+                                      axis_cell(pc.z, G.lo[2], G.inv_w[2], G.n[2], t[2]) - c0[2] + G.R[2]};
+                    float f[3], w[3], iw[3], far = 0.0f;
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        f[d] = (float)(t[d] - T(h[d] + c0[d] - G.R[d]));
+                        w[d] = (float)(G.w[d] * G.inv_h);
+                        iw[d] = (float)(G.inv_w[d] * G.h);
+                        far = fmaxf(far, (float)C.H[d] * w[d]);
+                    }
+                    // in units of h; relative coordinates are below `far`, each
+                    // rounded to 2^-24 far: 2^-19 far covers the displacement
+                    const float reach = 2.0f + 0x1p-19f * far;
+                    record_walk_f32(G.R, w, iw, reach * reach * (1.0f + 0x1p-18f) + 0x1p-19f * far * reach,
+                                    reach * reach * (1.0f + 0x1p-20f), C, h, f, sf[ja], lstart, sf, rec);
+                    const int n = rec.n;
+                    nbl.cnt[(size_t)blockIdx.x * oc + p] = n <= nbl.cap ? (uint16_t)n : kNbNone;
+                    if (n > nbl.cap) {
+                        particle_tile<T, DIM, MODE, true>(G, Ph, C, c0[0], c0[1], c0[2], pa, pc, a, lstart, spos, vel,
+                                                          mass, out_rho, pr_out, out_acc);
+                        continue;
+                    }
+                    read_list<T, DIM, MODE, true, false>(A, G, Ph, pa, spos, nbl.idx + lbase, oc, n);
+                }
+            } else if (MODE == 0 && listed) {
                 // density pass: record the neighbours in walk order
                 NbRec rec{nbl.idx + lbase, (uint32_t)oc, nbl.cap / 4, 0};
                 if (seamless)
@@ -631,11 +721,14 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-template <class T, int MODE> constexpr int tile_bytes_per_particle()
+template <class T, int DIM, int MODE> constexpr int tile_bytes_per_particle()
 {
-    return (int)sizeof(V4<T>) + (ModeUses<MODE>::vel ? (int)sizeof(V4<T>) : 0) +
+    return (int)sizeof(V4<T>) + (kPrefilter<T, DIM> && (MODE == 0 || MODE == 2) ? (int)sizeof(float4) : 0) + (ModeUses<MODE>::vel ? (int)sizeof(V4<T>) : 0) +
            (ModeUses<MODE>::rho ? (int)sizeof(T) : 0) + (MODE == 1 ? 4 : 0);
 }
+
+// Shared memory of the listing passes' tiles (the list belongs to their shape).
+template <class T, int DIM> constexpr int tile_budget() { return kPrefilter<T, DIM> ? kTileSmemWide : kTileSmemPos; }
 
 // Tile shape for a phase with `mean` particles per cell. The CTA's threads
 // take the owned particles in turn; a tile holds about 7/8 of them per
@@ -714,8 +807,8 @@ cudaError_t pair_launch(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, 
                         T *pr_out, V4<T> *out_acc, int32_t *cnt, uint64_t *fpr, double mean,
                         NbList nb = NbList{})
 {
-    constexpr int bpp = tile_bytes_per_particle<T, MODE>();
-    const int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : kTileSmemPos;
+    constexpr int bpp = tile_bytes_per_particle<T, DIM, MODE>();
+    const int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : tile_budget<T, DIM>();
     TileCfg C{};
     size_t smem = 0;
     if (plan_tiles(G, DIM, mean, bpp, budget, C, smem)) {
@@ -894,7 +987,9 @@ bool nblist_layout_t(const Geo<T> &G, int dim, int64_t n, int *cap, int *owned_c
     // the density pass's tiles (MODE 0 plan)
     TileCfg C{};
     size_t smem = 0;
-    if (!plan_tiles(G, dim, mean, tile_bytes_per_particle<T, 0>(), kTileSmemPos, C, smem) || C.cap > 0x7FFF) return false;
+    const int bpp = dim == 3 ? tile_bytes_per_particle<T, 3, 0>() : tile_bytes_per_particle<T, 1, 0>();
+    const int budget = dim == 3 ? tile_budget<T, 3>() : tile_budget<T, 1>();
+    if (!plan_tiles(G, dim, mean, bpp, budget, C, smem) || C.cap > 0x7FFF) return false;
     double owned = mean;
     for (int k = 0; k < dim; ++k) owned *= (double)C.T[k];
     const double cap_d = 32.0 * std::ceil(want / 32.0);

@@ -443,38 +443,45 @@ template <> __device__ __forceinline__ double pair_r2_min<double>() { return 4.9
 __device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
 
+// max(x, 0), and q < 1 for q >= 0. In binary64 from the high word, on the
+// integer pipe: the pair sums are bound by the 2-lane binary64 pipe.
+__device__ __forceinline__ float positive_part(float x) { return fmaxf(x, 0.0f); }
+__device__ __forceinline__ double positive_part(double x) { return __double2hiint(x) < 0 ? 0.0 : x; }
+__device__ __forceinline__ bool below_one(float q) { return q < 1.0f; }
+__device__ __forceinline__ bool below_one(double q) { return __double2hiint(q) < 0x3ff00000; }
+
 // M4 cubic spline (support 2h), branch free on q in [0, 2):
 //   W = wnorm * (q < 1 ? 1 - 3/2 q^2 + 3/4 q^3 : 1/4 (2 - q)^3)
 //   (1/r) dW/dr = fnorm * (q < 1 ? -3 + 9/4 q : -3/4 (2 - q)^2 / q)
 template <class T> __device__ __forceinline__ T kernel_w(const Geo<T> &G, T q)
 {
-    const T a = fmax(T(2) - q, T(0));
+    const T a = positive_part(T(2) - q);
     const T inner = T(1) + q * q * (T(-1.5) + T(0.75) * q);
     const T outer = T(0.25) * a * a * a;
-    return G.wnorm * (q < T(1) ? inner : outer);
+    return G.wnorm * (below_one(q) ? inner : outer);
 }
 
 // 4 W / (sigma_d / h^d): the density sums add this and scale once at the end
 //   (q < 1 ? 4 - 6 q^2 + 3 q^3 : (2 - q)^3)
 template <class T> __device__ __forceinline__ T kernel_w4(T q)
 {
-    const T a = fmax(T(2) - q, T(0));
+    const T a = positive_part(T(2) - q);
     const T inner = T(4) + q * q * (T(-6) + T(3) * q);
-    return q < T(1) ? inner : a * a * a;
+    return below_one(q) ? inner : a * a * a;
 }
 
 template <class T> __device__ __forceinline__ T kernel_f(const Geo<T> &G, T q, T inv_q)
 {
-    const T a = fmax(T(2) - q, T(0));
-    return G.fnorm * (q < T(1) ? T(-3) + T(2.25) * q : T(-0.75) * a * a * inv_q);
+    const T a = positive_part(T(2) - q);
+    return G.fnorm * (below_one(q) ? T(-3) + T(2.25) * q : T(-0.75) * a * a * inv_q);
 }
 
 // d/dr of (1/r) dW/dr:
 //   fnorm / h * (q < 1 ? 9/4 : 3/4 (2 - q)(2 + q) / q^2)
 template <class T> __device__ __forceinline__ T kernel_fprime(const Geo<T> &G, T q, T inv_q)
 {
-    const T a = fmax(T(2) - q, T(0));
-    return G.fnorm * G.inv_h * (q < T(1) ? T(2.25) : T(0.75) * a * (q + T(2)) * inv_q * inv_q);
+    const T a = positive_part(T(2) - q);
+    return G.fnorm * G.inv_h * (below_one(q) ? T(2.25) : T(0.75) * a * (q + T(2)) * inv_q * inv_q);
 }
 
 }  // namespace tfsph
