@@ -517,6 +517,7 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
     if ((rc = dalloc(c, &tmp, 64))) return bail(rc);
     c->d_err = static_cast<int *>(tmp);
     c->d_flags = c->d_err + 4;  // in the error word's block, zeroed below
+    c->xb.gate = c->d_err + 5;
     e = cudaMemset(c->d_err, 0, 64);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
     if (p->drag == TFSPH_DRAG_IDIC)

@@ -9,9 +9,11 @@
 // (wall) gas particles enter the density and pressure sums and take no part
 // in the drag.
 //
-// Cross-phase sums: one thread per target particle walks the other phase's
-// candidate cells in global memory (the row walk of the gas pair sums), with
-// the same neighbour decision r^2 < 4h^2.
+// Cross-phase sums, with the neighbour decision of the gas pair sums. In 3D
+// (FP32, isothermal, no walls) a CTA stages the source particles of a tile of
+// cells and its halo, 32 bytes each, and its threads take one target each
+// (k_xsum_tile). Otherwise one thread per target walks the other phase's
+// candidate cells in global memory (k_xsum).
 //   ISPH at gas a over dust:  rho^d_a = m_d sum W,  K_a,  u_a = m_d sum u_j/rho_j W
 //   ISPH at dust j over gas:  rho^g_j = m_g sum W,  v_j = m_g sum_moving v_a/rho_a W,
 //     e_j (adiabatic), pressure acceleration A_j = -(Q_j + q_j G_j) (Eq. 14)
@@ -26,6 +28,7 @@
 // or the MK explicit update v' = v + tau (A + D + g), u' = u + tau (D + g); then
 // x' = x + tau v' (periodic wrap) and the next cell keys.
 #include "pair.cuh"
+#include "tile.cuh"
 
 namespace tfsph {
 namespace {
@@ -43,20 +46,22 @@ template <class T> struct XArgs {
     // sources (the other phase)
     const V4<T> *spos, *svel;
     const uint32_t *sid;
-    const uint32_t *sstart;
+    const uint32_t *sstart, *tstart;  // cell ranges of the sources and the targets
     const T *srho;      // source density (rho_d for ISPH at gas, rho_g otherwise)
     int has_frozen;     // gas carries frozen flags (in tid for gas targets, sid for gas sources)
     // outputs
     V4<T> *out4;        // ISPH gas: (u_a, K_a); ISPH dust: (v_j, rho^g_j); MK: D
     V4<T> *out4b;       // ISPH dust: (A_j, 0)
     T *out1;            // ISPH gas: rho^d_a
+    // where both forms of the sums are launched: the word that tells which runs
+    const int *gate = nullptr;
+    int run_if = 0;
 };
 
+// One target's sums over its candidate cells in global memory.
 template <class T, int DIM, int KIND>
-__global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 12 : 1) k_xsum(Geo<T> G, Phys<T> Ph, XArgs<T> X)
+__device__ __forceinline__ void xsum_global(const Geo<T> &G, const Phys<T> &Ph, const XArgs<T> &X, uint32_t t)
 {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= X.n) return;
     const bool gas_target = KIND == kIsphAtGas || KIND == kMkAtGas;
     if (gas_target && X.has_frozen && (X.tid[t] & kFrozenBit)) return;
     const V4<T> pt = X.tpos[t];
@@ -140,6 +145,414 @@ __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 12 : 1) k_xsum(Geo
         o.x = c * a[0]; o.y = c * a[1]; o.z = c * a[2]; o.w = T(0);
         X.out4[t] = o;
     }
+}
+
+template <class T, int DIM, int KIND>
+__global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 12 : 1) k_xsum(Geo<T> G, Phys<T> Ph, XArgs<T> X)
+{
+    if (X.gate && *X.gate != X.run_if) return;
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < (uint32_t)X.n) xsum_global<T, DIM, KIND>(G, Ph, X, t);
+}
+
+// ---------------------------------------------------------------------------
+// Tiled sums (3D, FP32, isothermal, no walls)
+// ---------------------------------------------------------------------------
+// A source is staged as (x, y, z, c1) and (vx, vy, vz, c2): c1 = 1/t_j (ISPH and
+// MK at gas), p/rho^2 (ISPH at dust) or 1/rho (MK at dust), c2 = 1/rho (ISPH).
+//
+// Walking the candidates in global memory took 20,600 instructions per warp of
+// targets with 13 of 32 lanes active, each load touching up to 32 lines: the
+// 60-odd instructions of a pair ran in every iteration in which any lane had a
+// neighbour. Here the lanes of a warp go through the same rows of cells
+// together and only test candidates; each lane puts its neighbours in a small
+// queue of its own (kQueue entries in shared memory), and when a queue is half
+// full every lane evaluates one entry, so that the pair arithmetic runs with
+// nearly all lanes active.
+__device__ __forceinline__ float approx_rcp(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+constexpr int kXTileThreads = 512;
+constexpr int kQueue = 8;
+// 2 CTAs per SM: 2 x (112 KB + static + 1 KB reserved) of 228 KB
+constexpr int kXTileSmem = 112 * 1024;
+constexpr int kXQueueBytes = kQueue * kXTileThreads * 2;
+
+__device__ __noinline__ void xsum_global_far(const Geo<float> G, const Phys<float> Ph, const XArgs<float> X, uint32_t t,
+                                             int kind)
+{
+    if (kind == kIsphAtGas) xsum_global<float, 3, kIsphAtGas>(G, Ph, X, t);
+    else if (kind == kIsphAtDust) xsum_global<float, 3, kIsphAtDust>(G, Ph, X, t);
+    else if (kind == kMkAtGas) xsum_global<float, 3, kMkAtGas>(G, Ph, X, t);
+    else xsum_global<float, 3, kMkAtDust>(G, Ph, X, t);
+}
+
+// The targets of a staged tile. SEAM: displacements take the periodic image
+// (tiles that could not be staged with their seam shifts).
+template <int KIND, bool SEAM>
+__device__ __forceinline__ void xsum_tile_walk(const Geo<float> &G, const Phys<float> &Ph, const TileCfg &C,
+                                               const int c0[3], const float orig[3], const XArgs<float> &X,
+                                               const uint16_t *lstart, const int *rowpref, const int *rowg,
+                                               const float4 *sa, const float4 *sb, uint16_t *queue, int owned)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const float eta2 = 0.001f * G.h * G.h;
+    for (int p0 = (int)threadIdx.x - lane; p0 < owned; p0 += blockDim.x) {
+        const bool live = p0 + lane < owned;
+        const int p = min(p0 + lane, owned - 1);
+        int lo = 0, hi = C.nrows - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (rowpref[mid] <= p) lo = mid;
+            else hi = mid - 1;
+        }
+        const uint32_t t = (uint32_t)(rowg[lo] + p - rowpref[lo]);
+        float4 pt = X.tpos[t];
+        float4 vt = make_float4(0.0f, 0.0f, 0.0f, 1.0f);
+        if (KIND == kMkAtGas || KIND == kMkAtDust) vt = X.tvel[t];
+        float f[3];
+        int h[3];
+        {
+            float tc;
+            h[0] = axis_cell(pt.x, G.lo[0], G.inv_w[0], G.n[0], tc);
+            f[0] = tc - (float)h[0];
+            h[1] = axis_cell(pt.y, G.lo[1], G.inv_w[1], G.n[1], tc);
+            f[1] = tc - (float)h[1];
+            h[2] = axis_cell(pt.z, G.lo[2], G.inv_w[2], G.n[2], tc);
+            f[2] = tc - (float)h[2];
+#pragma unroll
+            for (int k = 0; k < 3; ++k) h[k] += G.R[k] - c0[k];
+        }
+        if (!SEAM) {
+            pt.x = sub_rn(pt.x, orig[0]);
+            pt.y = sub_rn(pt.y, orig[1]);
+            pt.z = sub_rn(pt.z, orig[2]);
+        }
+        float s0 = 0.0f, s1 = 0.0f, a[3] = {0.0f, 0.0f, 0.0f};
+        float gs[3] = {0.0f, 0.0f, 0.0f}, qs[3] = {0.0f, 0.0f, 0.0f};
+        uint32_t head = 0, tail = 0;
+        // queue positions in bytes
+        constexpr uint32_t kSlot = 2 * kXTileThreads, kWrap = (kQueue - 1) * kSlot;
+        unsigned char *qu = reinterpret_cast<unsigned char *>(queue + threadIdx.x);
+
+        // every lane takes one of its neighbours; the sums leave out the
+        // kernel's normalisation and the mass, applied once at the end
+        auto pop = [&] {
+            if (head == tail) return;
+            const int j = *reinterpret_cast<const uint16_t *>(qu + (head & kWrap));
+            head += kSlot;
+            const float4 q = sa[j], v = sb[j];
+            float d[3];
+            const float r2 = pair_r2<float, 3, SEAM>(G, pt, q, d);
+            if (KIND == kIsphAtDust) {
+                const float inv_r = r2 >= pair_r2_min<float>() ? pair_rsqrt(r2) : 0.0f;
+                const float qq = r2 * inv_r * G.inv_h;
+                const float w = kernel_w4(qq);
+                s0 += w;
+                const float c = w * v.w;
+                a[0] += c * v.x;
+                a[1] += c * v.y;
+                a[2] += c * v.z;
+                const float e = positive_part(2.0f - qq);
+                const float F = below_one(qq) ? -3.0f + 2.25f * qq : (e * e) * (Ph.hm075 * inv_r);
+                const float Fq = F * q.w;
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    gs[k] += F * d[k];
+                    qs[k] += Fq * d[k];
+                }
+            } else {
+                const float w = kernel_w4(pair_sqrt(r2) * G.inv_h);
+                if (KIND == kIsphAtGas) {
+                    s0 += w;
+                    s1 += w * q.w;
+                    const float c = w * v.w;
+                    a[0] += c * v.x;
+                    a[1] += c * v.y;
+                    a[2] += c * v.z;
+                } else {
+                    const float rel = (vt.x - v.x) * d[0] + (vt.y - v.y) * d[1] + (vt.z - v.z) * d[2];
+                    const float c = approx_rcp(r2 + eta2) * (q.w * rel) * w;
+                    a[0] += c * d[0];
+                    a[1] += c * d[1];
+                    a[2] += c * d[2];
+                }
+            }
+        };
+
+#pragma unroll 1
+        for (int oz = -G.R[2]; oz <= G.R[2]; ++oz) {
+            const float sz = slab_dist(oz, f[2]) * G.w[2];
+            // (rows outside the halo: only where a target on a cell face is
+            // placed one cell off, beyond the radius by a rounding)
+            const float remz = live && (unsigned)(h[2] + oz) < (unsigned)C.H[2] ? G.lim2 - sz * sz : -1.0f;
+            if (!__any_sync(kAll, remz > 0.0f)) continue;
+#pragma unroll 1
+            for (int oy = -G.R[1]; oy <= G.R[1]; oy += 2) {
+                // two rows of cells at a time: [ja, ja + na), then [jb, jb + nb)
+                int jr[2] = {0, 0}, nr[2] = {0, 0};
+#pragma unroll
+                for (int m = 0; m < 2; ++m) {
+                    const float sy = slab_dist(oy + m, f[1]) * G.w[1];
+                    const float rem = oy + m <= G.R[1] ? remz - sy * sy : -1.0f;
+                    if (rem > 0.0f && (unsigned)(h[1] + oy + m) < (unsigned)C.H[1]) {
+                        const float tx = pair_sqrt(rem) * G.inv_w[0];
+                        const int ohi = min(G.R[0], max(0, floor_int(f[0] + tx)));
+                        const int olo = -min(G.R[0], max(0, floor_int(tx - f[0] + 1.0f)));
+                        const int row = C.H[0] * ((h[1] + oy + m) + C.H[1] * (h[2] + oz));
+                        jr[m] = lstart[row + max(h[0] + olo, 0)];
+                        nr[m] = lstart[row + min(h[0] + ohi + 1, C.H[0])] - jr[m];
+                    }
+                }
+                const int len = nr[0] + nr[1], jump = jr[1] - nr[0] - jr[0];
+                const int most = __reduce_max_sync(kAll, len);
+#pragma unroll 1
+                for (int k0 = 0; k0 < most; k0 += kQueue / 2) {
+                    bool near[kQueue / 2];
+                    int j[kQueue / 2];
+#pragma unroll
+                    for (int u = 0; u < kQueue / 2; ++u) {
+                        const int k = k0 + u;
+                        // (past a lane's candidates: some other staged word)
+                        j[u] = jr[0] + k + (k >= nr[0] ? jump : 0);
+                        float d[3];
+                        near[u] = pair_r2<float, 3, SEAM>(G, pt, sa[j[u]], d) < G.h2x4 && k < len;
+                    }
+#pragma unroll
+                    for (int u = 0; u < kQueue / 2; ++u)
+                        if (near[u]) {
+                            *reinterpret_cast<uint16_t *>(qu + (tail & kWrap)) = (uint16_t)j[u];
+                            tail += kSlot;
+                        }
+                    // room for the next half queue in every lane
+                    while (__any_sync(kAll, tail - head >= kSlot * (kQueue / 2))) pop();
+                }
+            }
+        }
+        while (__any_sync(kAll, tail != head)) pop();
+        if (!live) continue;
+
+        const float mw = (KIND == kIsphAtGas || KIND == kMkAtGas ? Ph.m_d : Ph.m_g) * Ph.wnorm4;
+        if (KIND == kIsphAtGas) {
+            X.out4[t] = make_float4(mw * a[0], mw * a[1], mw * a[2], mw * s1);
+            X.out1[t] = mw * s0;
+        } else if (KIND == kIsphAtDust) {
+            s0 *= mw;
+            const float qj = s0 > 0.0f ? Ph.cs2 / s0 : 0.0f, mf = -Ph.mfnorm;
+            X.out4[t] = make_float4(mw * a[0], mw * a[1], mw * a[2], s0);
+            X.out4b[t] = make_float4(mf * (qs[0] + qj * gs[0]), mf * (qs[1] + qj * gs[1]), mf * (qs[2] + qj * gs[2]),
+                                     0.0f);
+        } else {
+            const float c = -3.0f * mw / (KIND == kMkAtGas ? X.trho[t] : vt.w);
+            X.out4[t] = make_float4(c * a[0], c * a[1], c * a[2], 0.0f);
+        }
+    }
+}
+
+template <int KIND>
+__global__ void __launch_bounds__(kXTileThreads, 2)
+k_xsum_tile(Geo<float> G, Phys<float> Ph, TileCfg C, XArgs<float> X)
+{
+    if (X.gate && *X.gate != X.run_if) return;
+    extern __shared__ __align__(64) unsigned char smem[];
+    __shared__ int wsum[kXTileThreads / 32];
+    uint16_t *lstart = reinterpret_cast<uint16_t *>(smem);                 // nhalo + 1
+    int *rowpref = reinterpret_cast<int *>(smem + lstart_bytes(C.nhalo));  // nrows + 1
+    int *rowg = rowpref + C.nrows + 1;                                     // nrows
+    float4 *sa = reinterpret_cast<float4 *>(smem + C.offset);
+    float4 *sb = sa + C.cap;
+    uint16_t *queue = reinterpret_cast<uint16_t *>(sb + C.cap);
+
+    const int tid = threadIdx.x;
+    int b = blockIdx.x;
+    const int tx = b % C.nt[0];
+    b /= C.nt[0];
+    const int ty = b % C.nt[1], tz = b / C.nt[1];
+    const int c0[3] = {tx * C.T[0], ty * C.T[1], tz * C.T[2]};
+    int ext[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) ext[k] = min(C.T[k], G.n[k] - c0[k]);
+
+    // seam shifts, as in the gas pair sums: exact where lo = 0 and the halo
+    // lies over one seam of the axis only
+    int low[3] = {0, 0, 0}, high[3] = {0, 0, 0};
+    bool crosses = false, exact = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        if (!G.per[k]) continue;
+        low[k] = c0[k] < G.R[k];
+        high[k] = c0[k] + ext[k] + G.R[k] > G.n[k];
+        if (low[k] || high[k]) {
+            crosses = true;
+            if (!(G.lo[k] == 0.0f) || (low[k] && high[k]) || (high[k] && 2 * (c0[k] - G.R[k]) < G.n[k])) exact = false;
+        }
+    }
+    const bool shifted = crosses && exact;
+    float orig[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) orig[k] = shifted && high[k] ? G.L[k] : 0.0f;
+
+    for (int r = tid; r < C.nrows; r += blockDim.x) {
+        const int oy = r % C.T[1], oz = r / C.T[1];
+        int c = 0, g = 0;
+        if (oy < ext[1] && oz < ext[2]) {
+            const uint32_t key = (uint32_t)G.n[0] * ((uint32_t)(c0[1] + oy) + (uint32_t)G.n[1] * (uint32_t)(c0[2] + oz));
+            g = (int)X.tstart[key + c0[0]];
+            c = (int)X.tstart[key + c0[0] + ext[0]] - g;
+        }
+        rowg[r] = g;
+        rowpref[r] = c;
+    }
+    // the global cell of halo cell h, or -1
+    auto halo_key = [&](int h, int hk[3]) -> int {
+        halo_coords(h, C, hk[0], hk[1], hk[2]);
+        int g[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) g[k] = hk[k] < ext[k] + 2 * G.R[k] ? halo_cell(G, k, c0[k], hk[k]) : -1;
+        if (g[0] < 0 || g[1] < 0 || g[2] < 0) return -1;
+        return (int)((uint32_t)g[0] + (uint32_t)G.n[0] * ((uint32_t)g[1] + (uint32_t)G.n[1] * (uint32_t)g[2]));
+    };
+    for (int h = tid; h < C.nhalo; h += blockDim.x) {
+        int hk[3];
+        const int key = halo_key(h, hk);
+        // a count that does not fit 16 bits makes the tile exceed cap anyway
+        lstart[h] = key < 0 ? 0 : (uint16_t)min(X.sstart[key + 1] - X.sstart[key], 0xFFFFu);
+    }
+    __syncthreads();
+    const int total = block_scan_smem(lstart, C.nhalo, wsum);
+    block_scan_smem(rowpref, C.nrows, wsum);
+    const int owned = rowpref[C.nrows];
+    if (total > C.cap) {  // the halo does not fit: candidates from global memory
+        for (int p = tid; p < owned; p += blockDim.x) {
+            int lo = 0, hi = C.nrows - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi + 1) >> 1;
+                if (rowpref[mid] <= p) lo = mid;
+                else hi = mid - 1;
+            }
+            xsum_global_far(G, Ph, X, (uint32_t)(rowg[lo] + p - rowpref[lo]), KIND);
+        }
+        return;
+    }
+    for (int h = tid; h < C.nhalo; h += blockDim.x) {
+        const int j0 = lstart[h], j1 = lstart[h + 1];
+        if (j1 == j0) continue;
+        int hk[3];
+        const int key = halo_key(h, hk);
+        const uint32_t g0 = X.sstart[key];
+        float sh[3] = {0.0f, 0.0f, 0.0f};
+        if (shifted) {
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                const int raw = c0[k] - G.R[k] + hk[k];
+                if ((high[k] && raw < G.n[k]) || (low[k] && raw < 0)) sh[k] = G.L[k];
+            }
+        }
+        for (int j = j0; j < j1; ++j) {
+            const uint32_t gi = g0 + (uint32_t)(j - j0);
+            float4 q = X.spos[gi], v = X.svel[gi];
+            const float t = v.w;
+            q.x = sub_rn(q.x, sh[0]);
+            q.y = sub_rn(q.y, sh[1]);
+            q.z = sub_rn(q.z, sh[2]);
+            if (KIND == kIsphAtGas || KIND == kMkAtGas) q.w = approx_div(1.0f, t);
+            if (KIND == kMkAtDust) q.w = approx_div(1.0f, X.srho[gi]);
+            if (KIND == kIsphAtGas || KIND == kIsphAtDust) v.w = approx_div(1.0f, X.srho[gi]);
+            sa[j] = q;
+            sb[j] = v;
+        }
+    }
+    __syncthreads();
+    if (crosses && !shifted)
+        xsum_tile_walk<KIND, true>(G, Ph, C, c0, orig, X, lstart, rowpref, rowg, sa, sb, queue, owned);
+    else
+        xsum_tile_walk<KIND, false>(G, Ph, C, c0, orig, X, lstart, rowpref, rowg, sa, sb, queue, owned);
+}
+
+// Whether the particles have left their lattice: 1 when their places inside
+// their cells, over kSample evenly spaced particles, spread by more than 0.1
+// cells (mean square over the axes; a lattice displaced by up to 0.17 of a
+// spacing has that, one out of step with the cells has 0.29). One CTA.
+constexpr int kSample = 4096;
+__global__ void __launch_bounds__(512) k_scattered(Geo<float> G, const float4 *__restrict__ pos, uint32_t n, int *out)
+{
+    const uint32_t m = min((uint32_t)kSample, n);
+    float s[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
+        const float4 p = pos[(uint32_t)((uint64_t)i * n / m)];
+        const float x[3] = {p.x, p.y, p.z};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float t = (x[k] - G.lo[k]) * G.inv_w[k], f = t - floorf(t);
+            s[k] += f;
+            s[3 + k] += f * f;
+        }
+    }
+    __shared__ float part[16][6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
+        if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][k] = s[k];
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        float var = 0.0f;
+        for (int k = 0; k < 3; ++k) {
+            float a = 0.0f, b = 0.0f;
+            for (int w = 0; w < 16; ++w) {
+                a += part[w][k];
+                b += part[w][3 + k];
+            }
+            var += b / (float)m - (a / (float)m) * (a / (float)m);
+        }
+        *out = var > 3.0f * 0.01f ? 1 : 0;
+    }
+}
+
+// Targets that fill the chip with one thread each (12 CTAs an SM).
+constexpr int64_t kXFill = (int64_t)kSmCount * 12 * kXThreads;
+
+// The sums of one kind. Where the tiled form applies (sources of `mean` per
+// cell, a tile for every SM): alone when a thread per target would not fill
+// the chip (50^3 targets: 69 us against 126-130 us on the lattice, 106 against
+// 208 us off it); beyond, only once the particles have left their lattice.
+// There (884,736 targets displaced by up to 0.35 of a spacing) it takes 613
+// and 653 us against 702 and 898 us for ISPH and 625 against 711-722 us for
+// MK, because the lanes' rows differ in length; on a lattice (0.05) they do
+// not, and a thread per target takes 367-449 us against 426-453. Which runs is
+// decided on the device, where the cell ranges are (both are launched; the
+// other returns at once).
+template <class T, int DIM, int KIND>
+cudaError_t launch_xsum(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, XArgs<T> X, double mean, int *gate)
+{
+    const unsigned blocks = (unsigned)((X.n + kXThreads - 1) / kXThreads);
+    if constexpr (sizeof(T) == 4 && DIM == 3) {
+        TileCfg C{};
+        size_t smem = 0;
+        if (!X.has_frozen && Ph.eos == TFSPH_EOS_ISOTHERMAL &&
+            plan_tiles(G, 3, mean, 32, kXTileSmem - kXQueueBytes, kXTileThreads, C, smem) && C.cap <= 0xFFFF &&
+            (int64_t)C.nt[0] * C.nt[1] * C.nt[2] >= kSmCount) {
+            // (per call: the attribute belongs to the device's copy of the kernel)
+            cudaError_t e = cudaFuncSetAttribute(k_xsum_tile<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXTileSmem);
+            if (e != cudaSuccess) return e;
+            const bool choose = X.n > kXFill;
+            if (choose) {
+                X.gate = gate;
+                X.run_if = 0;
+                k_xsum<T, DIM, KIND><<<blocks, kXThreads, 0, L.stream>>>(G, Ph, X);
+                X.run_if = 1;
+            }
+            k_xsum_tile<KIND><<<(unsigned)(C.nt[0] * C.nt[1] * C.nt[2]), kXTileThreads, smem + kXQueueBytes, L.stream>>>(
+                G, Ph, C, X);
+            return cudaGetLastError();
+        }
+    }
+    k_xsum<T, DIM, KIND><<<blocks, kXThreads, 0, L.stream>>>(G, Ph, X);
+    return cudaGetLastError();
 }
 
 // Per-particle updates. SCHEME: TFSPH_DRAG_ISPH or TFSPH_DRAG_MK.
@@ -267,19 +680,25 @@ cudaError_t xdrag_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     auto *dvel = static_cast<V4<T> *>(Dp.vel[Dp.cur]);
     const T *rg = static_cast<const T *>(rho_g);
     const T *rd = static_cast<const T *>(rho_d);
-    XArgs<T> at_gas{gpos, gvel, Gp.id[Gp.cur], rg, ng, dpos, dvel, Dp.id[Dp.cur], Dp.start, rd, S.has_frozen,
+    XArgs<T> at_gas{gpos, gvel, Gp.id[Gp.cur], rg, ng, dpos, dvel, Dp.id[Dp.cur], Dp.start, Gp.start, rd,
+                    S.has_frozen,
                     static_cast<V4<T> *>(B.g4), nullptr, static_cast<T *>(B.g1)};
-    XArgs<T> at_dust{dpos, dvel, Dp.id[Dp.cur], rd, nd, gpos, gvel, Gp.id[Gp.cur], Gp.start, rg, S.has_frozen,
+    XArgs<T> at_dust{dpos, dvel, Dp.id[Dp.cur], rd, nd, gpos, gvel, Gp.id[Gp.cur], Gp.start, Dp.start, rg,
+                     S.has_frozen,
                      static_cast<V4<T> *>(B.d4), static_cast<V4<T> *>(B.d4b), nullptr};
     const bool isph = scheme == TFSPH_DRAG_ISPH;
-    if (ng > 0) {
-        if (isph) k_xsum<T, DIM, kIsphAtGas><<<blocks_for(ng, kXThreads), kXThreads, 0, L.stream>>>(G, Ph, at_gas);
-        else k_xsum<T, DIM, kMkAtGas><<<blocks_for(ng, kXThreads), kXThreads, 0, L.stream>>>(G, Ph, at_gas);
-    }
-    if (nd > 0) {
-        if (isph) k_xsum<T, DIM, kIsphAtDust><<<blocks_for(nd, kXThreads), kXThreads, 0, L.stream>>>(G, Ph, at_dust);
-        else k_xsum<T, DIM, kMkAtDust><<<blocks_for(nd, kXThreads), kXThreads, 0, L.stream>>>(G, Ph, at_dust);
-    }
+    const double mean_g = (double)ng / (double)G.ncells, mean_d = (double)nd / (double)G.ncells;
+    cudaError_t e = cudaSuccess;
+    if constexpr (sizeof(T) == 4 && DIM == 3)
+        if (std::max(ng, nd) > kXFill)
+            k_scattered<<<1, 512, 0, L.stream>>>(G, ng > 0 ? gpos : dpos, (uint32_t)(ng > 0 ? ng : nd), B.gate);
+    if (ng > 0)
+        e = isph ? launch_xsum<T, DIM, kIsphAtGas>(L, G, Ph, at_gas, mean_d, B.gate)
+                 : launch_xsum<T, DIM, kMkAtGas>(L, G, Ph, at_gas, mean_d, B.gate);
+    if (e == cudaSuccess && nd > 0)
+        e = isph ? launch_xsum<T, DIM, kIsphAtDust>(L, G, Ph, at_dust, mean_g, B.gate)
+                 : launch_xsum<T, DIM, kMkAtDust>(L, G, Ph, at_dust, mean_g, B.gate);
+    if (e != cudaSuccess) return e;
     const T tau = T(S.tau), g0 = T(S.g[0]), g1 = T(S.g[1]), g2 = T(S.g[2]);
     if (ng > 0) {
         if (isph)
