@@ -109,8 +109,9 @@ template <class T, int DIM, int MODE, bool REC, bool SEAMLESS>
 __device__ __forceinline__ void walk_tile(PairAcc<T, MODE> &A, const Geo<T> &G, const Phys<T> &Ph, const TileCfg &C,
                                           const int c0[3], const V4<T> &pa, const V4<T> &pc, const uint16_t *lstart,
                                           const V4<T> *spos, const V4<T> *svel, const T *srho, const uint32_t *sid,
-                                          NbRec *rec)
+                                          NbRec *rec, int sub = 0, int step = 1)
 {
+    // (step > 1, 3D: lane sub of step lanes, which takes every step-th plane)
     // pa: the staged (possibly shifted) position the displacements use;
     // pc: the same position in box coordinates, for its cell and window
     T tx_, ty_ = T(0), tz_ = T(0);
@@ -136,7 +137,7 @@ __device__ __forceinline__ void walk_tile(PairAcc<T, MODE> &A, const Geo<T> &G, 
         oz0 = -min(G.R[2], max(0, floor_int(tz - fz + T(1))));
     }
 #pragma unroll 1
-    for (int oz = oz0; oz <= oz1; ++oz) {
+    for (int oz = oz0 + sub; oz <= oz1; oz += step) {
         T dz2 = T(0);
         int seam_z = 0;
         if (DIM > 2) {
@@ -242,12 +243,13 @@ __device__ __noinline__ void particle_tile(const Geo<T> G, const Phys<T> Ph, con
 // zero (its (2 - q) is clamped) and adds nothing.
 __device__ __forceinline__ void record_walk_f32(const int R[3], const float w[3], const float inv_w[3], float reach2,
                                                 float thr, const TileCfg &C, const int h[3], const float f[3],
-                                                const float4 pf, const uint16_t *lstart, const float4 *sf, NbRec &rec)
+                                                const float4 pf, const uint16_t *lstart, const float4 *sf, NbRec &rec,
+                                                int sub, int step)
 {
     const float tz = approx_sqrt(reach2) * inv_w[2];
     const int oz1 = min(R[2], max(0, floor_int(f[2] + tz))), oz0 = -min(R[2], max(0, floor_int(tz - f[2] + 1.0f)));
 #pragma unroll 1
-    for (int oz = oz0; oz <= oz1; ++oz) {
+    for (int oz = oz0 + sub; oz <= oz1; oz += step) {
         const float sz = slab_dist(oz, f[2]) * w[2], dz2 = sz * sz;
         const float ty = approx_sqrt(fmaxf(reach2 - dz2, 0.0f)) * inv_w[1];
         const int oy1 = min(R[1], max(0, floor_int(f[1] + ty))), oy0 = -min(R[1], max(0, floor_int(ty - f[1] + 1.0f)));
@@ -318,7 +320,10 @@ __device__ __forceinline__ void read_list(PairAcc<T, MODE> &A, const Geo<T> &G, 
     }
 }
 
-template <class T, int DIM, int MODE>
+// SPLIT: C.lanes threads share an owned particle (each takes every lanes-th
+// plane of cells and keeps its own part of the list), for problems whose tiles
+// of a thread per particle would not fill the chip.
+template <class T, int DIM, int MODE, bool SPLIT = false>
 __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? ((MODE == 0 || MODE == 2) ? 4 : 3)
                                                          : (kPrefilter<T, DIM> && (MODE == 0 || MODE == 2) ? 2 : 1))
 k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, const V4<T> *__restrict__ vel,
@@ -533,7 +538,9 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
     const bool tiled = total <= C.cap;
 
 
-    for (int p = tid; p < owned; p += blockDim.x) {
+    const int lanes = SPLIT ? C.lanes : 1;
+    for (int slot = tid; slot < owned * lanes; slot += blockDim.x) {
+        const int p = SPLIT ? slot / lanes : slot, sub = SPLIT ? slot & (lanes - 1) : 0;
         // owned row of p: the last r with rowpref[r] <= p
         int lo = 0, hi = C.nrows - 1;
         while (lo < hi) {
@@ -543,6 +550,7 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
         const int k = p - rowpref[lo];
         const uint32_t a = (uint32_t)(rowg[lo] + k);
         if (!tiled) {
+            if (SPLIT && sub != 0) continue;
             particle_global<T, DIM, MODE>(G, Ph, a, pos, vel, rho, id, start, mass, out_rho, pr_out, out_acc, cnt,
                                           fpr);
             continue;
@@ -560,9 +568,9 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                 if (DIM > 2) pc.z = add_rn(pa.z, orig[2]);
             }
             acc_init(A, Ph, pa, vel, rho, a);
-            const bool listed = nbl.idx && p < nbl.owned_cap;
+            const bool listed = nbl.idx && slot < nbl.owned_cap;
             const size_t oc = (size_t)nbl.owned_cap;
-            const size_t lbase = (size_t)blockIdx.x * (size_t)(nbl.cap / 4 + 1) * oc + (size_t)p;
+            const size_t lbase = (size_t)blockIdx.x * (size_t)(nbl.cap / 4 + 1) * oc + (size_t)slot;
             if (kPre && listed && seamless) {
                 if constexpr (kPre) {
                     NbRec rec{nbl.idx + lbase, (uint32_t)oc, nbl.cap / 4, 0};
@@ -583,36 +591,43 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                     // rounded to 2^-24 far: 2^-19 far covers the displacement
                     const float reach = 2.0f + 0x1p-19f * far;
                     record_walk_f32(G.R, w, iw, reach * reach * (1.0f + 0x1p-18f) + 0x1p-19f * far * reach,
-                                    reach * reach * (1.0f + 0x1p-20f), C, h, f, sf[ja], lstart, sf, rec);
+                                    reach * reach * (1.0f + 0x1p-20f), C, h, f, sf[ja], lstart, sf, rec, sub,
+                                    lanes);
                     const int n = rec.n;
-                    nbl.cnt[(size_t)blockIdx.x * oc + p] = n <= nbl.cap ? (uint16_t)n : kNbNone;
-                    if (n > nbl.cap) {
+                    nbl.cnt[(size_t)blockIdx.x * oc + slot] = n <= nbl.cap ? (uint16_t)n : kNbNone;
+                    if (SPLIT && n > nbl.cap) {
+                        walk_tile<T, DIM, MODE, false, true>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid,
+                                                             nullptr, sub, lanes);
+                    } else if (n > nbl.cap) {
                         particle_tile<T, DIM, MODE, true>(G, Ph, C, c0[0], c0[1], c0[2], pa, pc, a, lstart, spos, vel,
                                                           mass, out_rho, pr_out, out_acc);
                         continue;
+                    } else {
+                        read_list<T, DIM, MODE, true, false>(A, G, Ph, pa, spos, nbl.idx + lbase, oc, n);
                     }
-                    read_list<T, DIM, MODE, true, false>(A, G, Ph, pa, spos, nbl.idx + lbase, oc, n);
                 }
             } else if (MODE == 0 && listed) {
                 // density pass: record the neighbours in walk order
                 NbRec rec{nbl.idx + lbase, (uint32_t)oc, nbl.cap / 4, 0};
                 if (seamless)
-                    walk_tile<T, DIM, MODE, true, true>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, &rec);
+                    walk_tile<T, DIM, MODE, true, true>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, &rec,
+                                                        sub, lanes);
                 else
-                    walk_tile<T, DIM, MODE, true, false>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, &rec);
-                nbl.cnt[(size_t)blockIdx.x * oc + p] = rec.n <= nbl.cap ? (uint16_t)rec.n : kNbNone;
-            } else if (MODE == 2 && listed && nbl.cnt[(size_t)blockIdx.x * oc + p] != kNbNone) {
+                    walk_tile<T, DIM, MODE, true, false>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, &rec,
+                                                         sub, lanes);
+                nbl.cnt[(size_t)blockIdx.x * oc + slot] = rec.n <= nbl.cap ? (uint16_t)rec.n : kNbNone;
+            } else if (MODE == 2 && listed && nbl.cnt[(size_t)blockIdx.x * oc + slot] != kNbNone) {
                 // force pass: the density pass's list of this binning, same order
-                const int n = nbl.cnt[(size_t)blockIdx.x * oc + p];
+                const int n = nbl.cnt[(size_t)blockIdx.x * oc + slot];
                 const unsigned long long *e = nbl.idx + lbase;
                 const size_t st = oc;
                 if (seamless)
                     read_list<T, DIM, MODE, true>(A, G, Ph, pa, spos, e, st, n);
                 else
                     read_list<T, DIM, MODE, false>(A, G, Ph, pa, spos, e, st, n);
-            } else if (MODE == 0) {
+            } else if (MODE == 0 && !SPLIT) {
                 // a particle the density pass does not list (rare): out of line
-                if constexpr (MODE == 0) {
+                if constexpr (MODE == 0 && !SPLIT) {
                     if (seamless)
                         particle_tile<T, DIM, MODE, true>(G, Ph, C, c0[0], c0[1], c0[2], pa, pc, a, lstart, spos, vel,
                                                           mass, out_rho, pr_out, out_acc);
@@ -622,10 +637,26 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                 }
                 continue;
             } else if (seamless) {
-                walk_tile<T, DIM, MODE, false, true>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, nullptr);
+                walk_tile<T, DIM, MODE, false, true>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, nullptr,
+                                                     sub, lanes);
             } else {
-                walk_tile<T, DIM, MODE, false, false>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, nullptr);
+                walk_tile<T, DIM, MODE, false, false>(A, G, Ph, C, c0, pa, pc, lstart, spos, svel, srho, sid, nullptr,
+                                                      sub, lanes);
             }
+        }
+        if constexpr (SPLIT) {
+            // the lanes of a particle lie in one warp and got here together
+            const unsigned mask = ((1u << lanes) - 1u) << ((tid & 31) & ~(lanes - 1));
+            for (int o = lanes >> 1; o > 0; o >>= 1) {
+                if (MODE == 0) {
+                    A.sum += __shfl_xor_sync(mask, A.sum, o);
+                } else {
+                    A.ax += __shfl_xor_sync(mask, A.ax, o);
+                    A.ay += __shfl_xor_sync(mask, A.ay, o);
+                    A.az += __shfl_xor_sync(mask, A.az, o);
+                }
+            }
+            if (sub != 0) continue;
         }
         acc_store(A, Ph, a, mass, vel, out_rho, pr_out, out_acc, cnt, fpr);
     }
@@ -643,6 +674,29 @@ template <class T, int DIM, int MODE> constexpr int tile_bytes_per_particle()
 // Shared memory of the listing passes' tiles (the list belongs to their shape).
 template <class T, int DIM> constexpr int tile_budget() { return kPrefilter<T, DIM> ? kTileSmemWide : kTileSmemPos; }
 
+// Tiles of the listing passes (density and isothermal force). In 3D a problem
+// of few tiles takes smaller ones, with up to eight lanes per particle, until
+// there are two CTAs per SM (binary64: one, which fills its pipe). A 24^3 box:
+// density 56 -> 17 us, force 24 -> 15 us; 16^3: step 254 -> 98 us; 44^3, two
+// lanes: 181 -> 174 us; at 52^3, with 2.5 CTAs per SM, two lanes would lose
+// (211 -> 219 us).
+template <class T>
+bool plan_listing(const Geo<T> &G, int dim, double mean, TileCfg &C, size_t &smem)
+{
+    const int bpp = dim == 3 ? tile_bytes_per_particle<T, 3, 0>() : tile_bytes_per_particle<T, 1, 0>();
+    const int budget = dim == 3 ? tile_budget<T, 3>() : tile_budget<T, 1>();
+    if (!plan_tiles(G, dim, mean, bpp, budget, kTileThreads, C, smem)) return false;
+    const int64_t want = (int64_t)kSmCount * (sizeof(T) == 4 ? 2 : 1);
+    for (int lanes = 2; dim == 3 && lanes <= 8 && (int64_t)C.nt[0] * C.nt[1] * C.nt[2] < want; lanes *= 2) {
+        TileCfg S{};
+        size_t sm = 0;
+        if (!plan_tiles(G, dim, mean, bpp, budget, kTileThreads, S, sm, lanes)) break;
+        C = S;
+        smem = sm;
+    }
+    return true;
+}
+
 template <class T, int DIM, int MODE>
 cudaError_t pair_launch(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, int n, T mass, const V4<T> *pos,
                         const V4<T> *vel, const T *rho, const uint32_t *id, const uint32_t *start, T *out_rho,
@@ -651,21 +705,30 @@ cudaError_t pair_launch(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, 
 {
     constexpr int bpp = tile_bytes_per_particle<T, DIM, MODE>();
     const int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : tile_budget<T, DIM>();
+    constexpr bool kListing = MODE == 0 || MODE == 2;
     TileCfg C{};
     size_t smem = 0;
-    if (plan_tiles(G, DIM, mean, bpp, budget, kTileThreads, C, smem)) {
+    if (kListing ? plan_listing(G, DIM, mean, C, smem)
+                 : plan_tiles(G, DIM, mean, bpp, budget, kTileThreads, C, smem)) {
         static bool attr_set = false;
         if (!attr_set) {
             cudaError_t e = cudaFuncSetAttribute(k_pair_tile<T, DIM, MODE>,
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, budget);
+            if constexpr (kListing && DIM == 3)
+                if (e == cudaSuccess)
+                    e = cudaFuncSetAttribute(k_pair_tile<T, DIM, MODE, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, budget);
             if (e != cudaSuccess) return e;
             attr_set = true;
         }
         const int blocks = C.nt[0] * C.nt[1] * C.nt[2];
         // tile-local indices must fit the list's 15 index bits
         if (C.cap > 0x7FFF) nb = NbList{};
-        k_pair_tile<T, DIM, MODE><<<blocks, kTileThreads, smem, L.stream>>>(G, Ph, C, pos, vel, rho, id, start, mass,
-                                                                            out_rho, pr_out, out_acc, cnt, fpr, nb);
+        auto kern = k_pair_tile<T, DIM, MODE>;
+        if constexpr (kListing && DIM == 3)
+            if (C.lanes > 1) kern = k_pair_tile<T, DIM, MODE, true>;
+        kern<<<blocks, kTileThreads, smem, L.stream>>>(G, Ph, C, pos, vel, rho, id, start, mass, out_rho, pr_out,
+                                                       out_acc, cnt, fpr, nb);
     } else {
         const int threads = 128;
         k_pair_global<T, DIM, MODE><<<(n + threads - 1) / threads, threads, 0, L.stream>>>(
@@ -826,15 +889,16 @@ bool nblist_layout_t(const Geo<T> &G, int dim, int64_t n, int *cap, int *owned_c
     const double mean = (double)n / (double)G.ncells;
     const double want = 1.5 * mean * ball / cellv + 16.0;
     if (want > 1024.0) return false;
-    // the density pass's tiles (MODE 0 plan)
+    // the density pass's tiles
     TileCfg C{};
     size_t smem = 0;
-    const int bpp = dim == 3 ? tile_bytes_per_particle<T, 3, 0>() : tile_bytes_per_particle<T, 1, 0>();
-    const int budget = dim == 3 ? tile_budget<T, 3>() : tile_budget<T, 1>();
-    if (!plan_tiles(G, dim, mean, bpp, budget, kTileThreads, C, smem) || C.cap > 0x7FFF) return false;
-    double owned = mean;
+    if (!plan_listing(G, dim, mean, C, smem) || C.cap > 0x7FFF) return false;
+    // a lane's part of a split particle's neighbours: the planes of cells it
+    // takes, at most about 2/5 of them more than its even share
+    const double part = C.lanes == 1 ? want : (want - 16.0) * std::min(1.0, 1.0 / C.lanes + 0.3) + 16.0;
+    double owned = mean * C.lanes;
     for (int k = 0; k < dim; ++k) owned *= (double)C.T[k];
-    const double cap_d = 32.0 * std::ceil(want / 32.0);
+    const double cap_d = 32.0 * std::ceil(part / 32.0);
     const double oc_d = 32.0 * std::ceil((1.25 * owned + 32.0) / 32.0);
     // cap is a multiple of 32 (so of the 4 entries of a group); a particle's
     // 16-bit slots lie within cap * owned_cap + 4 of its first (32-bit offsets)

@@ -19,6 +19,7 @@ struct TileCfg {
     int nrows;    // T1 T2 owned rows
     int cap;      // particles that fit in shared memory
     int offset;   // byte offset of the particle arrays in shared memory
+    int lanes = 1;  // lanes per owned particle (listing passes of small 3D problems)
     float invH[2];  // 1 / H0, 1 / H1
 };
 
@@ -109,9 +110,10 @@ __device__ __forceinline__ int halo_seam(const Geo<T> &G, int k, int c0, int hc)
 // of the shared-memory capacity (a tile whose halo exceeds it takes the
 // global-memory walk; the 3D box's halos stay within 4 % of their mean).
 // Returns false when an axis wraps fully.
+// lanes > 1: small tiles, of one pass with that many threads per particle.
 template <class T>
 bool plan_tiles(const Geo<T> &G, int dim, double mean, int bytes_pp, int smem_budget, int threads, TileCfg &C,
-                size_t &smem)
+                size_t &smem, int lanes = 1)
 {
     for (int k = 0; k < dim; ++k)
         if (G.full[k]) return false;
@@ -129,10 +131,10 @@ bool plan_tiles(const Geo<T> &G, int dim, double mean, int bytes_pp, int smem_bu
     // one pass over the owned particles (7/8 of the threads) unless the halo
     // outweighs the tile (more than 3 halo cells per owned cell, as in 3D
     // with R = 3), then two nearly full passes to spread it
-    shape(0.875);
+    shape(0.875 / lanes);
     double halo_ratio = 1.0;
     for (int k = 0; k < dim; ++k) halo_ratio *= (double)(Tt[k] + 2 * G.R[k]) / (double)Tt[k];
-    if (halo_ratio > 3.0) shape(1.97);
+    if (halo_ratio > 3.0 && lanes == 1) shape(1.97);
     for (;;) {
         int H[3] = {1, 1, 1};
         long nh = 1;
@@ -164,6 +166,7 @@ bool plan_tiles(const Geo<T> &G, int dim, double mean, int bytes_pp, int smem_bu
             C.invH[1] = 1.0f / (float)H[1];
             C.cap = (int)cap;
             C.offset = (int)offset;
+            C.lanes = lanes;
             smem = (size_t)offset + (size_t)cap * (size_t)bytes_pp;
             return true;
         }
