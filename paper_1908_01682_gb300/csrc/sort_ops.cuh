@@ -104,20 +104,23 @@ __device__ __forceinline__ void rank_move(uint32_t s, const uint32_t *__restrict
         atomicOr(err, kErrInternal);
         return;
     }
+    // the particle's state is loaded with its key, not after the chain of
+    // loads that finds its place
     const uint32_t k = key[i];
+    const V4<T> p = pos[i], v = vel[i];
+    const uint32_t w = id[i], mine = tid[s];
     const uint32_t b = start[k], e = start[k + 1];
     uint32_t d = b;
     if (e - b > 1) {
-        const uint32_t mine = tid[s];
         for (uint32_t t = b; t < e; ++t) d += tid[t] < mine ? 1u : 0u;
     }
     if (d >= e) {
         atomicOr(err, kErrInternal);
         return;
     }
-    opos[d] = pos[i];
-    ovel[d] = vel[i];
-    oid[d] = id[i];
+    opos[d] = p;
+    ovel[d] = v;
+    oid[d] = w;
 }
 
 }  // namespace tfsph
