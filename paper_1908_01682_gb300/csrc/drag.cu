@@ -194,7 +194,102 @@ __device__ __noinline__ int cell_adjoint_wide(const Phys<T> Ph, const StepVals S
                                               *O);
 }
 
-template <class T, class A, int DIM>
+// The same by four consecutive lanes, lane k on component k and lane 3 on the
+// stopping times (df only; a sum over the components is added up at the end,
+// which two-float sums leave far below the rounding of the results). Lane k
+// returns its component in lv, lA, lu; the scalars come back in every lane.
+template <class T, int DIM>
+__device__ __forceinline__ int cell_adjoint_lanes(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
+                                                  const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
+                                                  const V4<T> *__restrict__ acc, const V4<T> *__restrict__ dvel,
+                                                  const V4<T> *__restrict__ lgx, const V4<T> *lgv,
+                                                  const V4<T> *__restrict__ ldx, const V4<T> *ldu, const CellRange &R,
+                                                  unsigned mask, CellLam<T> &O)
+{
+    const int k = threadIdx.x & 3;
+    const bool axis = k < DIM, last = k == 3;
+    const df one = df(1.0f), zero = df(0.0f);
+    const df tau = S.tau;
+    const df g = k == 0 ? S.g[0] : (k == 1 ? S.g[1] : S.g[2]);
+    auto at = [k](const V4<T> *p, uint32_t a) { return reinterpret_cast<const T *>(p + a)[k]; };
+    uint32_t ng = 0;
+    const uint32_t nd = R.de - R.ds;
+    df sv = zero, sa = zero, su = zero;
+#pragma unroll 2
+    for (uint32_t a = R.gs; a < R.ge; ++a) {
+        if (has_frozen && (gid[a] & kFrozenBit)) continue;
+        ++ng;
+        sv += at(gvel, a);
+        sa += at(acc, a);
+    }
+#pragma unroll 2
+    for (uint32_t j = R.ds; j < R.de; ++j) {
+        const T u = at(dvel, j);
+        if (harmonic && last) su += one / df(u);
+        else su += u;
+    }
+    if (ng == 0 || nd == 0) return 0;
+    const df st = lane_value(mask, su, (threadIdx.x & 31) | 3);
+    const df N = df(ng), L = df(nd);
+    const df eps = df(Ph.m_d) * L / (df(Ph.m_g) * N);
+    const df tst = harmonic ? L / st : st / L;
+    const df rt = tau / tst;
+    const df den = one + rt * (one + eps);
+    const df ig = one / (one + rt * eps), id = one / (one + rt);
+    bool fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    df wn = zero, un = zero, vn = zero, S_un = zero, S_vn = zero, S_ig = zero, S_id = zero;
+    if (axis) {
+        wn = ((sv / N - su / L) + tau * (sa / N)) / den;
+        un = su / L + tau * g + rt * wn;
+        vn = un + wn;
+        fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p60f, 0x1p60f) &&
+               df_in(vn, -0x1p60f, 0x1p60f);
+        for (uint32_t a = R.gs; a < R.ge; ++a) {
+            if (has_frozen && (gid[a] & kFrozenBit)) continue;
+            const df l = df(at(lgv, a)) + tau * df(at(lgx, a));
+            S_un += (one - ig) * l;
+            S_ig += (df(at(gvel, a)) + tau * (df(at(acc, a)) + g) - un) * l;
+        }
+        for (uint32_t j = R.ds; j < R.de; ++j) {
+            const df l = df(at(ldu, j)) + tau * df(at(ldx, j));
+            S_vn += (one - id) * l;
+            S_id += (df(at(dvel, j)) + tau * g - vn) * l;
+        }
+    }
+    const df l_un = S_un + S_vn;
+    const df l_wn = S_vn + rt * l_un;
+    const df l_w = l_wn / den;
+    O.lv[0] = T(l_w / N);               // lambda of vbar, per gas particle
+    O.lA[0] = T(tau * l_wn / den / N);  // lambda of Abar, per gas particle
+    O.lu[0] = T((l_un - l_w) / L);      // lambda of ubar, per dust particle
+    fits = fits && !df_small(S_vn) && !df_small(l_un) && !df_small(l_wn) && df_in(l_un, -0x1p60f, 0x1p60f) &&
+           df_in(l_wn, -0x1p60f, 0x1p60f);
+    // over the components (lanes without one hold zeros)
+    df l_rt = wn * l_un, l_den = -(wn * l_wn / den);
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        const int other = (threadIdx.x & 31) ^ o;
+        l_rt += lane_value(mask, l_rt, other);
+        l_den += lane_value(mask, l_den, other);
+        S_ig += lane_value(mask, S_ig, other);
+        S_id += lane_value(mask, S_id, other);
+    }
+    l_rt += (one + eps) * l_den;
+    l_rt -= eps * ig * ig * S_ig;
+    l_rt -= id * id * S_id;
+    const df lt = -(rt / tst) * l_rt;
+    fits = fits && !df_small(S_ig) && !df_small(S_id) && !df_small(l_rt) && df_in(l_rt, -0x1p60f, 0x1p60f) &&
+           df_in(lt, -0x1p100f, 0x1p100f);
+    O.lt = T(lt);  // lambda of t*
+    O.ig = T(ig);
+    O.id = T(id);
+    O.tst = T(tst);
+    O.L = T(L);
+    return __all_sync(mask, fits) ? 1 : 2;
+}
+
+// LANES: as in the cell update (4 with df only).
+template <class T, class A, int DIM, int LANES>
 __global__ void __launch_bounds__(kCellsPerCta)
 k_cell_adjoint(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen,
                const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid, const uint32_t *__restrict__ gstart,
@@ -207,40 +302,54 @@ k_cell_adjoint(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen,
     __shared__ int s_drag[kCellsPerCta];
 
     const uint32_t ncells = G.ncells;
-    const uint32_t c0 = blockIdx.x * kCellsPerCta;
-    const uint32_t c = c0 + threadIdx.x;
+    const uint32_t cpc = kCellsPerCta / LANES;
+    const uint32_t c0 = blockIdx.x * cpc;
+    const uint32_t lc0 = threadIdx.x / LANES;
+    const uint32_t c = c0 + lc0;
     int drag = 0;
     if (c < ncells) {
         const CellRange R{gstart[c], gstart[c + 1], dstart[c], dstart[c + 1]};
         CellLam<T> O;
-        drag = cell_adjoint_solve<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu, R,
-                                             O);
+        const int k = threadIdx.x & 3;
+        bool all = LANES == 1;  // this thread holds every component
+        if constexpr (LANES == 1)
+            drag = cell_adjoint_solve<T, A, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu,
+                                                 R, O);
+        else
+            drag = cell_adjoint_lanes<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu, R,
+                                              0xfu << (threadIdx.x & 28), O);
         if constexpr (std::is_same<A, df>::value) {
-            if (drag == 2) {
+            if (drag == 2 && (LANES == 1 || k == 0)) {
                 CellLam<T> W;
-                drag = cell_adjoint_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu,
-                                                 R, &W);
+                cell_adjoint_wide<T, DIM>(Ph, S, harmonic, has_frozen, gvel, gid, acc, dvel, lgx, lgv, ldx, ldu, R, &W);
                 O = W;
+                all = true;
             }
         }
-        if (drag) {
+        if (drag && all) {
 #pragma unroll
-            for (int k = 0; k < DIM; ++k) {
-                s_lv[k][threadIdx.x] = O.lv[k];
-                s_lA[k][threadIdx.x] = O.lA[k];
-                s_lu[k][threadIdx.x] = O.lu[k];
+            for (int m = 0; m < DIM; ++m) {
+                s_lv[m][lc0] = O.lv[m];
+                s_lA[m][lc0] = O.lA[m];
+                s_lu[m][lc0] = O.lu[m];
             }
-            s_lt[threadIdx.x] = O.lt;
-            s_ig[threadIdx.x] = O.ig;
-            s_id[threadIdx.x] = O.id;
-            s_tst[threadIdx.x] = O.tst;
-            s_L[threadIdx.x] = O.L;
+        } else if (drag == 1 && k < DIM) {
+            s_lv[k][lc0] = O.lv[0];
+            s_lA[k][lc0] = O.lA[0];
+            s_lu[k][lc0] = O.lu[0];
+        }
+        if (drag && (LANES == 1 || k == 0)) {
+            s_lt[lc0] = O.lt;
+            s_ig[lc0] = O.ig;
+            s_id[lc0] = O.id;
+            s_tst[lc0] = O.tst;
+            s_L[lc0] = O.L;
         }
     }
-    s_drag[threadIdx.x] = drag;
+    if (LANES == 1 || (threadIdx.x & 3) == 0) s_drag[lc0] = drag;
     __syncthreads();
 
-    const uint32_t c1 = min(c0 + (uint32_t)kCellsPerCta, ncells);
+    const uint32_t c1 = min(c0 + cpc, ncells);
     const T tau_t = step_val<T>(S.tau, S.dtau);
     for (uint32_t a = gstart[c0] + threadIdx.x; a < gstart[c1]; a += blockDim.x) {
         V4<T> la;
@@ -255,7 +364,7 @@ k_cell_adjoint(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen,
         lv.y += tau_t * lx.y;
         lv.z += tau_t * lx.z;
         const uint32_t lc = cell_key<T, DIM>(G, p.x, p.y, p.z) - c0;
-        if (lc < (uint32_t)kCellsPerCta && s_drag[lc]) {
+        if (lc < cpc && s_drag[lc]) {
             const T ig = s_ig[lc];
             la.x = tau_t * ig * lv.x + s_lA[0][lc];
             lv.x = ig * lv.x + s_lv[0][lc];
@@ -277,7 +386,7 @@ k_cell_adjoint(Geo<T> G, Phys<T> Ph, StepVals S, int harmonic, int has_frozen,
         lu.y += tau_t * lx.y;
         lu.z += tau_t * lx.z;
         const uint32_t lc = cell_key<T, DIM>(G, p.x, p.y, p.z) - c0;
-        if (lc < (uint32_t)kCellsPerCta && s_drag[lc]) {
+        if (lc < cpc && s_drag[lc]) {
             const T id = s_id[lc];
             lu.x = id * lu.x + s_lu[0][lc];
             if (DIM > 1) lu.y = id * lu.y + s_lu[1][lc];
@@ -299,8 +408,17 @@ cudaError_t cell_adjoint_t(const LaunchCtx &L, const void *geo, const void *phys
 {
     const Geo<T> &Gg = *static_cast<const Geo<T> *>(geo);
     const Phys<T> &Ph = *static_cast<const Phys<T> *>(phys);
-    const uint32_t blocks = (Gg.ncells + kCellsPerCta - 1) / kCellsPerCta;
-    k_cell_adjoint<T, A, DIM><<<blocks, kCellsPerCta, 0, L.stream>>>(
+    // four lanes per cell where cells hold several particles (see the update):
+    // 512^2 column 62 -> 44 us
+    bool lanes = false;
+    auto kern = k_cell_adjoint<T, A, DIM, 1>;
+    if constexpr (std::is_same<A, df>::value) {
+        lanes = (double)std::max(G.n, D.n) >= 1.5 * (double)Gg.ncells;
+        if (lanes) kern = k_cell_adjoint<T, A, DIM, 4>;
+    }
+    const uint32_t cpc = kCellsPerCta / (lanes ? 4 : 1);
+    const uint32_t blocks = (Gg.ncells + cpc - 1) / cpc;
+    kern<<<blocks, kCellsPerCta, 0, L.stream>>>(
         Gg, Ph, step_vals(S.tau, S.g), S.tstar_mode == TFSPH_TSTAR_HARMONIC, S.has_frozen,
         static_cast<const V4<T> *>(G.vel[G.cur]), G.id[G.cur], G.start, static_cast<const V4<T> *>(acc),
         static_cast<const V4<T> *>(G.pos[G.cur]), static_cast<const V4<T> *>(D.vel[D.cur]),
