@@ -772,11 +772,16 @@ struct SnapHeader {
 };
 constexpr uint64_t kSnapMagic = 0x3254535048504654ull;
 
-__global__ void k_check_snapshot(const SnapHeader *h, int64_t ng, int64_t nd, int dim, int precision,
+// Reads the header in words: a snapshot buffer need only be 4-byte aligned.
+__global__ void k_check_snapshot(const uint32_t *words, int64_t ng, int64_t nd, int dim, int precision,
                                  uint32_t ncells, int *err)
 {
-    if (h->magic != kSnapMagic || h->n_gas != ng || h->n_dust != nd || h->dim != dim || h->precision != precision ||
-        h->ncells != ncells)
+    uint32_t w[sizeof(SnapHeader) / 4];
+    for (int k = 0; k < (int)(sizeof(SnapHeader) / 4); ++k) w[k] = words[k];
+    SnapHeader h;
+    memcpy(&h, w, sizeof h);
+    if (h.magic != kSnapMagic || h.n_gas != ng || h.n_dust != nd || h.dim != dim || h.precision != precision ||
+        h.ncells != ncells)
         atomicOr(err, kErrInternal);
 }
 
@@ -945,10 +950,11 @@ int tfsph_load_state(tfsph_ctx *c, const void *buf, int mem_kind)
     SnapHeader h{};
     const char *src = static_cast<const char *>(buf);
     if (mem_kind == TFSPH_MEM_DEVICE) {
+        if (reinterpret_cast<uintptr_t>(buf) % 4 != 0) return fail(c, TFSPH_E_INVALID_ARG, "buf must be 4-byte aligned");
         // checked on the device, without a host round trip; a mismatch is
         // reported by the next tfsph_sync (the copies below use this
         // context's sizes, so they stay in bounds either way)
-        k_check_snapshot<<<1, 1, 0, c->stream>>>(reinterpret_cast<const SnapHeader *>(src), c->G.n, c->D.n, c->dim,
+        k_check_snapshot<<<1, 1, 0, c->stream>>>(reinterpret_cast<const uint32_t *>(src), c->G.n, c->D.n, c->dim,
                                                  c->precision, c->ncells, c->d_err);
         TF_CUDA(c, cudaGetLastError());
         c->launches += 1;
@@ -961,7 +967,6 @@ int tfsph_load_state(tfsph_ctx *c, const void *buf, int mem_kind)
     }
     src += sizeof h;
     if (mem_kind == TFSPH_MEM_DEVICE) {
-        if (reinterpret_cast<uintptr_t>(buf) % 4 != 0) return fail(c, TFSPH_E_INVALID_ARG, "buf must be 4-byte aligned");
         CopyList L{};
         for (const SnapPart &q : snap_parts(c)) {
             if (q.bytes) L.add(src, q.ptr, q.bytes);
