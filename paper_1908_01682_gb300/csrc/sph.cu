@@ -749,9 +749,11 @@ cudaError_t density_t(const LaunchCtx &L, const void *geo, const void *phys, Pha
     T *pr = gas ? reinterpret_cast<T *>(pos) : nullptr;
     const T mass = gas ? Ph.m_g : Ph.m_d;
     const double mean = (double)P.n / (double)G.ncells;
+    // the neighbour statistics are an export: p/rho^2 of the state stays the
+    // density pass's (whose sums may be split over lanes and round otherwise)
     if (cnt)
         return pair_launch<T, DIM, 1>(L, G, Ph, (int)P.n, mass, pos, vel, nullptr, P.id[P.cur], P.start,
-                                      static_cast<T *>(rho), pr, nullptr, cnt, fprint, mean);
+                                      static_cast<T *>(rho), nullptr, nullptr, cnt, fprint, mean);
     return pair_launch<T, DIM, 0>(L, G, Ph, (int)P.n, mass, pos, vel, nullptr, P.id[P.cur], P.start,
                                   static_cast<T *>(rho), pr, nullptr, nullptr, nullptr, mean,
                                   (gas && nbl) ? *nbl : NbList{});
