@@ -14,7 +14,7 @@ namespace tfsph {
 
 // Distance, in cell units, from a particle at fractional cell position f to
 // the slab of the cell o cells away along one axis (0 for its own cell).
-template <class T> __device__ __forceinline__ T slab_dist(int o, T f)
+template <class T> __host__ __device__ __forceinline__ T slab_dist(int o, T f)
 {
     if (o > 0) return fmax(T(0), T(o) - f);
     if (o < 0) return fmax(T(0), f + T(-o) - T(1));

@@ -20,6 +20,7 @@
 #include <cmath>
 
 #include "pair.cuh"
+#include "prefilter.cuh"
 #include "tile.cuh"
 
 namespace tfsph {
@@ -233,42 +234,27 @@ __device__ __noinline__ void particle_tile(const Geo<T> G, const Phys<T> Ph, con
     acc_store(A, Ph, a, mass, vel, out_rho, pr_out, out_acc, nullptr, nullptr);
 }
 
-// The recording walk of a binary64 particle in 3D (seamless tiles): rows and
-// candidates are taken in binary32 from a copy of the staged positions
-// relative to the tile, in units of h (sf; pf the particle's own), so that the binary64 pipe,
-// at 2 lanes per SM and clock the bound of these sums, only sees the listed
-// pairs. thr and reach2 carry margins over 4h^2 and the pruning radius that
-// cover the rounding of the relative coordinates, of the cell fractions f and
-// of the arithmetic here; a pair between 4h^2 and thr lies where the kernel is
-// zero (its (2 - q) is clamped) and adds nothing.
-__device__ __forceinline__ void record_walk_f32(const int R[3], const float w[3], const float inv_w[3], float reach2,
-                                                float thr, const TileCfg &C, const int h[3], const float f[3],
-                                                const float4 pf, const uint16_t *lstart, const float4 *sf, NbRec &rec,
-                                                int sub, int step)
+// The recording walk of a binary64 particle in 3D (seamless tiles whose staged
+// particles all lie within the prefilter's range): rows and candidates are
+// taken in binary32 from a copy of the staged positions relative to the tile
+// (sf; pf the particle's own), so that the binary64 pipe, at 2 lanes per SM
+// and clock the bound of these sums, only sees the listed pairs. The margins
+// over 4h^2 and the pruning radius cover the rounding of the relative
+// coordinates, of the cell fractions f and of the arithmetic; a pair between
+// 4h^2 and thr lies where the kernel is zero (its (2 - q) is clamped) and adds
+// nothing.
+__device__ __forceinline__ void record_walk_f32(const int R[3], const Prefilter &P, const TileCfg &C, const int h[3],
+                                                const float f[3], const float4 pf, const uint16_t *lstart,
+                                                const float4 *sf, NbRec &rec, int sub, int step)
 {
-    const float tz = approx_sqrt(reach2) * inv_w[2];
-    const int oz1 = min(R[2], max(0, floor_int(f[2] + tz))), oz0 = -min(R[2], max(0, floor_int(tz - f[2] + 1.0f)));
+    prefilter_rows(P, R, C.H, h, f, sub, step, [&](int u0, int u1) {
+        const int j1 = lstart[u1];
 #pragma unroll 1
-    for (int oz = oz0 + sub; oz <= oz1; oz += step) {
-        const float sz = slab_dist(oz, f[2]) * w[2], dz2 = sz * sz;
-        const float ty = approx_sqrt(fmaxf(reach2 - dz2, 0.0f)) * inv_w[1];
-        const int oy1 = min(R[1], max(0, floor_int(f[1] + ty))), oy0 = -min(R[1], max(0, floor_int(ty - f[1] + 1.0f)));
-#pragma unroll 1
-        for (int oy = oy0; oy <= oy1; ++oy) {
-            const float sy = slab_dist(oy, f[1]) * w[1];
-            const float tx = approx_sqrt(fmaxf(reach2 - dz2 - sy * sy, 0.0f)) * inv_w[0];
-            const int ohi = min(R[0], max(0, floor_int(f[0] + tx)));
-            const int olo = -min(R[0], max(0, floor_int(tx - f[0] + 1.0f)));
-            const int hrow = C.H[0] * ((h[1] + oy) + C.H[1] * (h[2] + oz)) + h[0];
-            const int j1 = lstart[hrow + ohi + 1];
-#pragma unroll 1
-            for (int j = lstart[hrow + olo]; j < j1; ++j) {
-                const float4 q = sf[j];
-                const float dx = pf.x - q.x, dy = pf.y - q.y, dz = pf.z - q.z;
-                if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < thr) rec.push(j, false);
-            }
+        for (int j = lstart[u0]; j < j1; ++j) {
+            const float4 q = sf[j];
+            if (prefilter_near(P, pf.x - q.x, pf.y - q.y, pf.z - q.z)) rec.push(j, false);
         }
-    }
+    });
 }
 
 // Pair sums over a particle's recorded list (groups `e[g * st]` of four
@@ -401,9 +387,21 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
 #pragma unroll
         for (int k = 0; k < DIM; ++k) org[k] = G.lo[k] + T(c0[k]) * G.w[k] - orig[k];
     }
+    // whether the tile has staged a particle beyond the prefilter's range (this thread's, then the CTA's)
+    bool beyond = false;
+    Prefilter pre{};
+    if constexpr (kPre) pre = prefilter_of(G, C);
     auto copy32 = [&](int j, const V4<T> &q) {
-        if constexpr (kPre) sf[j] = make_float4((float)((q.x - org[0]) * G.inv_h), (float)((q.y - org[1]) * G.inv_h),
-                                (float)((q.z - org[2]) * G.inv_h), 0.0f);
+        if constexpr (kPre) {
+            const float4 s = make_float4((float)((q.x - org[0]) * G.inv_h), (float)((q.y - org[1]) * G.inv_h),
+                                         (float)((q.z - org[2]) * G.inv_h), 0.0f);
+            beyond = beyond || !prefilter_holds(pre, s.x, s.y, s.z);
+            sf[j] = s;
+        }
+    };
+    auto staged = [&] {
+        if constexpr (kPre) beyond = __syncthreads_or(beyond);
+        else __syncthreads();
     };
 
     // owned rows: global start and particle count
@@ -475,7 +473,7 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                 }
             }
         }
-        __syncthreads();
+        staged();
     } else {
         // halo cell counts; a ragged tile needs only ext + 2R halo cells per axis,
         // which keeps every raw coordinate within (-n, 2n) so one wrap suffices
@@ -531,7 +529,7 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                     if (MODE == 1) sid[j] = id[gi];
                 }
             }
-            __syncthreads();
+            staged();
         }
     }
     const int owned = rowpref[C.nrows];
@@ -571,7 +569,7 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
             const bool listed = nbl.idx && slot < nbl.owned_cap;
             const size_t oc = (size_t)nbl.owned_cap;
             const size_t lbase = (size_t)blockIdx.x * (size_t)(nbl.cap / 4 + 1) * oc + (size_t)slot;
-            if (kPre && listed && seamless) {
+            if (kPre && listed && seamless && !beyond) {
                 if constexpr (kPre) {
                     NbRec rec{nbl.idx + lbase, (uint32_t)oc, nbl.cap / 4, 0};
                     const int ja = lstart[hrow + G.R[0]] + k;
@@ -579,20 +577,10 @@ k_pair_tile(Geo<T> G, Phys<T> Ph, TileCfg C, const V4<T> *__restrict__ pos, cons
                     const int h[3] = {axis_cell(pc.x, G.lo[0], G.inv_w[0], G.n[0], t[0]) - c0[0] + G.R[0],
                                       axis_cell(pc.y, G.lo[1], G.inv_w[1], G.n[1], t[1]) - c0[1] + G.R[1],
                                       axis_cell(pc.z, G.lo[2], G.inv_w[2], G.n[2], t[2]) - c0[2] + G.R[2]};
-                    float f[3], w[3], iw[3], far = 0.0f;
+                    float f[3];
 #pragma unroll
-                    for (int d = 0; d < 3; ++d) {
-                        f[d] = (float)(t[d] - T(h[d] + c0[d] - G.R[d]));
-                        w[d] = (float)(G.w[d] * G.inv_h);
-                        iw[d] = (float)(G.inv_w[d] * G.h);
-                        far = fmaxf(far, (float)C.H[d] * w[d]);
-                    }
-                    // in units of h; relative coordinates are below `far`, each
-                    // rounded to 2^-24 far: 2^-19 far covers the displacement
-                    const float reach = 2.0f + 0x1p-19f * far;
-                    record_walk_f32(G.R, w, iw, reach * reach * (1.0f + 0x1p-18f) + 0x1p-19f * far * reach,
-                                    reach * reach * (1.0f + 0x1p-20f), C, h, f, sf[ja], lstart, sf, rec, sub,
-                                    lanes);
+                    for (int d = 0; d < 3; ++d) f[d] = (float)(t[d] - T(h[d] + c0[d] - G.R[d]));
+                    record_walk_f32(G.R, pre, C, h, f, sf[ja], lstart, sf, rec, sub, lanes);
                     const int n = rec.n;
                     nbl.cnt[(size_t)blockIdx.x * oc + slot] = n <= nbl.cap ? (uint16_t)n : kNbNone;
                     if (SPLIT && n > nbl.cap) {
