@@ -242,7 +242,13 @@ void make_geo_phys(const tfsph_params &p, const int ncell[3], uint32_t ncells, G
         const int n = ncell[d];
         const double w = L / (double)n;
         G.n[d] = n;
-        G.R[d] = (int)floor(reach / w) + 1;
+        // The walks look floor(f + t) cells up and floor(t - f + 1) down, with t
+        // the pruning radius in cells as they round it and f the fraction of
+        // the rounded cell estimate. Where that is one cell off the particle's
+        // own cell, f lies within the estimate's error of the face and both
+        // must stay below R: R counts the radius with that error and the
+        // rounding of t on top.
+        G.R[d] = (int)floor((reach + 8.0 * u * span) / w * (1.0 + 32.0 * u)) + 1;
         G.per[d] = p.periodic[d] ? 1 : 0;
         G.full[d] = (G.per[d] && 2 * G.R[d] + 1 >= n) ? 1 : 0;
         G.lo[d] = T(p.lo[d]);
