@@ -30,12 +30,14 @@ __global__ void k_keys(Geo<T> G, const V4<T> *__restrict__ pos, int n, uint32_t 
 }
 
 // AGG: the warp's atomics on one counter are combined (cells holding several
-// particles of a phase).
+// particles of a phase). counted: see launch_bin.
 template <bool AGG>
 __global__ void k_count(const uint32_t *__restrict__ kg, int ng, uint32_t *__restrict__ cg,
-                        const uint32_t *__restrict__ kd, int nd, uint32_t *__restrict__ cd)
+                        const uint32_t *__restrict__ kd, int nd, uint32_t *__restrict__ cd,
+                        const int *__restrict__ counted)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (counted && *counted) return;
     if (i >= ng + nd) return;
     uint32_t *c = i < ng ? &cg[kg[i]] : &cd[kd[i - ng]];
     if (AGG) count_add_agg(c);
@@ -129,6 +131,7 @@ k_scan_down(const uint32_t *__restrict__ cg, const uint32_t *__restrict__ cd, ui
 {
     const uint32_t *cnt = blockIdx.y == 0 ? cg : cd;
     uint32_t *st = blockIdx.y == 0 ? sg : sd;
+    const uint32_t n = blockIdx.y == 0 ? ng : nd;
     const uint32_t base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
     load_items(cnt, base, ncells, v);
@@ -141,7 +144,7 @@ k_scan_down(const uint32_t *__restrict__ cg, const uint32_t *__restrict__ cd, ui
     uint32_t o[kScanItems];
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        o[k] = run;
+        o[k] = min(run, n);  // (past n: counts of a step that gave up)
         run += v[k];
     }
     if (base + kScanItems <= ncells) {
@@ -153,7 +156,7 @@ k_scan_down(const uint32_t *__restrict__ cg, const uint32_t *__restrict__ cd, ui
         for (int k = 0; k < kScanItems; ++k)
             if (base + k < ncells) st[base + k] = o[k];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) st[ncells] = blockIdx.y == 0 ? ng : nd;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st[ncells] = n;
 }
 
 template <bool AGG>
@@ -184,9 +187,10 @@ __global__ void k_rank_gather(const uint32_t *__restrict__ kg, const uint32_t *_
                               const uint32_t *__restrict__ tidd, const V4<T> *__restrict__ pd,
                               const V4<T> *__restrict__ vd, const uint32_t *__restrict__ id_,
                               V4<T> *__restrict__ opd, V4<T> *__restrict__ ovd, uint32_t *__restrict__ oid, int nd,
-                              int *err)
+                              int *err, int *__restrict__ counted)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s == 0 && counted) *counted = 0;  // the scatter has taken the counts
     if (s < ng) rank_move<T>((uint32_t)s, kg, sg, srcg, tidg, pg, vg, ig, opg, ovg, oig, (uint32_t)ng, err);
     else if (s < ng + nd)
         rank_move<T>((uint32_t)(s - ng), kd, sd, srcd, tidd, pd, vd, id_, opd, ovd, oid, (uint32_t)nd, err);
@@ -453,7 +457,7 @@ cudaError_t keys_t(const LaunchCtx &L, const void *geo, const PhaseBufs &P)
 
 template <class T>
 cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D, uint32_t *bsum, int64_t nblk,
-                  bool counted)
+                  int *counted)
 {
     const Geo<T> &Gm = *static_cast<const Geo<T> *>(geo);
     const int ng = (int)G.n, nd = (int)D.n;
@@ -461,9 +465,9 @@ cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &
     const uint32_t ncells = Gm.ncells;
     // combined atomics pay when a phase has on average more than one particle per cell
     const bool agg = (double)std::max(ng, nd) >= 1.5 * (double)ncells;
-    if (ntot > 0 && !counted) {
-        if (agg) k_count<true><<<grid_for(ntot, 256), 256, 0, L.stream>>>(G.key, ng, G.count, D.key, nd, D.count);
-        else k_count<false><<<grid_for(ntot, 256), 256, 0, L.stream>>>(G.key, ng, G.count, D.key, nd, D.count);
+    if (ntot > 0) {
+        auto count = agg ? k_count<true> : k_count<false>;
+        count<<<grid_for(ntot, 256), 256, 0, L.stream>>>(G.key, ng, G.count, D.key, nd, D.count, counted);
     }
     if (L.ev) cudaEventRecord(L.ev[1], L.stream);
     dim3 sg((unsigned)nblk, 2);
@@ -484,7 +488,8 @@ cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &
             static_cast<const V4<T> *>(G.vel[G.cur]), G.id[G.cur], static_cast<V4<T> *>(G.pos[og]),
             static_cast<V4<T> *>(G.vel[og]), G.id[og], ng, D.key, D.start, D.tmp_src, D.tmp_id,
             static_cast<const V4<T> *>(D.pos[D.cur]), static_cast<const V4<T> *>(D.vel[D.cur]), D.id[D.cur],
-            static_cast<V4<T> *>(D.pos[od]), static_cast<V4<T> *>(D.vel[od]), D.id[od], nd, L.d_err);
+            static_cast<V4<T> *>(D.pos[od]), static_cast<V4<T> *>(D.vel[od]), D.id[od], nd, L.d_err,
+            counted);
         G.cur = og;
         D.cur = od;
     } else if (L.ev) {
@@ -575,7 +580,7 @@ cudaError_t launch_keys(const LaunchCtx &L, const void *geo, const PhaseBufs &P)
 }
 
 cudaError_t launch_bin(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D, uint32_t *bsum,
-                       int64_t nblk, bool counted)
+                       int64_t nblk, int *counted)
 {
     return L.precision == TFSPH_FP64 ? bin_t<double>(L, geo, G, D, bsum, nblk, counted)
                                      : bin_t<float>(L, geo, G, D, bsum, nblk, counted);

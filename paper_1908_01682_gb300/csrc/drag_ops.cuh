@@ -343,8 +343,8 @@ __device__ __forceinline__ void dust_particle_update(const Geo<T> &G, T tau_t, c
 
 // The cells [c0, c0 + cpc) and their particles, by one CTA (see drag.cu):
 // phase 1 with LANES threads per cell, then the particle updates and the next
-// cell keys; the dust loop starts at thread dust_tid. With COUNT and gcnt the
-// next keys are counted too (gcnt, dcnt: all zero before). The caller syncs before it
+// cell keys; the dust loop starts at thread dust_tid. With COUNT the next keys
+// are counted too (gcnt, dcnt: all zero before). The caller syncs before it
 // reuses the shared arrays.
 template <class T> struct CellShared {
     T us[3][kCellsPerCta], vs[3][kCellsPerCta], ig[kCellsPerCta], id[kCellsPerCta];
@@ -441,7 +441,7 @@ cell_update_cta(CellShared<T> &s, const Geo<T> &G, const Phys<T> &Ph, const Step
             if (has_frozen && (gid[a] & kFrozenBit)) {
                 const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
                 gkey[a] = key;
-                if (COUNT && gcnt) atomicAdd(&gcnt[key], 1u);
+                if (COUNT) atomicAdd(&gcnt[key], 1u);
                 continue;
             }
             V4<T> v = gvel[a];
@@ -460,7 +460,7 @@ cell_update_cta(CellShared<T> &s, const Geo<T> &G, const Phys<T> &Ph, const Step
             gvel[a] = v;
             const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
             gkey[a] = key;
-            if (COUNT && gcnt) atomicAdd(&gcnt[key], 1u);
+            if (COUNT) atomicAdd(&gcnt[key], 1u);
         }
     }
     {
@@ -482,7 +482,7 @@ cell_update_cta(CellShared<T> &s, const Geo<T> &G, const Phys<T> &Ph, const Step
             dvel[j] = u;
             const uint32_t key = cell_key<T, DIM, EST>(G, p.x, p.y, p.z);
             dkey[j] = key;
-            if (COUNT && gcnt) atomicAdd(&dcnt[key], 1u);
+            if (COUNT) atomicAdd(&dcnt[key], 1u);
         }
     }
 }

@@ -44,8 +44,7 @@ template <class T> struct SmallArgs {
     uint32_t ng, nd;
     int lanes;    // lanes per particle of the pair sums (1, or up to 8: binary64 in 1D)
     uint32_t cpc; // cells a CTA updates at a time
-    int count;    // count the next keys in the update
-    int counted;  // gcnt, dcnt hold the counts of the current keys (the last step left them)
+    int *counted; // nonzero: gcnt, dcnt hold the counts of the current keys (the last step left them)
     int cluster;  // the grid is one cluster
     int harmonic, has_frozen, adiabatic;
 };
@@ -105,7 +104,7 @@ template <class T> __device__ __forceinline__ void small_scan(const SmallArgs<T>
         uint32_t run = before + e;
 #pragma unroll
         for (int k = 0; k < kScanItems; ++k) {
-            if (base + k < nc) st[base + k] = run;
+            if (base + k < nc) st[base + k] = min(run, dust ? B.nd : B.ng);  // (past n: a step that gave up)
             run += v[k];
         }
         if (first == 0 && threadIdx.x == 0) st[nc] = dust ? B.nd : B.ng;
@@ -261,7 +260,12 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const SmallArgs
     const uint32_t rank = blockIdx.x * blockDim.x + threadIdx.x, count = gridDim.x * blockDim.x;
     const uint32_t n = B.ng + B.nd;
 
-    if (!B.counted) {
+    // a step behind one whose barrier gave up does nothing (it finds its
+    // counts and its barrier half done)
+    const int err = *reinterpret_cast<volatile int *>(B.err);
+    const int counted = *reinterpret_cast<volatile int *>(B.counted);
+    if (err & kErrTimeout) return;
+    if (!counted) {
         for (uint32_t i = rank; i < n; i += count)
             count_add_agg(i < B.ng ? &B.gcnt[B.gkey[i]] : &B.dcnt[B.dkey[i - B.ng]]);
         if (!barrier()) return;
@@ -285,6 +289,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const SmallArgs
     if (!barrier()) return;
     small_pairs<T, DIM, FMODE>(B);
     if (!barrier()) return;
+    if (rank == 0) *B.counted = 1;
     for (uint32_t c0 = blockIdx.x * B.cpc; c0 < B.G.ncells; c0 += gridDim.x * B.cpc) {
         // the dust starts half a CTA away from the gas, so that a CTA with
         // few particles updates both at once
@@ -292,15 +297,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const SmallArgs
         const uint32_t dust_tid = threadIdx.x < half ? threadIdx.x + half : threadIdx.x - half;
         // binary64: one lane per cell unless the CTA has only a few cells
         // (four lanes repeat the scalar part of the solve)
-        uint32_t *gcnt = B.count ? B.gcnt : nullptr, *dcnt = B.count ? B.dcnt : nullptr;
         if (sizeof(T) == 4 || B.cpc <= 16)
             cell_update_cta<T, A, DIM, false, 4, true>(cs, B.G, B.Ph, B.S, B.harmonic, B.has_frozen, B.adiabatic, c0,
                                                        B.cpc, dust_tid, B.gpb, B.gvb, B.gib, B.gkey, B.gstart, B.acc,
-                                                       B.dpb, B.dvb, B.dkey, B.dstart, gcnt, dcnt);
+                                                       B.dpb, B.dvb, B.dkey, B.dstart, B.gcnt, B.dcnt);
         else
             cell_update_cta<T, A, DIM, false, 1, true>(cs, B.G, B.Ph, B.S, B.harmonic, B.has_frozen, B.adiabatic, c0,
                                                        B.cpc, dust_tid, B.gpb, B.gvb, B.gib, B.gkey, B.gstart, B.acc,
-                                                       B.dpb, B.dvb, B.dkey, B.dstart, gcnt, dcnt);
+                                                       B.dpb, B.dvb, B.dkey, B.dstart, B.gcnt, B.dcnt);
         __syncthreads();
     }
 }
@@ -321,8 +325,7 @@ void *pick(int precision, int cell_acc, int dim, bool full)
 
 template <class T>
 cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D, void *rho,
-                    void *acc, const StepArgs &S, const SmallPlan &P, GridBar *bar, bool counted,
-                    bool count)
+                    void *acc, const StepArgs &S, const SmallPlan &P, GridBar *bar, int *counted)
 {
     SmallArgs<T> B{};
     B.G = *static_cast<const Geo<T> *>(geo);
@@ -360,7 +363,6 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.nd = (uint32_t)D.n;
     B.lanes = P.lanes;
     B.counted = counted;
-    B.count = count;
     B.cluster = P.cluster;
     // cells shared out evenly over the CTAs, at most what four lanes each allow
     B.cpc = std::min((uint32_t)P.threads / 4, std::max(1u, (B.G.ncells + (uint32_t)P.grid - 1) / (uint32_t)P.grid));
@@ -427,12 +429,11 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
 }
 
 cudaError_t launch_step_small(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
-                              void *rho, void *acc, const StepArgs &S, const SmallPlan &P, void *bar, bool counted,
-                              bool count)
+                              void *rho, void *acc, const StepArgs &S, const SmallPlan &P, void *bar, int *counted)
 {
     GridBar *b = static_cast<GridBar *>(bar);
-    return L.precision == TFSPH_FP64 ? small_t<double>(L, geo, phys, G, D, rho, acc, S, P, b, counted, count)
-                                     : small_t<float>(L, geo, phys, G, D, rho, acc, S, P, b, counted, count);
+    return L.precision == TFSPH_FP64 ? small_t<double>(L, geo, phys, G, D, rho, acc, S, P, b, counted)
+                                     : small_t<float>(L, geo, phys, G, D, rho, acc, S, P, b, counted);
 }
 
 }  // namespace tfsph

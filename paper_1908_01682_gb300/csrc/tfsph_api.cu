@@ -56,7 +56,13 @@ struct tfsph_ctx {
     bool prepared = false;      // binning and density of the current state are done
     bool forced = false;        // ... and acc holds its pressure acceleration
     bool counts_dirty = false;  // a binning did not finish: zero the cell counts first
-    bool counted = false;       // the cell counts are those of the current keys (else zero)
+    // Both phases' cell counts and, behind them, the word that tells whether
+    // they are those of the current keys (a one-launch step leaves them) or
+    // zero. Both change in stream order only, with the keys they belong to, so
+    // that graphs of steps can be captured and replayed between other calls.
+    void *counts = nullptr;
+    size_t counts_bytes = 0;
+    int *counted = nullptr;     // that word (NULL: no one-launch step, the counts stay zero)
     bool has_frozen = false;
     int64_t steps = 0;
     int64_t device_bytes = 0;
@@ -210,6 +216,9 @@ int stage_inputs(tfsph_ctx *c, const void *const *arrs, int narr, int64_t n, con
     return TFSPH_OK;
 }
 
+// Zeroes both phases' cell counts, which then belong to no keys.
+cudaError_t clear_counts(tfsph_ctx *c) { return cudaMemsetAsync(c->counts, 0, c->counts_bytes, c->stream); }
+
 // Loads a full particle state, computes keys and checks it (synchronises).
 int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, const uint8_t *frozen, int mem_kind)
 {
@@ -228,6 +237,7 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     c->G.cur = 0;
     c->D.cur = 0;
     PhaseBufs G = c->G;
+    if (c->counted) TF_CUDA(c, clear_counts(c));  // counts of the keys that are replaced
     if (staged) {
         // the staging area is reused for dust only after the gas is packed
         PhaseBufs no_dust = c->D;
@@ -257,8 +267,6 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
         }
     }
     c->has_frozen = any_frozen;
-    c->counts_dirty = c->counts_dirty || c->counted;  // counts of the replaced keys
-    c->counted = false;
     c->prepared = false;
     c->forced = false;
     c->nbl_valid = false;
@@ -300,32 +308,6 @@ int next_events(tfsph_ctx *c, cudaEvent_t **out)
     return TFSPH_OK;
 }
 
-// Whether the context's stream is being captured into a graph. Only contexts
-// of the one-launch step ask: a captured step leaves no counts for the next
-// one, so that a graph of steps can be replayed.
-bool capturing(const tfsph_ctx *c)
-{
-    if (!c->small.fn) return false;
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->stream, &st) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return st != cudaStreamCaptureStatusNone;
-}
-
-// Zeroes the cell counts after a binning that did not finish, or where a
-// capture meets counts left by the step before it.
-int clear_counts(tfsph_ctx *c, bool cap)
-{
-    if (c->counts_dirty || (cap && c->counted)) {
-        TF_CUDA(c, cudaMemsetAsync(c->G.count, 0, (size_t)c->ncells * 4, c->stream));
-        TF_CUDA(c, cudaMemsetAsync(c->D.count, 0, (size_t)c->ncells * 4, c->stream));
-        c->counted = false;
-    }
-    return TFSPH_OK;
-}
-
 int prepare(tfsph_ctx *c, cudaEvent_t *ev = nullptr)
 {
     if (c->prepared) {
@@ -335,13 +317,11 @@ int prepare(tfsph_ctx *c, cudaEvent_t *ev = nullptr)
     }
     LaunchCtx L = lctx(c);
     L.ev = ev;
-    const bool cap = capturing(c);
-    if (int rc = clear_counts(c, cap)) return rc;
+    if (c->counts_dirty) TF_CUDA(c, clear_counts(c));
     c->counts_dirty = true;
     TF_CUDA(c, launch_bin(L, c->geo, c->G, c->D, c->bsum, c->nblk, c->counted));
-    c->counts_dirty = cap;  // the memset of a capture has not run yet
-    c->launches += (c->G.n + c->D.n > 0) ? (c->counted ? 5 : 6) : 3;
-    c->counted = false;
+    c->counts_dirty = false;
+    c->launches += (c->G.n + c->D.n > 0) ? 6 : 3;
     TF_CUDA(c, launch_density(L, c->geo, c->phys, c->G, c->rho_g, true, nullptr, nullptr,
                               c->nbl.idx ? &c->nbl : nullptr));
     c->nbl_valid = c->nbl.idx != nullptr;
@@ -473,11 +453,16 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
         P->tmp_src = static_cast<uint32_t *>(tmp);
         if ((rc = dalloc(c, &tmp, n * 4))) return bail(rc);
         P->tmp_id = static_cast<uint32_t *>(tmp);
-        if ((rc = dalloc(c, &tmp, (size_t)c->ncells * 4))) return bail(rc);
-        P->count = static_cast<uint32_t *>(tmp);
         if ((rc = dalloc(c, &tmp, ((size_t)c->ncells + 1) * 4))) return bail(rc);
         P->start = static_cast<uint32_t *>(tmp);
-        e = cudaMemset(P->count, 0, (size_t)c->ncells * 4);
+    }
+    {
+        const size_t one = ((size_t)c->ncells * 4 + 15) / 16 * 16;  // (the scans read 16-byte words)
+        c->counts_bytes = 2 * one + 16;
+        if ((rc = dalloc(c, &c->counts, c->counts_bytes))) return bail(rc);
+        c->G.count = static_cast<uint32_t *>(c->counts);
+        c->D.count = c->G.count + one / 4;
+        e = cudaMemset(c->counts, 0, c->counts_bytes);
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
     }
     if ((rc = dalloc(c, &c->rho_g, (size_t)n_gas * c->tsize))) return bail(rc);
@@ -522,6 +507,7 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
     if (p->drag == TFSPH_DRAG_IDIC)
         small_plan(c->geo, c->phys, c->precision, c->cell_acc, c->dim, n_gas, n_dust, &c->small);
+    if (c->small.fn) c->counted = reinterpret_cast<int *>(static_cast<char *>(c->counts) + c->counts_bytes - 16);
     c->bar = c->d_err + 8;  // in the error word's block
     // staging for host I/O: the larger phase's input arrays (+ frozen flags), or a field export
     const int64_t nmax = std::max<int64_t>(n_gas, n_dust);
@@ -599,13 +585,10 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
     // a small context steps in one launch, unless its phases are being timed
     // or a field export or snapshot has already done the first of them
     if (c->small.fn && !ev && !c->prepared) {
-        const bool cap = capturing(c);
-        if ((rc = clear_counts(c, cap))) return rc;
+        if (c->counts_dirty) TF_CUDA(c, clear_counts(c));
         c->counts_dirty = true;
-        TF_CUDA(c, launch_step_small(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->acc, S, c->small, c->bar, c->counted,
-                                     !cap));
-        c->counts_dirty = cap;
-        c->counted = !cap;
+        TF_CUDA(c, launch_step_small(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->acc, S, c->small, c->bar, c->counted));
+        c->counts_dirty = false;
         c->launches += 1;
         c->forced = false;
         c->nbl_valid = false;
@@ -987,8 +970,9 @@ int tfsph_load_state(tfsph_ctx *c, const void *buf, int mem_kind)
     c->prepared = true;
     c->forced = true;
     c->nbl_valid = false;  // the neighbour list is not part of a snapshot
-    c->counts_dirty = true;
-    c->counted = false;
+    // (the counts in step with the stream: a one-launch step may have left some)
+    if (c->counted) TF_CUDA(c, clear_counts(c));
+    else c->counts_dirty = true;
     if (h.steps >= 0) c->steps = h.steps;
     return TFSPH_OK;
 }
@@ -1163,8 +1147,8 @@ int tfsph_sync(tfsph_ctx *c)
         TF_CUDA(c, cudaMemset(c->d_err, 0, sizeof(int)));
         if (err & kErrTimeout) {
             // the barrier and the counts were left as the wait found them
-            TF_CUDA(c, cudaMemset(c->bar, 0, 32));
-            c->counts_dirty = true;
+            TF_CUDA(c, cudaMemsetAsync(c->bar, 0, 32, c->stream));
+            TF_CUDA(c, clear_counts(c));
             return fail(c, TFSPH_E_TIMEOUT, "a grid barrier of the one-launch step waited too long");
         }
         if (err & kErrBadTstop) return fail(c, TFSPH_E_NONFINITE, "a t_stop value was <= 0 or not finite");

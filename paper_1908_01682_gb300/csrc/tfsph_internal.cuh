@@ -159,9 +159,11 @@ struct LaunchCtx {
 
 // bin.cu
 cudaError_t launch_keys(const LaunchCtx &L, const void *geo, const PhaseBufs &P);
-// counted: the cell counts of the current keys are there already.
+// counted (or NULL): a device word, nonzero where the step before has left the
+// counts of the current keys; zero afterwards, as the counts then are. It lies
+// on the device because a replayed graph of steps changes it without the host.
 cudaError_t launch_bin(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &D,
-                       uint32_t *bsum, int64_t nblk, bool counted);
+                       uint32_t *bsum, int64_t nblk, int *counted);
 cudaError_t launch_pack(const LaunchCtx &L, PhaseBufs &P, const void *const *src, int ncomp_v,
                         const uint8_t *frozen, bool is_gas);
 cudaError_t launch_unpack(const LaunchCtx &L, const PhaseBufs &P, int what, void *out, int order,
@@ -302,8 +304,7 @@ cudaError_t launch_cell_update(const LaunchCtx &L, const void *geo, const void *
 // small.cu: the whole IDIC step of a small context in one cooperative launch.
 // small_plan decides once per context whether it takes it (up to
 // kSmallParticles particles of both phases and kSmallCells cells). counted:
-// the cell counts are those of the current keys; count: leave those of the
-// next keys.
+// the word of launch_bin; the step leaves the counts of the next keys and 1.
 constexpr int64_t kSmallParticles = 65536;
 constexpr uint32_t kSmallCells = 32768;
 struct SmallPlan {
@@ -314,7 +315,7 @@ struct SmallPlan {
 bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, int dim, int64_t ng, int64_t nd,
                 SmallPlan *P);
 cudaError_t launch_step_small(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
-                              void *rho, void *acc, const StepArgs &S, const SmallPlan &P, void *bar, bool counted, bool count);
+                              void *rho, void *acc, const StepArgs &S, const SmallPlan &P, void *bar, int *counted);
 
 // xdrag.cu: the ISPH or MK drag and particle update (scheme TFSPH_DRAG_ISPH |
 // TFSPH_DRAG_MK) after binning, gas and dust densities and the gas pressure
