@@ -63,6 +63,7 @@ struct tfsph_ctx {
     void *counts = nullptr;
     size_t counts_bytes = 0;
     int *counted = nullptr;     // that word (NULL: no one-launch step, the counts stay zero)
+    bool flags_dirty = false;   // d_flags may be nonzero
     bool has_frozen = false;
     int64_t steps = 0;
     int64_t device_bytes = 0;
@@ -231,13 +232,33 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     std::vector<const void *> gv, dv;
     const uint8_t *dfz = nullptr, *none = nullptr;
     const int gas_w = c->p.eos == TFSPH_EOS_ADIABATIC;
+    for (int k = 0; k < ndust_arr && c->D.n > 0; ++k)
+        if (!dust[k]) return fail(c, TFSPH_E_INVALID_ARG, "NULL input array");
     bool staged = false;
     int rc = stage_inputs(c, gas, ngas_arr, c->G.n, frozen, mem_kind, gv, &dfz, &staged);
     if (rc) return rc;
+    // from here on the state is replaced, whether its check accepts it or not:
+    // nothing of the one before it may be taken for its own
     c->G.cur = 0;
     c->D.cur = 0;
+    c->prepared = false;
+    c->forced = false;
+    c->nbl_valid = false;
+    bool any_frozen = false;
+    if (frozen && c->G.n > 0) {
+        if (mem_kind == TFSPH_MEM_HOST) {
+            const uint8_t *f = frozen;
+            for (int64_t i = 0; i < c->G.n && !any_frozen; ++i) any_frozen = f[i] != 0;
+        } else {
+            any_frozen = true;  // device flags: assume present (only costs an id read per particle)
+        }
+    }
+    c->has_frozen = any_frozen;
     PhaseBufs G = c->G;
-    if (c->counted) TF_CUDA(c, clear_counts(c));  // counts of the keys that are replaced
+    if (c->counted) TF_CUDA(c, clear_counts(c));
+    // the flags are zero between loads, unless one failed before they were read
+    if (c->flags_dirty) TF_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
+    c->flags_dirty = true;
     if (staged) {
         // the staging area is reused for dust only after the gas is packed
         PhaseBufs no_dust = c->D;
@@ -252,24 +273,10 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     int flags = 0;
     TF_CUDA(c, cudaMemcpyAsync(&flags, c->d_flags, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     TF_CUDA(c, cudaStreamSynchronize(c->stream));
-    // the flags are zero between loads
-    if (flags) TF_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
+    c->flags_dirty = flags != 0;
     if (flags & 1) return fail(c, TFSPH_E_NONFINITE, "non-finite position, velocity or energy in the input");
     if (flags & 4) return fail(c, TFSPH_E_NONFINITE, "dust t_stop must be finite and > 0");
     if (flags & 2) return fail(c, TFSPH_E_OUT_OF_DOMAIN, "a moving particle lies outside [lo, hi)");
-    bool any_frozen = false;
-    if (frozen && c->G.n > 0) {
-        if (mem_kind == TFSPH_MEM_HOST) {
-            const uint8_t *f = frozen;
-            for (int64_t i = 0; i < c->G.n && !any_frozen; ++i) any_frozen = f[i] != 0;
-        } else {
-            any_frozen = true;  // device flags: assume present (only costs an id read per particle)
-        }
-    }
-    c->has_frozen = any_frozen;
-    c->prepared = false;
-    c->forced = false;
-    c->nbl_valid = false;
     c->steps = 0;
     return TFSPH_OK;
 }
