@@ -326,11 +326,12 @@ __device__ __forceinline__ void x_window(const Geo<T> &G, T fx, T rem, int &olo,
 // A neighbour's term apart from its addition, without a branch on membership
 // (zero for candidates outside, which leaves the sums as they are), for walks
 // that evaluate several candidates at once and add them in order. MODE 0: the
-// kernel value; MODE 2: the factor s of the displacement. With add_term the
-// same sums as add(), bit for bit.
+// kernel value; MODE 2: the factor s of the displacement, which is zeroed with
+// it (a candidate that is no number would turn 0 d into one). With add_term
+// the same sums as add(), bit for bit.
 template <class T, int DIM, int MODE>
 __device__ __forceinline__ T pair_term(const PairAcc<T, MODE> &A, const Geo<T> &G, const Phys<T> &Ph, const V4<T> &pb,
-                                       T r2, const T d[3], bool in)
+                                       T r2, T d[3], bool in)
 {
     static_assert(MODE == 0 || MODE == 2, "density and isothermal force");
     if (MODE == 0) {
@@ -341,6 +342,8 @@ __device__ __forceinline__ T pair_term(const PairAcc<T, MODE> &A, const Geo<T> &
     const T q = r2 * inv_r * G.inv_h;
     const T a = positive_part(T(2) - q);
     const T g = below_one(q) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
+#pragma unroll
+    for (int k = 0; k < DIM; ++k) d[k] = in ? d[k] : T(0);
     return in ? (A.qa + pb.w) * g : T(0);
 }
 template <class T, int DIM, int MODE>
