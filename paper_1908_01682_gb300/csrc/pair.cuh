@@ -189,9 +189,9 @@ template <class T, int MODE> struct PairAcc {
             const T a = positive_part(T(2) - q);
             const T g = below_one(q) ? T(-3) + T(2.25) * q : (a * a) * (Ph.hm075 * inv_r);
             const T s = (qa + pb.w) * g;
-            ax -= s * d[0];
-            ay -= s * d[1];
-            az -= s * d[2];
+            ax = fma_rn(-s, d[0], ax);
+            ay = fma_rn(-s, d[1], ay);
+            az = fma_rn(-s, d[2], az);
         } else {
             if (!(r2 >= pair_r2_min<T>())) return;  // self or coincident particle: zero gradient
             const T inv_r = pair_inv_dist<T, DIM>(r2, d);
@@ -352,9 +352,9 @@ __device__ __forceinline__ void add_term(PairAcc<T, MODE> &A, T s, const T d[3])
     if (MODE == 0) {
         A.sum += s;
     } else {
-        A.ax -= s * d[0];
-        if (DIM > 1) A.ay -= s * d[1];
-        if (DIM > 2) A.az -= s * d[2];
+        A.ax = fma_rn(-s, d[0], A.ax);
+        if (DIM > 1) A.ay = fma_rn(-s, d[1], A.ay);
+        if (DIM > 2) A.az = fma_rn(-s, d[2], A.az);
     }
 }
 
