@@ -194,27 +194,32 @@ template <class T, int MODE> struct PairAcc {
             az = fma_rn(-s, d[2], az);
         } else {
             if (!(r2 >= pair_r2_min<T>())) return;  // self or coincident particle: zero gradient
+            // every rounding explicit: the kernels this is compiled into (tiled,
+            // one-launch, batch) would else contract its products differently
             const T inv_r = pair_inv_dist<T, DIM>(r2, d);
-            const T F = kernel_f(G, r2 * inv_r * G.inv_h, G.h * inv_r);  // (1/r) dW/dr
-            T coef = qa + pb.w;
+            const T q = mul_rn(mul_rn(r2, inv_r), G.inv_h), a = positive_part(sub_rn(T(2), q));
+            // (1/r) dW/dr, as kernel_f
+            const T F = mul_rn(G.fnorm, below_one(q) ? fma_rn(T(2.25), q, T(-3))
+                                                     : mul_rn(mul_rn(mul_rn(T(-0.75), a), a), mul_rn(G.h, inv_r)));
+            T coef = add_rn(qa, pb.w);
             if (MODE == 3) {
-                const T vx = va.x - vb->x, vy = va.y - vb->y, vz = va.z - vb->z;
-                const T vr = vx * d[0] + vy * d[1] + vz * d[2];
+                const T vx = sub_rn(va.x, vb->x), vy = sub_rn(va.y, vb->y), vz = sub_rn(va.z, vb->z);
+                const T vr = fma_rn(vz, d[2], fma_rn(vx, d[0], mul_rn(vy, d[1])));
                 T pi = T(0);
                 if (Ph.av && vr < T(0)) {
-                    const T mu = approx_div(Ph.h * vr, r2 + Ph.eta2);
+                    const T mu = approx_div(mul_rn(Ph.h, vr), add_rn(r2, Ph.eta2));
                     const T cb = Ph.eos == TFSPH_EOS_ADIABATIC ? approx_sqrt(Ph.gamma * Ph.gm1 * vb->w) : Ph.cs;
-                    const T cbar = T(0.5) * (ca + cb);
-                    const T rbar = T(0.5) * (rhoa + rhob);
-                    pi = approx_div(-Ph.av_alpha * cbar * mu + Ph.av_beta * mu * mu, rbar);
+                    const T cbar = mul_rn(T(0.5), add_rn(ca, cb));
+                    const T rbar = mul_rn(T(0.5), add_rn(rhoa, rhob));
+                    pi = approx_div(fma_rn(mul_rn(-Ph.av_alpha, cbar), mu, mul_rn(mul_rn(Ph.av_beta, mu), mu)), rbar);
                 }
-                coef += pi;
-                de += (qa + T(0.5) * pi) * vr * F;
+                coef = add_rn(coef, pi);
+                de = fma_rn(mul_rn(fma_rn(T(0.5), pi, qa), vr), F, de);
             }
-            const T s = coef * F;
-            ax -= s * d[0];
-            ay -= s * d[1];
-            az -= s * d[2];
+            const T s = mul_rn(coef, F);
+            ax = fma_rn(-s, d[0], ax);
+            ay = fma_rn(-s, d[1], ay);
+            az = fma_rn(-s, d[2], az);
         }
     }
 };

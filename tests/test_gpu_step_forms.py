@@ -1,0 +1,61 @@
+"""The step rounds alike whatever came before it: after a density export, with
+its phases timed, or as it is (one launch for small contexts, one per phase
+otherwise). States are equal bit for bit: adiabatic and viscous gases."""
+import numpy as np
+import pytest
+
+import workloads
+from conftest import gpu_context, gpu_lib
+
+pytestmark = pytest.mark.gpu
+
+
+def _states(b, w, steps=3):
+    out = []
+    for form in ("plain", "export", "phases"):
+        with gpu_context(w) as c:
+            c.profile(form == "phases")
+            for _ in range(steps):
+                if form == "export":
+                    c.field(b.TFSPH_FIELD_RHO_G)
+                c.step(w.tau, w.g)
+            c.sync()
+            fields = [b.TFSPH_FIELD_POS_G, b.TFSPH_FIELD_VEL_G, b.TFSPH_FIELD_POS_D, b.TFSPH_FIELD_VEL_D,
+                      b.TFSPH_FIELD_RHO_G] + ([b.TFSPH_FIELD_ENERGY_G] if w.params["eos"] == 1 else [])
+            out.append([c.field(f) for f in fields])
+    return out
+
+
+def _same(out):
+    for other in out[1:]:
+        for a, r in zip(out[0], other):
+            assert np.array_equal(a, r)
+
+
+def _stir(w, speed, seed=1):
+    rng = np.random.default_rng(seed)
+    w.gv += speed * rng.standard_normal(w.gv.shape) * (1 if w.frozen is None else w.frozen == 0)
+    w.du += speed * rng.standard_normal(w.du.shape)
+    dt = np.float64 if w.params["precision"] else np.float32
+    w.gv, w.du = w.gv.astype(dt).astype(np.float64), w.du.astype(dt).astype(np.float64)
+    return w
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("case", ["shock", "shock_large", "viscous_wave", "viscous_column", "adiabatic_box"])
+def test_viscous_and_energy_terms(case, prec):
+    b = gpu_lib()
+    if case.startswith("shock"):
+        big = case == "shock_large"
+        w = workloads.dustyshock(n_left=17000 if big else 803, n_right=2125 if big else 100, precision=prec)
+    elif case == "viscous_wave":
+        w = workloads.dustywave(n=1000, precision=prec, amp=1e-2)
+        w.params.update(av_alpha=1.0, av_beta=2.0)
+    elif case == "viscous_column":
+        w = workloads.column2d(nside=40, precision=prec)
+        w.params.update(av_alpha=1.0, av_beta=2.0)
+    else:
+        w = workloads.box3d(nside=12, precision=prec, jitter=0.2)
+        w.params.update(av_alpha=1.0, av_beta=2.0, eos=1)
+        w.ge = np.linspace(1.0, 2.0, w.n_gas).astype(np.float32).astype(np.float64)
+    _same(_states(b, _stir(w, 0.05)))
