@@ -366,13 +366,14 @@ __device__ __forceinline__ void add_term(PairAcc<T, MODE> &A, T s, const T d[3])
 // Calls f(b, n, seam) for every contiguous storage range [b, b + n) of cells
 // that may hold neighbours of a particle at (px, py, pz): per row of cells
 // (fixed y, z), the part of its x window wrapped below 0, the part wrapped
-// above n - 1, then the main part (TILE_ORDER: the main part before the one
-// wrapped above, the order of the tiled walks). seam is true when the range lies across a
+// above n - 1, then the main part (tile_order: the main part before the one
+// wrapped above, the order of the tiled walks, so that a sum rounds alike
+// whichever walk takes it). seam is true when the range lies across a
 // periodic seam from the particle, so its displacements need the periodic
 // image; within the particle's own image the plain difference is exact.
-template <class T, int DIM, bool TILE_ORDER = false, class F>
+template <class T, int DIM, class F>
 __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *__restrict__ start,
-                                               T px, T py, T pz, F &&f)
+                                               T px, T py, T pz, F &&f, bool tile_order = false)
 {
     T tx, ty = T(0), tz = T(0);
     const int cx = axis_cell(px, G.lo[0], G.inv_w[0], G.n[0], tx);
@@ -453,7 +454,7 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                 int olo, ohi;
                 x_window<T, DIM>(G, fx, G.lim2 - dz2 - dy2, olo, ohi);
                 int x0 = cx + olo, x1 = cx + ohi;
-                uint32_t hb = 0, hn = 0;  // the part wrapped above, kept for last in TILE_ORDER
+                uint32_t hb = 0, hn = 0;  // the part wrapped above, kept for last in tile_order
                 if (G.per[0]) {
                     if (x0 < 0) {
                         const uint32_t b = start[row + x0 + nx];
@@ -463,7 +464,7 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                     if (x1 >= nx) {
                         hb = start[row];
                         hn = start[row + (x1 - nx) + 1] - hb;
-                        if (!TILE_ORDER) f(hb, hn, true);
+                        if (!tile_order) f(hb, hn, true);
                         x1 = nx - 1;
                     }
                 } else {
@@ -472,7 +473,7 @@ __device__ __forceinline__ void for_each_range(const Geo<T> &G, const uint32_t *
                 }
                 const uint32_t b = start[row + x0];
                 f(b, start[row + x1 + 1] - b, row_seam);
-                if (TILE_ORDER && hn) f(hb, hn, true);
+                if (tile_order && hn) f(hb, hn, true);
             }
         }
     }
@@ -482,7 +483,8 @@ template <class T, int DIM, int MODE>
 __device__ __forceinline__ void walk_global(PairAcc<T, MODE> &A, const Geo<T> &G, const Phys<T> &Ph,
                                             const V4<T> &pa, const V4<T> *__restrict__ pos,
                                             const V4<T> *__restrict__ vel, const T *__restrict__ rho,
-                                            const uint32_t *__restrict__ id, const uint32_t *__restrict__ start)
+                                            const uint32_t *__restrict__ id, const uint32_t *__restrict__ start,
+                                            bool tile_order = false)
 {
     auto range = [&](uint32_t b0, uint32_t n, auto seam) {
         for (uint32_t b = b0; b < b0 + n; ++b) {
@@ -501,7 +503,7 @@ __device__ __forceinline__ void walk_global(PairAcc<T, MODE> &A, const Geo<T> &G
     for_each_range<T, DIM>(G, start, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {
         if (seam) range(b0, n, SeamTag<true>{});
         else range(b0, n, SeamTag<false>{});
-    });
+    }, tile_order);
 }
 
 }  // namespace tfsph

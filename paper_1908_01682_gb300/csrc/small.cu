@@ -8,8 +8,8 @@
 // one launch, separated by barriers (of a cluster for the smallest, else of
 // the grid, with bounded waits), and every phase is spread over all CTAs: consecutive warps of particles go to
 // different SMs. The phases compute what the kernels of bin.cu, sph.cu and
-// drag.cu compute, with the sums in the tiled walks' order: the results are the
-// same bit for bit. 1D and 2D only: in 3D the lanes of a warp would read their
+// drag.cu compute, with the sums in their order: the results are the same bit
+// for bit. 1D and 2D only: in 3D the lanes of a warp would read their
 // candidates from 32 places of global memory at a time (a 24^3 box: density
 // 50 us against 55 us of its few tiles).
 #include <algorithm>
@@ -46,6 +46,7 @@ template <class T> struct SmallArgs {
     uint32_t cpc; // cells a CTA updates at a time
     int *counted; // nonzero: gcnt, dcnt hold the counts of the current keys (the last step left them)
     int cluster;  // the grid is one cluster
+    int order[2]; // density, force: the sums in the order of the tiled walks (gas_sums_tiled)
     int harmonic, has_frozen, adiabatic;
 };
 
@@ -157,10 +158,10 @@ template <class T, int DIM, int MODE> __device__ __forceinline__ void small_pair
                 A.template add<DIM>(B.G, B.Ph, pb, &vb, rhob, 0u, r2, d);
             }
         };
-        for_each_range<T, DIM, true>(B.G, B.gstart, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {
+        for_each_range<T, DIM>(B.G, B.gstart, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {
             if (seam) range(b0, n, SeamTag<true>{});
             else range(b0, n, SeamTag<false>{});
-        });
+        }, B.order[MODE != 0]);
         if (MODE == 0)
             acc_store<T, MODE>(A, B.Ph, a, B.Ph.m_g, vel, B.rho, reinterpret_cast<T *>(B.gpb), nullptr, nullptr,
                                nullptr);
@@ -190,7 +191,7 @@ template <class T, int MODE> __device__ __forceinline__ void small_pair_lanes(co
         uint32_t rb[3] = {0, 0, 0}, rn[3] = {0, 0, 0}, seams = 0;
         int nr = 0;
         if (live)
-            for_each_range<T, 1, true>(B.G, B.gstart, pa.x, T(0), T(0), [&](uint32_t b0, uint32_t n, bool seam) {
+            for_each_range<T, 1>(B.G, B.gstart, pa.x, T(0), T(0), [&](uint32_t b0, uint32_t n, bool seam) {
 #pragma unroll
                 for (int k = 0; k < 3; ++k)
                     if (nr == k) {
@@ -199,7 +200,7 @@ template <class T, int MODE> __device__ __forceinline__ void small_pair_lanes(co
                     }
                 seams |= (seam ? 1u : 0u) << nr;
                 ++nr;
-            });
+            }, B.order[MODE != 0]);
         const uint32_t m = rn[0] + rn[1] + rn[2];
         const uint32_t most = __reduce_max_sync(0xffffffffu, m);
         for (uint32_t c0 = 0; c0 < most; c0 += (uint32_t)lanes) {
@@ -364,6 +365,8 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.lanes = P.lanes;
     B.counted = counted;
     B.cluster = P.cluster;
+    B.order[0] = P.density_tiles;
+    B.order[1] = P.force_tiles;
     // cells shared out evenly over the CTAs, at most what four lanes each allow
     B.cpc = std::min((uint32_t)P.threads / 4, std::max(1u, (B.G.ncells + (uint32_t)P.grid - 1) / (uint32_t)P.grid));
     B.harmonic = S.tstar_mode == TFSPH_TSTAR_HARMONIC;
@@ -405,7 +408,10 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     const int av = f64 ? static_cast<const Phys<double> *>(phys)->av : static_cast<const Phys<float> *>(phys)->av;
     const int eos = f64 ? static_cast<const Phys<double> *>(phys)->eos : static_cast<const Phys<float> *>(phys)->eos;
     if (dim > 2 || ng <= 0 || nd <= 0 || ng + nd > kSmallParticles || ncells > kSmallCells) return false;
-    P->fn = pick(precision, cell_acc, dim, av || eos == TFSPH_EOS_ADIABATIC);
+    const bool full = av || eos == TFSPH_EOS_ADIABATIC;
+    P->fn = pick(precision, cell_acc, dim, full);
+    P->density_tiles = gas_sums_tiled(geo, precision, dim, ng, 0);
+    P->force_tiles = gas_sums_tiled(geo, precision, dim, ng, full ? 3 : 2);
     int dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||

@@ -211,7 +211,7 @@ __device__ __noinline__ void particle_global(const Geo<T> G, const Phys<T> Ph, u
     PairAcc<T, MODE> A;
     const V4<T> pa = pos[a];
     acc_init(A, Ph, pa, vel, rho, a);
-    walk_global<T, DIM, MODE>(A, G, Ph, pa, pos, vel, rho, id, start);
+    walk_global<T, DIM, MODE>(A, G, Ph, pa, pos, vel, rho, id, start, true);
     acc_store(A, Ph, a, mass, vel, out_rho, pr_out, out_acc, cnt, fpr);
 }
 
@@ -685,19 +685,25 @@ bool plan_listing(const Geo<T> &G, int dim, double mean, TileCfg &C, size_t &sme
     return true;
 }
 
+// Tiles of any pair pass (false: none, each particle walks global memory).
+template <class T, int DIM, int MODE> bool plan_pass(const Geo<T> &G, double mean, TileCfg &C, size_t &smem)
+{
+    if constexpr (MODE == 0 || MODE == 2) return plan_listing(G, DIM, mean, C, smem);
+    constexpr int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : tile_budget<T, DIM>();
+    return plan_tiles(G, DIM, mean, tile_bytes_per_particle<T, DIM, MODE>(), budget, kTileThreads, C, smem);
+}
+
 template <class T, int DIM, int MODE>
 cudaError_t pair_launch(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, int n, T mass, const V4<T> *pos,
                         const V4<T> *vel, const T *rho, const uint32_t *id, const uint32_t *start, T *out_rho,
                         T *pr_out, V4<T> *out_acc, int32_t *cnt, uint64_t *fpr, double mean,
                         NbList nb = NbList{})
 {
-    constexpr int bpp = tile_bytes_per_particle<T, DIM, MODE>();
-    const int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : tile_budget<T, DIM>();
+    constexpr int budget = (ModeUses<MODE>::vel || ModeUses<MODE>::rho) ? 72 * 1024 : tile_budget<T, DIM>();
     constexpr bool kListing = MODE == 0 || MODE == 2;
     TileCfg C{};
     size_t smem = 0;
-    if (kListing ? plan_listing(G, DIM, mean, C, smem)
-                 : plan_tiles(G, DIM, mean, bpp, budget, kTileThreads, C, smem)) {
+    if (plan_pass<T, DIM, MODE>(G, mean, C, smem)) {
         static bool attr_set = false;
         if (!attr_set) {
             cudaError_t e = cudaFuncSetAttribute(k_pair_tile<T, DIM, MODE>,
@@ -899,6 +905,26 @@ bool nblist_layout_t(const Geo<T> &G, int dim, int64_t n, int *cap, int *owned_c
     return true;
 }
 }  // namespace
+
+namespace {
+template <class T, int DIM> bool gas_sums_tiled_t(const void *geo, int64_t n, int mode)
+{
+    const Geo<T> &G = *static_cast<const Geo<T> *>(geo);
+    const double mean = (double)n / (double)G.ncells;
+    TileCfg C{};
+    size_t smem = 0;
+    return mode == 3 ? plan_pass<T, DIM, 3>(G, mean, C, smem) : plan_pass<T, DIM, 0>(G, mean, C, smem);
+}
+}  // namespace
+
+bool gas_sums_tiled(const void *geo, int precision, int dim, int64_t n, int mode)
+{
+    if (precision == TFSPH_FP64)
+        return dim == 1 ? gas_sums_tiled_t<double, 1>(geo, n, mode)
+                        : (dim == 2 ? gas_sums_tiled_t<double, 2>(geo, n, mode) : gas_sums_tiled_t<double, 3>(geo, n, mode));
+    return dim == 1 ? gas_sums_tiled_t<float, 1>(geo, n, mode)
+                    : (dim == 2 ? gas_sums_tiled_t<float, 2>(geo, n, mode) : gas_sums_tiled_t<float, 3>(geo, n, mode));
+}
 
 bool nblist_layout(const void *geo, int precision, int dim, int64_t n, int *cap, int *owned_cap, int64_t *tiles)
 {

@@ -198,6 +198,9 @@ cudaError_t launch_force(const LaunchCtx &L, const void *geo, const void *phys, 
 // owned particles per tile with a list, and tiles; false when the density
 // pass of this geometry is not tiled or its tiles cannot index a list.
 bool nblist_layout(const void *geo, int precision, int dim, int64_t n, int *cap, int *owned_cap, int64_t *tiles);
+// Whether a gas pair pass (MODE 0, 2 or 3) of n particles runs on tiles, which
+// sets the order of its sums.
+bool gas_sums_tiled(const void *geo, int precision, int dim, int64_t n, int mode);
 cudaError_t launch_force_adjoint(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G,
                                  const void *lamA, void *out);
 cudaError_t launch_density_adjoint(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G,
@@ -311,6 +314,7 @@ struct SmallPlan {
     void *fn = nullptr;  // NULL: not taken
     int grid = 0, threads = 128, lanes = 1;
     bool cluster = false;
+    bool density_tiles = true, force_tiles = true;  // the order of the phase-per-launch sums
 };
 bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, int dim, int64_t ng, int64_t nd,
                 SmallPlan *P);

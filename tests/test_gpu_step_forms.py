@@ -1,6 +1,8 @@
 """The step rounds alike whatever came before it: after a density export, with
 its phases timed, or as it is (one launch for small contexts, one per phase
-otherwise). States are equal bit for bit: adiabatic and viscous gases."""
+otherwise). States are equal bit for bit: adiabatic and viscous gases, axes
+that wrap fully, cells much finer than the particles' spacing, and clusters
+whose tile does not fit shared memory."""
 import numpy as np
 import pytest
 
@@ -59,3 +61,36 @@ def test_viscous_and_energy_terms(case, prec):
         w.params.update(av_alpha=1.0, av_beta=2.0, eos=1)
         w.ge = np.linspace(1.0, 2.0, w.n_gas).astype(np.float32).astype(np.float64)
     _same(_states(b, _stir(w, 0.05)))
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("viscous", [False, True])
+@pytest.mark.parametrize("case", ["full_y", "full_x", "full_1d", "fine_cells", "cluster_1d", "cluster_2d"])
+def test_order_of_the_sums(case, viscous, prec):
+    """Random particles, so that the last bits tell one order of a sum from another."""
+    b = gpu_lib()
+    rng = np.random.default_rng(8)
+    dim = 1 if case in ("full_1d", "fine_cells", "cluster_1d") else 2
+    n = 900
+    x = lambda: rng.uniform(0.0, 0.999, (dim, n))
+    h = {"full_y": 0.03, "full_x": 0.03, "full_1d": 0.1, "fine_cells": 0.01, "cluster_1d": 0.004,
+         "cluster_2d": 0.02}[case]
+    cell = {"full_1d": 0.3, "fine_cells": 1e-4}.get(case, 2.0 * h)
+    hi = {"full_y": (1.0, 0.17), "full_x": (0.17, 1.0)}.get(case, (1.0, 1.0))[:dim]
+    w = workloads.dustywave(n=n, precision=prec)
+    w.gx, w.dx = x(), x()
+    if case.startswith("cluster"):
+        w.gx = np.concatenate([w.gx, 0.99 + 0.009 * rng.uniform(size=(dim, 6000)), 0.003 * rng.uniform(size=(dim, 3000))],
+                              axis=1)
+    for k in range(dim):
+        w.gx[k] *= hi[k]
+        w.dx[k] *= hi[k]
+    if prec == 0:
+        w.gx, w.dx = (a.astype(np.float32).astype(np.float64) for a in (w.gx, w.dx))
+    w.gv, w.du = np.zeros_like(w.gx), np.zeros_like(w.dx)
+    w.params.update(dim=dim, periodic=(1,) * dim + (0,) * (3 - dim), hi=hi + (1.0,) * (3 - dim), h=h, cell_size=cell,
+                    m_gas=1.0 / n, m_dust=1.0 / n)
+    if viscous:
+        w.params.update(av_alpha=1.0, av_beta=2.0)
+    w.tau = 1e-5
+    _same(_states(b, _stir(w, 0.5)))
