@@ -61,7 +61,7 @@ __host__ __device__ __forceinline__ int prefilter_floor(float x)
 
 // Calls row(u0, u1) with the half-open range of halo cells, u0 <= u1, of
 // every row within reach of a particle in halo cell h at fractions f of it;
-// lane sub of step lanes takes every step-th plane. h is the rounded estimate
+// lane sub of step lanes takes its planes (first_plane). h is the rounded estimate
 // of the cell, up to one off the cell the particle is stored in, and the
 // margins widen the radius, so a range may end past the staged halo where 2h
 // is just short of a whole number of cells; no neighbour lies there, and the
@@ -74,7 +74,7 @@ __host__ __device__ __forceinline__ void prefilter_rows(const Prefilter &P, cons
     const int oz1 = min(min(R[2], max(0, prefilter_floor(f[2] + tz))), H[2] - 1 - h[2]);
     const int oz0 = max(-min(R[2], max(0, prefilter_floor(tz - f[2] + 1.0f))), -h[2]);
 #pragma unroll 1
-    for (int oz = oz0 + sub; oz <= oz1; oz += step) {
+    for (int oz = first_plane(oz0, R[2], sub, step); oz <= oz1; oz += step) {
         const float sz = slab_dist(oz, f[2]) * P.w[2], dz2 = sz * sz;
         const float ty = prefilter_sqrt(fmaxf(P.reach2 - dz2, 0.0f)) * P.inv_w[1];
         const int oy1 = min(min(R[1], max(0, prefilter_floor(f[1] + ty))), H[1] - 1 - h[1]);

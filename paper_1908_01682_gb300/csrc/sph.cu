@@ -112,7 +112,7 @@ __device__ __forceinline__ void walk_tile(PairAcc<T, MODE> &A, const Geo<T> &G, 
                                           const V4<T> *spos, const V4<T> *svel, const T *srho, const uint32_t *sid,
                                           NbRec *rec, int sub = 0, int step = 1)
 {
-    // (step > 1, 3D: lane sub of step lanes, which takes every step-th plane)
+    // (step > 1, 3D: lane sub of step lanes, which takes its planes)
     // pa: the staged (possibly shifted) position the displacements use;
     // pc: the same position in box coordinates, for its cell and window
     T tx_, ty_ = T(0), tz_ = T(0);
@@ -138,7 +138,7 @@ __device__ __forceinline__ void walk_tile(PairAcc<T, MODE> &A, const Geo<T> &G, 
         oz0 = -min(G.R[2], max(0, floor_int(tz - fz + T(1))));
     }
 #pragma unroll 1
-    for (int oz = oz0 + sub; oz <= oz1; oz += step) {
+    for (int oz = first_plane(oz0, G.R[2], sub, step); oz <= oz1; oz += step) {
         T dz2 = T(0);
         int seam_z = 0;
         if (DIM > 2) {
@@ -307,7 +307,7 @@ __device__ __forceinline__ void read_list(PairAcc<T, MODE> &A, const Geo<T> &G, 
 }
 
 // SPLIT: C.lanes threads share an owned particle (each takes every lanes-th
-// plane of cells and keeps its own part of the list), for problems whose tiles
+// plane of cells (first_plane) and keeps its own part of the list), for problems whose tiles
 // of a thread per particle would not fill the chip.
 template <class T, int DIM, int MODE, bool SPLIT = false>
 __global__ void __launch_bounds__(kTileThreads, sizeof(T) == 4 ? ((MODE == 0 || MODE == 2) ? 4 : 3)

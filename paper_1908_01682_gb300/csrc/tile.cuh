@@ -85,6 +85,15 @@ __device__ inline int block_scan_smem(E *a, int m, int *wsum)
     return total;
 }
 
+// First plane from oz0 on that belongs to lane sub of step lanes (a power of
+// two), a plane's lane being its distance from plane -R modulo step: the lanes
+// of a particle then share out the planes whatever window each of them takes
+// (one whose list overflows walks in other arithmetic than the others).
+__host__ __device__ __forceinline__ int first_plane(int oz0, int R, int sub, int step)
+{
+    return oz0 + ((sub - (oz0 + R)) & (step - 1));
+}
+
 // Global cell coordinate of halo coordinate hc along axis k (-1: none).
 template <class T>
 __device__ __forceinline__ int halo_cell(const Geo<T> &G, int k, int c0, int hc)
