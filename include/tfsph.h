@@ -66,8 +66,13 @@ extern "C" {
 #define TFSPH_TSTAR_ARITHMETIC 0 /* t*_stop = mean of the cell's t_j */
 #define TFSPH_TSTAR_HARMONIC   1 /* t*_stop = L / sum 1/t_j */
 
-#define TFSPH_CELL_ACC_FP32 0   /* per-cell sums and drag solve in float */
-#define TFSPH_CELL_ACC_FP64 1   /* per-cell sums and drag solve in double */
+/* Per-cell sums and drag solve (and their adjoint), rounded to the state's type
+ * once at the end. FP64: in double on an FP64 state. On an FP32 state in
+ * two-float arithmetic: pairs of floats, 48 significant bits (each operation
+ * within 2^-48 to 15 * 2^-48 relative; tau and g enter as such pairs), and in
+ * double for a cell that leaves its exponent range. */
+#define TFSPH_CELL_ACC_FP32 0   /* in float */
+#define TFSPH_CELL_ACC_FP64 1   /* in double, or two-float arithmetic on an FP32 state */
 
 /* drag scheme (tfsph_params.drag). K = rho_d / t_stop (Eq. 7) with the
  * per-particle stopping times throughout. */

@@ -109,22 +109,21 @@ __device__ __forceinline__ int cell_adjoint_solve(const Phys<T> &Ph, const StepV
     }
     if (ng == 0 || nd == 0) return 0;
     const A N = A(ng), L = A(nd);
-    const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
+    const A dust = A(Ph.m_d) * L, gas = A(Ph.m_g) * N;
+    const A eps = dust / gas;
     const A tst = harmonic ? L / st : st / L;
     const A rt = tau / tst;
     const A den = one + rt * (one + eps);
     const A ig = one / (one + rt * eps), id = one / (one + rt);
     bool fits = true;
-    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    if constexpr (kPair) fits = df_drag_fits(tau, st, gas, dust, rt, eps);
     A wn[3] = {zero, zero, zero}, un[3] = {zero, zero, zero}, vn[3] = {zero, zero, zero};
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
         wn[k] = ((sv[k] / N - su[k] / L) + tau * (sa[k] / N)) / den;
         un[k] = su[k] / L + tau * gv[k] + rt * wn[k];
         vn[k] = un[k] + wn[k];
-        if constexpr (kPair)
-            fits = fits && !df_small(wn[k]) && !df_small(un[k]) && !df_small(vn[k]) &&
-                   df_in(un[k], -0x1p60f, 0x1p60f) && df_in(vn[k], -0x1p60f, 0x1p60f);
+        if constexpr (kPair) fits = fits && df_vel_fits(wn[k], un[k], vn[k], 0x1p60f);
     }
     // sums over the cell's particles of the lambdas reaching u*', v*', ig, id
     A S_un[3] = {zero, zero, zero}, S_vn[3] = {zero, zero, zero}, S_ig = zero, S_id = zero;
@@ -231,19 +230,19 @@ __device__ __forceinline__ int cell_adjoint_lanes(const Phys<T> &Ph, const StepV
     if (ng == 0 || nd == 0) return 0;
     const df st = lane_value(mask, su, (threadIdx.x & 31) | 3);
     const df N = df(ng), L = df(nd);
-    const df eps = df(Ph.m_d) * L / (df(Ph.m_g) * N);
+    const df dust = df(Ph.m_d) * L, gas = df(Ph.m_g) * N;
+    const df eps = dust / gas;
     const df tst = harmonic ? L / st : st / L;
     const df rt = tau / tst;
     const df den = one + rt * (one + eps);
     const df ig = one / (one + rt * eps), id = one / (one + rt);
-    bool fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    bool fits = df_drag_fits(tau, st, gas, dust, rt, eps);
     df wn = zero, un = zero, vn = zero, S_un = zero, S_vn = zero, S_ig = zero, S_id = zero;
     if (axis) {
         wn = ((sv / N - su / L) + tau * (sa / N)) / den;
         un = su / L + tau * g + rt * wn;
         vn = un + wn;
-        fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p60f, 0x1p60f) &&
-               df_in(vn, -0x1p60f, 0x1p60f);
+        fits = fits && df_vel_fits(wn, un, vn, 0x1p60f);
         for (uint32_t a = R.gs; a < R.ge; ++a) {
             if (has_frozen && (gid[a] & kFrozenBit)) continue;
             const df l = df(at(lgv, a)) + tau * df(at(lgx, a));

@@ -45,9 +45,9 @@ template <class A> __device__ __forceinline__ A step_val(df pair, double wide)
 // which is the cell average of the implicit Eqs. 19-20. Returns 1 when the
 // cell holds moving gas and dust (drag applies) and then sets un = u_*',
 // vn = v_*', ig = 1/(1 + tau eps*/t*) and id = 1/(1 + tau/t*). With A = df it
-// returns 2 where the binary32 exponent range may not hold the solve: tau/t*
-// outside [2^-60, 2^24], eps* outside [2^-40, 2^40], or a velocity so small
-// (nonzero, below 2^-80) or so large that low parts are lost.
+// returns 2 where the binary32 exponent range may not hold the solve: a scalar
+// outside the bounds of df_drag_fits, or a velocity so small (nonzero, below
+// 2^-80) or so large that low parts are lost.
 template <class T, class A, int DIM>
 __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals &S, int harmonic, int has_frozen,
                                                const V4<T> *__restrict__ gvel, const uint32_t *__restrict__ gid,
@@ -102,7 +102,8 @@ __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals
     if (ng == 0 || nd == 0) return 0;
     const A tau = step_val<A>(S.tau, S.dtau);
     const A N = A(ng), L = A(nd);
-    const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
+    const A dust = A(Ph.m_d) * L, gas = A(Ph.m_g) * N;
+    const A eps = dust / gas;
     // 1/N and 1/L from one division (N L is an exact product of counts)
     const A invNL = one / (N * L);
     const A invN = L * invNL, invL = N * invNL;
@@ -111,7 +112,7 @@ __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals
     const A den = one + rt * (one + eps);
     const A invden = one / den;  // one division for the DIM components
     bool fits = true;
-    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    if constexpr (kPair) fits = df_drag_fits(tau, st, gas, dust, rt, eps);
 #pragma unroll
     for (int k = 0; k < DIM; ++k) {
         const A vs = sv[k] * invN;
@@ -122,9 +123,7 @@ __device__ __forceinline__ int cell_drag_solve(const Phys<T> &Ph, const StepVals
         const A vn = un + wn;
         un_out[k] = T(un);
         vn_out[k] = T(vn);
-        if constexpr (kPair)
-            fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p100f, 0x1p100f) &&
-                   df_in(vn, -0x1p100f, 0x1p100f);
+        if constexpr (kPair) fits = fits && df_vel_fits(wn, un, vn, 0x1p100f);
     }
     // 1/(1 + rt eps) and 1/(1 + rt) from one division
     const A dg = one + rt * eps, dd = one + rt;
@@ -249,7 +248,8 @@ __device__ __forceinline__ int cell_drag_lanes(const Phys<T> &Ph, const StepVals
     const A st = lane_value(mask, su, (threadIdx.x & 31) | 3);
     const A tau = step_val<A>(S.tau, S.dtau);
     const A N = A(ng), L = A(nd);
-    const A eps = A(Ph.m_d) * L / (A(Ph.m_g) * N);
+    const A dust = A(Ph.m_d) * L, gas = A(Ph.m_g) * N;
+    const A eps = dust / gas;
     const A invNL = one / (N * L);
     const A invN = L * invNL, invL = N * invNL;
     const A rt = harmonic ? tau * st * invL : tau * L / st;
@@ -260,7 +260,7 @@ __device__ __forceinline__ int cell_drag_lanes(const Phys<T> &Ph, const StepVals
     ig_out = T(dd * invgd);
     id_out = T(dg * invgd);
     bool fits = true;
-    if constexpr (kPair) fits = df_in(rt, 0x1p-60f, 0x1p24f) && df_in(eps, 0x1p-40f, 0x1p40f);
+    if constexpr (kPair) fits = df_drag_fits(tau, st, gas, dust, rt, eps);
     if (axis) {
         const A g = k == 0 ? step_val<A>(S.g[0], S.dg[0])
                            : (k == 1 ? step_val<A>(S.g[1], S.dg[1]) : step_val<A>(S.g[2], S.dg[2]));
@@ -270,9 +270,7 @@ __device__ __forceinline__ int cell_drag_lanes(const Phys<T> &Ph, const StepVals
         const A vn = un + wn;
         un_out = T(un);
         vn_out = T(vn);
-        if constexpr (kPair)
-            fits = fits && !df_small(wn) && !df_small(un) && !df_small(vn) && df_in(un, -0x1p100f, 0x1p100f) &&
-                   df_in(vn, -0x1p100f, 0x1p100f);
+        if constexpr (kPair) fits = fits && df_vel_fits(wn, un, vn, 0x1p100f);
     }
     if constexpr (kPair) {
         if (!__all_sync(mask, fits)) return 2;
