@@ -237,7 +237,11 @@ int tfsph_debug(tfsph_ctx *c, int what, void *out, int mem_kind);
 int tfsph_info(const tfsph_ctx *c, tfsph_info_t *out);
 
 /* Start (enable = 1, clearing the totals) or stop (0) timing the phases of
- * tfsph_step with CUDA events recorded on the context's stream. */
+ * tfsph_step with CUDA events recorded on the context's stream. A timed step
+ * launches its phases one by one. Small 1D and 2D contexts otherwise run them
+ * all in one launch (the same results, and for the smallest a third of the
+ * time), so the phases of those are timed in another form than untimed steps
+ * take. */
 int tfsph_profile(tfsph_ctx *c, int enable);
 
 /* Synchronise and read the accumulated time per phase (TFSPH_PROF_*, ms,
@@ -246,8 +250,16 @@ int tfsph_profile(tfsph_ctx *c, int enable);
 int tfsph_profile_read(tfsph_ctx *c, double *ms, int64_t *steps, int64_t *launches);
 
 /* Wait for the context's stream and report any error raised on the device
- * since the last call (NONFINITE for bad t_stop values, INTERNAL otherwise). */
+ * since the last call: NONFINITE for bad t_stop values, TIMEOUT for a
+ * one-launch step of a small context whose grid barrier waited too long
+ * (INTERNAL otherwise). After TIMEOUT the step and what was queued behind it
+ * did not complete: steps and density exports are refused (TIMEOUT) until the
+ * state is set again (tfsph_set_state or tfsph_load_state). */
 int tfsph_sync(tfsph_ctx *c);
+
+/* How long a grid barrier of a one-launch step waits before it gives up, in
+ * milliseconds (>= 0; 2000 to begin with). */
+int tfsph_barrier_timeout(tfsph_ctx *c, double ms);
 
 /* Message of the last error of `c` (or of the last failed tfsph_init when c
  * is NULL). The string lives until the next call on the same context. */

@@ -124,6 +124,7 @@ def load() -> C.CDLL:
     lib.tfsph_info.argtypes = [ctxp, C.POINTER(tfsph_info_t)]
     lib.tfsph_sync.argtypes = [ctxp]
     lib.tfsph_profile.argtypes = [ctxp, i32]
+    lib.tfsph_barrier_timeout.argtypes = [ctxp, d]
     lib.tfsph_cell_ranges_noalloc.argtypes = [vp, i64, C.c_uint32, vp, vp]
     lib.tfsph_profile_read.argtypes = [ctxp, vp, vp, vp]
     lib.tfsph_dust_profile.argtypes = [C.POINTER(tfsph_grid_spec), vp, i64, vp, vp, vp, vp, vp]
@@ -152,7 +153,7 @@ def load() -> C.CDLL:
         getattr(lib, name).restype = C.c_int
     for name in ("tfsph_init", "tfsph_set_state", "tfsph_set_stream", "tfsph_step", "tfsph_step_adjoint", "tfsph_max_dt",
                  "tfsph_fields", "tfsph_debug", "tfsph_info", "tfsph_sync", "tfsph_version",
-                 "tfsph_profile", "tfsph_profile_read", "tfsph_cell_ranges_noalloc", "tfsph_state_bytes",
+                 "tfsph_profile", "tfsph_profile_read", "tfsph_barrier_timeout", "tfsph_cell_ranges_noalloc", "tfsph_state_bytes",
                  "tfsph_save_state", "tfsph_load_state", "tfsph_dust_profile"):
         getattr(lib, name).restype = C.c_int
     _lib = lib
@@ -235,6 +236,10 @@ def tfsph_info(ctx):
 
 def tfsph_sync(ctx) -> int:
     return load().tfsph_sync(ctx)
+
+
+def tfsph_barrier_timeout(ctx, ms: float) -> int:
+    return load().tfsph_barrier_timeout(ctx, float(ms))
 
 
 def tfsph_profile(ctx, enable: int) -> int:
@@ -520,7 +525,12 @@ class Context:
     def sync(self):
         _check(tfsph_sync(self.ctx), self.ctx)
 
+    def barrier_timeout(self, ms: float):
+        """How long a grid barrier of a small context's one-launch step waits before the step gives up."""
+        _check(tfsph_barrier_timeout(self.ctx, ms), self.ctx)
+
     def profile(self, enable: bool = True):
+        """Times the phases of the steps that follow (each its own launches, in small contexts too)."""
         _check(tfsph_profile(self.ctx, 1 if enable else 0), self.ctx)
 
     def profile_read(self):

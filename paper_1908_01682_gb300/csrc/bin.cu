@@ -127,11 +127,14 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_top(uint32_t *__restrict_
 __global__ void __launch_bounds__(kScanThreads)
 k_scan_down(const uint32_t *__restrict__ cg, const uint32_t *__restrict__ cd, uint32_t ncells,
             const uint32_t *__restrict__ bsum, uint32_t nblk, uint32_t *__restrict__ sg,
-            uint32_t *__restrict__ sd, uint32_t ng, uint32_t nd)
+            uint32_t *__restrict__ sd, uint32_t ng, uint32_t nd, const int *__restrict__ err)
 {
     const uint32_t *cnt = blockIdx.y == 0 ? cg : cd;
     uint32_t *st = blockIdx.y == 0 ? sg : sd;
-    const uint32_t n = blockIdx.y == 0 ? ng : nd;
+    // err (or NULL): behind a one-launch step that gave up, keys and positions
+    // may not belong together; every cell is then left empty, so that the
+    // passes that follow touch no particle
+    const uint32_t n = err && (*err & kErrTimeout) ? 0u : (blockIdx.y == 0 ? ng : nd);
     const uint32_t base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
     uint32_t v[kScanItems];
     load_items(cnt, base, ncells, v);
@@ -144,7 +147,7 @@ k_scan_down(const uint32_t *__restrict__ cg, const uint32_t *__restrict__ cd, ui
     uint32_t o[kScanItems];
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        o[k] = min(run, n);  // (past n: counts of a step that gave up)
+        o[k] = min(run, n);
         run += v[k];
     }
     if (base + kScanItems <= ncells) {
@@ -474,7 +477,7 @@ cudaError_t bin_t(const LaunchCtx &L, const void *geo, PhaseBufs &G, PhaseBufs &
     k_scan_reduce<<<sg, kScanThreads, 0, L.stream>>>(G.count, D.count, ncells, bsum, (uint32_t)nblk);
     k_scan_top<<<2, kScanThreads, 0, L.stream>>>(bsum, (uint32_t)nblk);
     k_scan_down<<<sg, kScanThreads, 0, L.stream>>>(G.count, D.count, ncells, bsum, (uint32_t)nblk, G.start,
-                                                   D.start, (uint32_t)ng, (uint32_t)nd);
+                                                   D.start, (uint32_t)ng, (uint32_t)nd, counted ? L.d_err : nullptr);
     if (L.ev) cudaEventRecord(L.ev[2], L.stream);
     if (ntot > 0) {
         auto scatter = agg ? k_scatter<true> : k_scatter<false>;

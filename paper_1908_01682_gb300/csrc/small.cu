@@ -24,7 +24,6 @@ namespace {
 
 constexpr int kSmallThreads = 512;  // most threads of a CTA
 constexpr int kSmallCluster = 8;    // most CTAs of the cluster form
-constexpr long long kSmallSpin = 4000000000ll;  // clock cycles a barrier waits at most (two seconds)
 
 template <class T> struct SmallArgs {
     Geo<T> G;
@@ -359,7 +358,7 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.acc = static_cast<V4<T> *>(acc);
     B.err = L.d_err;
     B.bar = bar;
-    B.spin = kSmallSpin;
+    B.spin = P.spin;
     B.ng = (uint32_t)G.n;
     B.nd = (uint32_t)D.n;
     B.lanes = P.lanes;

@@ -64,6 +64,7 @@ struct tfsph_ctx {
     size_t counts_bytes = 0;
     int *counted = nullptr;     // that word (NULL: no one-launch step, the counts stay zero)
     bool flags_dirty = false;   // d_flags may be nonzero
+    bool lost = false;          // a one-launch step gave up: the state is incomplete
     bool has_frozen = false;
     int64_t steps = 0;
     int64_t device_bytes = 0;
@@ -277,6 +278,7 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     if (flags & 1) return fail(c, TFSPH_E_NONFINITE, "non-finite position, velocity or energy in the input");
     if (flags & 4) return fail(c, TFSPH_E_NONFINITE, "dust t_stop must be finite and > 0");
     if (flags & 2) return fail(c, TFSPH_E_OUT_OF_DOMAIN, "a moving particle lies outside [lo, hi)");
+    c->lost = false;
     c->steps = 0;
     return TFSPH_OK;
 }
@@ -315,8 +317,14 @@ int next_events(tfsph_ctx *c, cudaEvent_t **out)
     return TFSPH_OK;
 }
 
+int refuse_lost(tfsph_ctx *c)
+{
+    return c->lost ? fail(c, TFSPH_E_TIMEOUT, "a step gave up at a grid barrier: set a new state first") : TFSPH_OK;
+}
+
 int prepare(tfsph_ctx *c, cudaEvent_t *ev = nullptr)
 {
+    if (int rc = refuse_lost(c)) return rc;
     if (c->prepared) {
         if (ev)
             for (int k = 1; k <= TFSPH_PROF_DENSITY + 1; ++k) TF_CUDA(c, cudaEventRecord(ev[k], c->stream));
@@ -453,6 +461,9 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
             if ((rc = dalloc(c, &P->vel[b], n * v4))) return bail(rc);
             if ((rc = dalloc(c, &tmp, n * 4))) return bail(rc);
             P->id[b] = static_cast<uint32_t *>(tmp);
+            // (ids in range from the start: a first step that gives up leaves some of them unwritten)
+            e = cudaMemset(tmp, 0, n * 4);
+            if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
         }
         if ((rc = dalloc(c, &tmp, n * 4))) return bail(rc);
         P->key = static_cast<uint32_t *>(tmp);
@@ -554,6 +565,7 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
             gg[k] = k < c->dim ? g[k] : 0.0;
         }
     }
+    if (int rc = refuse_lost(c)) return rc;
     LaunchCtx L = lctx(c);
     const int64_t launches0 = c->launches;
     if (t_stop && c->D.n > 0) {
@@ -627,6 +639,16 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
     c->forced = false;
     c->nbl_valid = false;
     c->steps += 1;
+    return TFSPH_OK;
+}
+
+int tfsph_barrier_timeout(tfsph_ctx *c, double ms)
+{
+    if (!c) return fail(nullptr, TFSPH_E_INVALID_ARG, "ctx is NULL");
+    if (!(ms >= 0) || !std::isfinite(ms)) return fail(c, TFSPH_E_INVALID_ARG, "timeout must be finite and >= 0");
+    int khz = 0;
+    TF_CUDA(c, cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, c->device));
+    c->small.spin = (long long)std::min(ms * std::max(khz, 1), 9e18);
     return TFSPH_OK;
 }
 
@@ -980,6 +1002,7 @@ int tfsph_load_state(tfsph_ctx *c, const void *buf, int mem_kind)
     // (the counts in step with the stream: a one-launch step may have left some)
     if (c->counted) TF_CUDA(c, clear_counts(c));
     else c->counts_dirty = true;
+    c->lost = false;
     if (h.steps >= 0) c->steps = h.steps;
     return TFSPH_OK;
 }
@@ -1156,6 +1179,7 @@ int tfsph_sync(tfsph_ctx *c)
             // the barrier and the counts were left as the wait found them
             TF_CUDA(c, cudaMemsetAsync(c->bar, 0, 32, c->stream));
             TF_CUDA(c, clear_counts(c));
+            c->lost = true;
             return fail(c, TFSPH_E_TIMEOUT, "a grid barrier of the one-launch step waited too long");
         }
         if (err & kErrBadTstop) return fail(c, TFSPH_E_NONFINITE, "a t_stop value was <= 0 or not finite");
