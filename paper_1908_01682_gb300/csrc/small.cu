@@ -45,7 +45,6 @@ template <class T> struct SmallArgs {
     uint32_t cpc; // cells a CTA updates at a time
     int *counted; // nonzero: gcnt, dcnt hold the counts of the current keys (the last step left them)
     int cluster;  // the grid is one cluster
-    int order[2]; // density, force: the sums in the order of the tiled walks (gas_sums_tiled)
     int harmonic, has_frozen, adiabatic;
 };
 
@@ -160,7 +159,7 @@ template <class T, int DIM, int MODE> __device__ __forceinline__ void small_pair
         for_each_range<T, DIM>(B.G, B.gstart, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {
             if (seam) range(b0, n, SeamTag<true>{});
             else range(b0, n, SeamTag<false>{});
-        }, B.order[MODE != 0]);
+        }, true);
         if (MODE == 0)
             acc_store<T, MODE>(A, B.Ph, a, B.Ph.m_g, vel, B.rho, reinterpret_cast<T *>(B.gpb), nullptr, nullptr,
                                nullptr);
@@ -199,7 +198,7 @@ template <class T, int MODE> __device__ __forceinline__ void small_pair_lanes(co
                     }
                 seams |= (seam ? 1u : 0u) << nr;
                 ++nr;
-            }, B.order[MODE != 0]);
+            }, true);
         const uint32_t m = rn[0] + rn[1] + rn[2];
         const uint32_t most = __reduce_max_sync(0xffffffffu, m);
         for (uint32_t c0 = 0; c0 < most; c0 += (uint32_t)lanes) {
@@ -364,8 +363,6 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.lanes = P.lanes;
     B.counted = counted;
     B.cluster = P.cluster;
-    B.order[0] = P.density_tiles;
-    B.order[1] = P.force_tiles;
     // cells shared out evenly over the CTAs, at most what four lanes each allow
     B.cpc = std::min((uint32_t)P.threads / 4, std::max(1u, (B.G.ncells + (uint32_t)P.grid - 1) / (uint32_t)P.grid));
     B.harmonic = S.tstar_mode == TFSPH_TSTAR_HARMONIC;
@@ -408,9 +405,14 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     const int eos = f64 ? static_cast<const Phys<double> *>(phys)->eos : static_cast<const Phys<float> *>(phys)->eos;
     if (dim > 2 || ng <= 0 || nd <= 0 || ng + nd > kSmallParticles || ncells > kSmallCells) return false;
     const bool full = av || eos == TFSPH_EOS_ADIABATIC;
+    // The sums here run in the order of the tiled walks. Where the passes do not
+    // run on tiles (cells much finer than the particles' spacing, a y axis that
+    // wraps fully), their order is another one and the step keeps their form;
+    // an x axis that wraps fully has one order only.
+    const int full_x = f64 ? static_cast<const Geo<double> *>(geo)->full[0] : static_cast<const Geo<float> *>(geo)->full[0];
+    if (!full_x && !(gas_sums_tiled(geo, precision, dim, ng, 0) && gas_sums_tiled(geo, precision, dim, ng, full ? 3 : 2)))
+        return false;
     P->fn = pick(precision, cell_acc, dim, full);
-    P->density_tiles = gas_sums_tiled(geo, precision, dim, ng, 0);
-    P->force_tiles = gas_sums_tiled(geo, precision, dim, ng, full ? 3 : 2);
     int dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||

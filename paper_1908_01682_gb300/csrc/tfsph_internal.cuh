@@ -315,7 +315,6 @@ struct SmallPlan {
     int grid = 0, threads = 128, lanes = 1;
     bool cluster = false;
     long long spin = 4000000000ll;  // clock cycles a grid barrier waits at most (about two seconds)
-    bool density_tiles = true, force_tiles = true;  // the order of the phase-per-launch sums
 };
 bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, int dim, int64_t ng, int64_t nd,
                 SmallPlan *P);
