@@ -322,6 +322,18 @@ void *pick(int precision, int cell_acc, int dim, bool full)
     return cell_acc == TFSPH_CELL_ACC_FP64 ? pick_dim<float, df>(dim, full) : pick_dim<float, float>(dim, full);
 }
 
+// Launch of a grid that is one cluster.
+void cluster_config(cudaLaunchConfig_t &cfg, cudaLaunchAttribute attr[1], const SmallPlan &P)
+{
+    cfg.gridDim = dim3((unsigned)P.grid);
+    cfg.blockDim = dim3((unsigned)P.threads);
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)P.grid;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+}
+
 template <class T>
 cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D, void *rho,
                     void *acc, const StepArgs &S, const SmallPlan &P, GridBar *bar, int *counted)
@@ -370,20 +382,18 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.adiabatic = B.Ph.eos == TFSPH_EOS_ADIABATIC;
     void *args[] = {&B};
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)P.grid);
-    cfg.blockDim = dim3((unsigned)P.threads);
-    cfg.stream = L.stream;
     cudaLaunchAttribute attr[1];
     if (P.cluster) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)P.grid;
-        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cluster_config(cfg, attr, P);
     } else {
+        cfg.gridDim = dim3((unsigned)P.grid);
+        cfg.blockDim = dim3((unsigned)P.threads);
         attr[0].id = cudaLaunchAttributeCooperative;
         attr[0].val.cooperative = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
     }
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.stream = L.stream;
     const cudaError_t e = cudaLaunchKernelExC(&cfg, P.fn, args);
     if (e != cudaSuccess) return e;
     G.cur = og;
@@ -405,6 +415,7 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     const int eos = f64 ? static_cast<const Phys<double> *>(phys)->eos : static_cast<const Phys<float> *>(phys)->eos;
     if (dim > 2 || ng <= 0 || nd <= 0 || ng + nd > kSmallParticles || ncells > kSmallCells) return false;
     const bool full = av || eos == TFSPH_EOS_ADIABATIC;
+    void *fn = pick(precision, cell_acc, dim, full);
     // The sums here run in the order of the tiled walks. Where the passes do not
     // run on tiles (cells much finer than the particles' spacing, a y axis that
     // wraps fully), their order is another one and the step keeps their form;
@@ -412,7 +423,6 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     const int full_x = f64 ? static_cast<const Geo<double> *>(geo)->full[0] : static_cast<const Geo<float> *>(geo)->full[0];
     if (!full_x && !(gas_sums_tiled(geo, precision, dim, ng, 0) && gas_sums_tiled(geo, precision, dim, ng, full ? 3 : 2)))
         return false;
-    P->fn = pick(precision, cell_acc, dim, full);
     int dev = 0, sms = 0, coop = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -432,6 +442,25 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     P->grid = (int)std::min<int64_t>(P->cluster ? kSmallCluster : sms, warps);
     P->threads = 128;
     while (P->threads < kSmallThreads && warps * 32 > (int64_t)P->grid * P->threads) P->threads *= 2;
+    // whether the device holds the cluster, or a CTA on every SM, at once
+    if (P->cluster) {
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[1];
+        cluster_config(cfg, attr, *P);
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, fn, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            return false;
+        }
+    } else {
+        int per_sm = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, P->threads, 0) != cudaSuccess ||
+            (int64_t)per_sm * sms < P->grid) {
+            cudaGetLastError();
+            return false;
+        }
+    }
+    P->fn = fn;
     return true;
 }
 

@@ -605,14 +605,21 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
     // or a field export or snapshot has already done the first of them
     if (c->small.fn && !ev && !c->prepared) {
         if (c->counts_dirty) TF_CUDA(c, clear_counts(c));
-        c->counts_dirty = true;
-        TF_CUDA(c, launch_step_small(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->acc, S, c->small, c->bar, c->counted));
-        c->counts_dirty = false;
-        c->launches += 1;
-        c->forced = false;
-        c->nbl_valid = false;
-        c->steps += 1;
-        return TFSPH_OK;
+        const cudaError_t e =
+            launch_step_small(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->acc, S, c->small, c->bar, c->counted);
+        if (e == cudaSuccess) {
+            c->launches += 1;
+            c->forced = false;
+            c->nbl_valid = false;
+            c->steps += 1;
+            return TFSPH_OK;
+        }
+        // fewer SMs than the device has (a stream of a partition of it, say):
+        // nothing has run, and the phases take their own launches from here on
+        if (e != cudaErrorCooperativeLaunchTooLarge && e != cudaErrorNotSupported)
+            return cuda_fail(c, e, "one-launch step");
+        cudaGetLastError();
+        c->small.fn = nullptr;
     }
     if (ev) TF_CUDA(c, cudaEventRecord(ev[0], c->stream));
     rc = forward_quantities(c, ev);
