@@ -45,6 +45,7 @@ template <class T> struct SmallArgs {
     uint32_t cpc; // cells a CTA updates at a time
     int *counted; // nonzero: gcnt, dcnt hold the counts of the current keys (the last step left them)
     int cluster;  // the grid is one cluster
+    int few;      // few candidates per particle: terms without a branch (binary64 in 1D)
     int harmonic, has_frozen, adiabatic;
 };
 
@@ -124,36 +125,44 @@ template <class T, int DIM, int MODE> __device__ __forceinline__ void small_pair
         const V4<T> pa = pos[a];
         acc_init(A, B.Ph, pa, vel, rho, a);
         auto range = [&](uint32_t b0, uint32_t n, auto seam) {
-            if constexpr (sizeof(T) == 8 && (MODE == 0 || MODE == 2)) {
-                // four chains of binary64 operations in flight
-                constexpr int kAhead = 4;
+            // four candidates loaded, and their distances formed, at a time
+            constexpr int kAhead = 4;
+            if constexpr (sizeof(T) == 8 && DIM == 1 && (MODE == 0 || MODE == 2)) {
+                if (B.few) {
+                    // four chains of binary64 operations in flight
 #pragma unroll 1
-                for (uint32_t b = b0; b < b0 + n; b += kAhead) {
-                    T s[kAhead], d[kAhead][3];
+                    for (uint32_t b = b0; b < b0 + n; b += kAhead) {
+                        T s[kAhead], d[kAhead][3];
 #pragma unroll
-                    for (int u = 0; u < kAhead; ++u) {
-                        const bool have = b + u < b0 + n;
-                        const V4<T> pb = pos[have ? b + u : b];
-                        const T r2 = pair_r2<T, DIM, decltype(seam)::value>(B.G, pa, pb, d[u]);
-                        s[u] = pair_term<T, DIM, MODE>(A, B.G, B.Ph, pb, r2, d[u], have && r2 < B.G.h2x4);
+                        for (int u = 0; u < kAhead; ++u) {
+                            const bool have = b + u < b0 + n;
+                            const V4<T> pb = pos[have ? b + u : b];
+                            const T r2 = pair_r2<T, DIM, decltype(seam)::value>(B.G, pa, pb, d[u]);
+                            s[u] = pair_term<T, DIM, MODE>(A, B.G, B.Ph, pb, r2, d[u], have && r2 < B.G.h2x4);
+                        }
+#pragma unroll
+                        for (int u = 0; u < kAhead; ++u) add_term<T, DIM, MODE>(A, s[u], d[u]);
                     }
-#pragma unroll
-                    for (int u = 0; u < kAhead; ++u) add_term<T, DIM, MODE>(A, s[u], d[u]);
+                    return;
                 }
-                return;
             }
 #pragma unroll 1
-            for (uint32_t b = b0; b < b0 + n; ++b) {
-                const V4<T> pb = pos[b];
-                T d[3];
-                const T r2 = pair_r2<T, DIM, decltype(seam)::value>(B.G, pa, pb, d);
-                V4<T> vb;
-                T rhob = T(1);
-                if (r2 < B.G.h2x4) {
-                    if (ModeUses<MODE>::vel) vb = vel[b];
-                    if (ModeUses<MODE>::rho) rhob = rho[b];
+            for (uint32_t b = b0; b < b0 + n; b += kAhead) {
+                V4<T> pb[kAhead];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) pb[u] = pos[b + u < b0 + n ? b + u : b];
+#pragma unroll
+                for (int u = 0; u < kAhead; ++u) {
+                    T d[3];
+                    const T r2 = pair_r2<T, DIM, decltype(seam)::value>(B.G, pa, pb[u], d);
+                    if (b + u < b0 + n && r2 < B.G.h2x4) {
+                        V4<T> vb;
+                        T rhob = T(1);
+                        if (ModeUses<MODE>::vel) vb = vel[b + u];
+                        if (ModeUses<MODE>::rho) rhob = rho[b + u];
+                        A.template add<DIM, true>(B.G, B.Ph, pb[u], &vb, rhob, 0u, r2, d);
+                    }
                 }
-                A.template add<DIM>(B.G, B.Ph, pb, &vb, rhob, 0u, r2, d);
             }
         };
         for_each_range<T, DIM>(B.G, B.gstart, pa.x, pa.y, pa.z, [&](uint32_t b0, uint32_t n, bool seam) {
@@ -375,6 +384,7 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     B.lanes = P.lanes;
     B.counted = counted;
     B.cluster = P.cluster;
+    B.few = (double)G.n * (2 * B.G.R[0] + 1) <= 16.0 * (double)B.G.ncells;
     // cells shared out evenly over the CTAs, at most what four lanes each allow
     B.cpc = std::min((uint32_t)P.threads / 4, std::max(1u, (B.G.ncells + (uint32_t)P.grid - 1) / (uint32_t)P.grid));
     B.harmonic = S.tstar_mode == TFSPH_TSTAR_HARMONIC;
@@ -403,8 +413,16 @@ cudaError_t small_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
 
 }  // namespace
 
-// Which contexts take the one-launch step. Beyond the limits the pair sums
-// fill the chip by themselves and the tiled kernels are the faster ones.
+// Which contexts take the one-launch step. us a step, one launch against one
+// per phase (2 x n particles):
+//   1D FP32 waves      2 x 1000 25 | 49, 2 x 16384 37 | 50, 2 x 32768 40 | 49, 2 x 131072 58 | 59
+//   1D FP64 waves      2 x 1000 31 | 64, 2 x 16384 60 | 70, 2 x 32768 67 | 70, 2 x 131072 138 | 152
+//   1D FP32, 600 candidates a particle   2 x 2000 216 | 303, 2 x 20000 223 | 325
+//   shocks, FP32 and FP64   2 x 16384 61 | 98 and 262 | 652
+//   2D columns, FP32   2 x 900 68 | 84, 2 x 4096 70 | 93, 2 x 16384 75 | 89
+//   2D columns, FP64   2 x 900 379 | 383, 2 x 4096 379 | 490, 2 x 16384 356 | 505
+// The particle limit is where the gain has become small in FP64; in FP32 it
+// still gains some beyond (2 x 49152 41 | 50).
 bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, int dim, int64_t ng, int64_t nd,
                 SmallPlan *P)
 {
@@ -435,6 +453,14 @@ bool small_plan(const void *geo, const void *phys, int precision, int cell_acc, 
     if (f64 && dim == 1)
         while (lanes < 8 && (ng * lanes * 2 + 31) / 32 <= (int64_t)4 * sms) lanes *= 2;
     P->lanes = lanes;
+    // A binary64 particle of many candidates with a lane of its own: the pair
+    // sums bound both forms, and the tiles have more warps, up to a tile per few
+    // cells (1D, isothermal, 20,000 + 20,000 particles, one launch against
+    // phases: 60 candidates 166 against 165 us a step, 90: 230 against 214, 180:
+    // 393 against 348, 600: 1317 against 1753).
+    const int reach = f64 ? static_cast<const Geo<double> *>(geo)->R[0] : 0;
+    const double seen = (double)ng * (2 * reach + 1) / (double)ncells;
+    if (f64 && dim == 1 && lanes == 1 && !full && seen > 64.0 && seen <= 400.0) return false;
     // up to one CTA an SM. Up to kSmallCluster CTAs' worth of warps: one
     // cluster, whose barrier takes 0.1 us against about 1.5 us for the grid's.
     const int64_t warps = std::max((ng * lanes + 31) / 32, (nd + 31) / 32);
