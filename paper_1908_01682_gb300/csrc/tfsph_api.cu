@@ -509,6 +509,9 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
         if ((rc = dalloc(c, &c->xb.g1, (size_t)n_gas * c->tsize))) return bail(rc);
         if ((rc = dalloc(c, &c->xb.d4, (size_t)n_dust * v4))) return bail(rc);
         if ((rc = dalloc(c, &c->xb.d4b, (size_t)n_dust * v4))) return bail(rc);
+        void *over = nullptr;
+        if (c->precision == TFSPH_FP32 && c->dim == 3 && (rc = dalloc(c, &over, 2 * (size_t)c->ncells))) return bail(rc);
+        c->xb.over = static_cast<uint8_t *>(over);
     }
     c->nblk = ((int64_t)c->ncells + kScanTile - 1) / kScanTile;
     void *tmp;
@@ -520,7 +523,8 @@ int tfsph_init(tfsph_ctx **out, const tfsph_params *p, const void *const *gas, i
     if ((rc = dalloc(c, &tmp, 64))) return bail(rc);
     c->d_err = static_cast<int *>(tmp);
     c->d_flags = c->d_err + 4;  // in the error word's block, zeroed below
-    c->xb.gate = c->d_err + 5;
+    c->xb.gate = c->d_err + 5;  // two words
+    c->xb.any = c->d_err + 7;
     e = cudaMemset(c->d_err, 0, 64);
     if (e != cudaSuccess) return bail(cuda_fail(c, e, "cudaMemset"));
     if (p->drag == TFSPH_DRAG_IDIC)

@@ -326,7 +326,11 @@ cudaError_t launch_step_small(const LaunchCtx &L, const void *geo, const void *p
 // force. Scratch per particle: g4, d4, d4b (V4) and g1 (T).
 struct XDragBufs {
     void *g4 = nullptr, *g1 = nullptr, *d4 = nullptr, *d4b = nullptr;
-    int *gate = nullptr;  // one word: which form of the cross sums runs
+    int *gate = nullptr;  // a word per phase: whether it has left its lattice (the tiled cross sums then run)
+    // FP32 3D: per phase a byte per tile (at most one per cell), 1 where its
+    // targets are left to a thread each, and a word, 1 where any tile's are
+    uint8_t *over = nullptr;
+    int *any = nullptr;
 };
 cudaError_t launch_xdrag(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
                          const void *rho_g, const void *rho_d, const void *acc, const XDragBufs &B,

@@ -13,7 +13,7 @@
 // (FP32, isothermal, no walls) a CTA stages the source particles of a tile of
 // cells and its halo, 32 bytes each, and its threads take one target each
 // (k_xsum_tile). Otherwise one thread per target walks the other phase's
-// candidate cells in global memory (k_xsum).
+// candidate cells in global memory (k_xsum; k_xsum_rest behind the tiles).
 //   ISPH at gas a over dust:  rho^d_a = m_d sum W,  K_a,  u_a = m_d sum u_j/rho_j W
 //   ISPH at dust j over gas:  rho^g_j = m_g sum W,  v_j = m_g sum_moving v_a/rho_a W,
 //     e_j (adiabatic), pressure acceleration A_j = -(Q_j + q_j G_j) (Eq. 14)
@@ -53,9 +53,12 @@ template <class T> struct XArgs {
     V4<T> *out4;        // ISPH gas: (u_a, K_a); ISPH dust: (v_j, rho^g_j); MK: D
     V4<T> *out4b;       // ISPH dust: (A_j, 0)
     T *out1;            // ISPH gas: rho^d_a
-    // where both forms of the sums are launched: the word that tells which runs
+    // Tiled sums: two words, one of which is set where they run (NULL: they do),
+    // per tile whether its targets are left to a thread each, and whether any are.
     const int *gate = nullptr;
-    int run_if = 0;
+    uint8_t *over = nullptr;
+    int *any = nullptr;
+    int tile[3] = {1, 1, 1}, tiles[3] = {1, 1, 1};  // cells of a tile, tiles per axis
 };
 
 // One target's sums over its candidate cells in global memory.
@@ -150,9 +153,32 @@ __device__ __forceinline__ void xsum_global(const Geo<T> &G, const Phys<T> &Ph, 
 template <class T, int DIM, int KIND>
 __global__ void __launch_bounds__(kXThreads, sizeof(T) == 4 ? 12 : 1) k_xsum(Geo<T> G, Phys<T> Ph, XArgs<T> X)
 {
-    if (X.gate && *X.gate != X.run_if) return;
     const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < (uint32_t)X.n) xsum_global<T, DIM, KIND>(G, Ph, X, t);
+}
+
+// Behind the tiled sums of both kinds (gas targets in the first gas_blocks
+// CTAs): all targets where the tiled sums did not run, else those of the tiles
+// left to it. One launch, which usually returns at once (4 us a step).
+template <int KIND> __device__ __forceinline__ void xsum_rest(const Geo<float> &G, const Phys<float> &Ph,
+                                                              const XArgs<float> &X, uint32_t t)
+{
+    const bool all = X.gate && !(X.gate[0] | X.gate[1]);
+    if (!all && !*X.any) return;
+    if (t >= (uint32_t)X.n) return;
+    if (!all) {
+        const float4 p = X.tpos[t];
+        const int c[3] = {exact_cell(G, 0, p.x), exact_cell(G, 1, p.y), exact_cell(G, 2, p.z)};
+        if (!X.over[c[0] / X.tile[0] + X.tiles[0] * (c[1] / X.tile[1] + X.tiles[1] * (c[2] / X.tile[2]))]) return;
+    }
+    xsum_global<float, 3, KIND>(G, Ph, X, t);
+}
+template <int AT_GAS, int AT_DUST>
+__global__ void __launch_bounds__(kXThreads, 12)
+k_xsum_rest(Geo<float> G, Phys<float> Ph, XArgs<float> Xg, XArgs<float> Xd, uint32_t gas_blocks)
+{
+    if (blockIdx.x < gas_blocks) xsum_rest<AT_GAS>(G, Ph, Xg, blockIdx.x * blockDim.x + threadIdx.x);
+    else xsum_rest<AT_DUST>(G, Ph, Xd, (blockIdx.x - gas_blocks) * blockDim.x + threadIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -180,15 +206,6 @@ constexpr int kQueue = 8;
 // 2 CTAs per SM: 2 x (112 KB + static + 1 KB reserved) of 228 KB
 constexpr int kXTileSmem = 112 * 1024;
 constexpr int kXQueueBytes = kQueue * kXTileThreads * 2;
-
-__device__ __noinline__ void xsum_global_far(const Geo<float> G, const Phys<float> Ph, const XArgs<float> X, uint32_t t,
-                                             int kind)
-{
-    if (kind == kIsphAtGas) xsum_global<float, 3, kIsphAtGas>(G, Ph, X, t);
-    else if (kind == kIsphAtDust) xsum_global<float, 3, kIsphAtDust>(G, Ph, X, t);
-    else if (kind == kMkAtGas) xsum_global<float, 3, kMkAtGas>(G, Ph, X, t);
-    else xsum_global<float, 3, kMkAtDust>(G, Ph, X, t);
-}
 
 // The targets of a staged tile. SEAM: displacements take the periodic image
 // (tiles that could not be staged with their seam shifts).
@@ -357,7 +374,7 @@ template <int KIND>
 __global__ void __launch_bounds__(kXTileThreads, 2)
 k_xsum_tile(Geo<float> G, Phys<float> Ph, TileCfg C, XArgs<float> X)
 {
-    if (X.gate && *X.gate != X.run_if) return;
+    if (X.gate && !(X.gate[0] | X.gate[1])) return;
     extern __shared__ __align__(64) unsigned char smem[];
     __shared__ int wsum[kXTileThreads / 32];
     uint16_t *lstart = reinterpret_cast<uint16_t *>(smem);                 // nhalo + 1
@@ -426,18 +443,18 @@ k_xsum_tile(Geo<float> G, Phys<float> Ph, TileCfg C, XArgs<float> X)
     const int total = block_scan_smem(lstart, C.nhalo, wsum);
     block_scan_smem(rowpref, C.nrows, wsum);
     const int owned = rowpref[C.nrows];
-    if (total > C.cap) {  // the halo does not fit: candidates from global memory
-        for (int p = tid; p < owned; p += blockDim.x) {
-            int lo = 0, hi = C.nrows - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi + 1) >> 1;
-                if (rowpref[mid] <= p) lo = mid;
-                else hi = mid - 1;
-            }
-            xsum_global_far(G, Ph, X, (uint32_t)(rowg[lo] + p - rowpref[lo]), KIND);
-        }
-        return;
+    // A halo that does not fit: the targets are left to k_xsum_rest. A tile's
+    // own threads, walking global memory for them, were the last to finish by far
+    // (both phases in a layer of a quarter of the box, 50^3: ISPH 3444 -> 2261 us, MK
+    // 2180 -> 827; 96^3: 7560 -> 5465 and 5531 -> 3401; of half: 1287 -> 1210, 809 -> 635,
+    // 4015 -> 3190, 2984 -> 2129), except where few tiles overflow a little
+    // (50^3, cells of 1.5 spacings: 389 -> 424 and 290 -> 319).
+    const bool later = total > C.cap;
+    if (tid == 0) {
+        X.over[blockIdx.x] = later;
+        if (later) *X.any = 1;
     }
+    if (later) return;
     for (int h = tid; h < C.nhalo; h += blockDim.x) {
         const int j0 = lstart[h], j1 = lstart[h + 1];
         if (j1 == j0) continue;
@@ -473,85 +490,123 @@ k_xsum_tile(Geo<float> G, Phys<float> Ph, TileCfg C, XArgs<float> X)
         xsum_tile_walk<KIND, false>(G, Ph, C, c0, orig, X, lstart, rowpref, rowg, sa, sb, queue, owned);
 }
 
-// Whether the particles have left their lattice: 1 when their places inside
-// their cells, over kSample evenly spaced particles, spread by more than 0.1
-// cells (mean square over the axes; a lattice displaced by up to 0.17 of a
-// spacing has that, one out of step with the cells has 0.29). One CTA.
+// Whether the tiled sums pay, from the places f of kSample particles of a phase
+// (block 0 gas, 1 dust) inside their cells: not while both phases sit on
+// lattices in step with the cells. Summed over the axes, the
+// variance of f is then at most 0.03 (displacements of up to 0.17 of a
+// spacing), or, wherever the lattice lies in the cells (on their faces f is
+// next to 0 or 1), they hold one phase exactly: 1 - R^2 below 0.01, R the length of
+// the mean of exp(2 pi i f). A lattice displaced about the faces has lanes in
+// cells on both sides of them and counts as scattered (0.05 of a spacing, tiles
+// against a thread per target: 96^3 ISPH 1327 against 1397 us, MK 1126 against
+// 1078; 75^3 639 against 844 and 529 against 652; not displaced at all, 96^3:
+// 1383 against 1021 and 1176 against 768).
 constexpr int kSample = 4096;
-__global__ void __launch_bounds__(512) k_scattered(Geo<float> G, const float4 *__restrict__ pos, uint32_t n, int *out)
+__global__ void __launch_bounds__(512)
+k_scattered(Geo<float> G, const float4 *__restrict__ gpos, uint32_t ng, const float4 *__restrict__ dpos, uint32_t nd,
+            int *out)
 {
-    const uint32_t m = min((uint32_t)kSample, n);
-    float s[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    const float4 *pos = blockIdx.x == 0 ? gpos : dpos;
+    const uint32_t n = blockIdx.x == 0 ? ng : nd, m = min((uint32_t)kSample, n);
+    constexpr int kSums = 12;  // per axis: f, f^2, cos, sin
+    float s[kSums] = {};
     for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
-        const float4 p = pos[(uint32_t)((uint64_t)i * n / m)];
+        // in scattered order (evenly spaced slots may all be the first of their cell)
+        const float4 p = pos[(uint32_t)((uint64_t)i * 2654435761ull % n)];
         const float x[3] = {p.x, p.y, p.z};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float t = (x[k] - G.lo[k]) * G.inv_w[k], f = t - floorf(t);
-            s[k] += f;
-            s[3 + k] += f * f;
+            s[4 * k] += f;
+            s[4 * k + 1] += f * f;
+            s[4 * k + 2] += cospif(2.0f * f);
+            s[4 * k + 3] += sinpif(2.0f * f);
         }
     }
-    __shared__ float part[16][6];
+    __shared__ float part[16][kSums];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
+    for (int k = 0; k < kSums; ++k) {
         for (int o = 16; o > 0; o >>= 1) s[k] += __shfl_xor_sync(0xffffffffu, s[k], o);
         if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5][k] = s[k];
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        float var = 0.0f;
+        float spread = 0.0f, lost = 0.0f;
         for (int k = 0; k < 3; ++k) {
-            float a = 0.0f, b = 0.0f;
-            for (int w = 0; w < 16; ++w) {
-                a += part[w][k];
-                b += part[w][3 + k];
-            }
-            var += b / (float)m - (a / (float)m) * (a / (float)m);
+            float a[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+            for (int w = 0; w < 16; ++w)
+                for (int q = 0; q < 4; ++q) a[q] += part[w][4 * k + q];
+            for (int q = 0; q < 4; ++q) a[q] /= (float)m;
+            spread += a[1] - a[0] * a[0];
+            lost += 1.0f - (a[2] * a[2] + a[3] * a[3]);
         }
-        *out = var > 3.0f * 0.01f ? 1 : 0;
+        out[blockIdx.x] = spread > 0.03f && lost > 0.01f;  // (no particles, or no numbers: 0)
     }
 }
 
 // Targets that fill the chip with one thread each (12 CTAs an SM).
 constexpr int64_t kXFill = (int64_t)kSmCount * 12 * kXThreads;
 
-// The sums of one kind. Where the tiled form applies (sources of `mean` per
-// cell, a tile for every SM): alone when a thread per target would not fill
-// the chip (50^3 targets: 69 us against 126-130 us on the lattice, 106 against
-// 208 us off it); beyond, only once the particles have left their lattice.
-// There (884,736 targets displaced by up to 0.35 of a spacing) it takes 613
-// and 653 us against 702 and 898 us for ISPH and 625 against 711-722 us for
-// MK, because the lanes' rows differ in length; on a lattice (0.05) they do
-// not, and a thread per target takes 367-449 us against 426-453. Which runs is
-// decided on the device, where the cell ranges are (both are launched; the
-// other returns at once).
-template <class T, int DIM, int KIND>
-cudaError_t launch_xsum(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, XArgs<T> X, double mean, int *gate)
+// Most sources per cell of the tiled form beyond kXFill targets (cells of 1.5
+// spacings, 3.4 sources: 96^3 ISPH 1435 us against 1744, MK 1058 against 1253;
+// of two spacings, 8 sources: 2109 and 1645 against 1864 and 1306).
+constexpr double kXMean = 5.0;
+
+// The tiled sums of one kind, where they apply (a tile for every SM): alone when
+// a thread per target would not fill the chip (50^3 targets: 69 us against
+// 126-130 us on the lattice, 106 against 208 us off it); beyond, only while
+// k_scattered tells that they pay. There (884,736 targets displaced by up to
+// 0.35 of a spacing) they take 613 and 653 us against 702 and 898 us for ISPH
+// and 625 against 711-722 us for MK, because the lanes' rows differ in length;
+// on a lattice (0.05) they do not, and a thread per target takes 367-449 us
+// against 426-453. False: not launched.
+template <int KIND>
+bool launch_xsum_tile(const LaunchCtx &L, const Geo<float> &G, const Phys<float> &Ph, XArgs<float> &X, double mean,
+                      const XDragBufs &B, bool dust, cudaError_t &e)
 {
-    const unsigned blocks = (unsigned)((X.n + kXThreads - 1) / kXThreads);
+    TileCfg C{};
+    size_t smem = 0;
+    if (X.n <= 0 || X.has_frozen || Ph.eos != TFSPH_EOS_ISOTHERMAL || (mean > kXMean && X.n > kXFill) ||
+        !plan_tiles(G, 3, mean, 32, kXTileSmem - kXQueueBytes, kXTileThreads, C, smem) || C.cap > 0xFFFF ||
+        (int64_t)C.nt[0] * C.nt[1] * C.nt[2] < kSmCount)
+        return false;
+    // (per call: the attribute belongs to the device's copy of the kernel)
+    e = cudaFuncSetAttribute(k_xsum_tile<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXTileSmem);
+    if (e != cudaSuccess) return false;
+    if (X.n > kXFill) X.gate = B.gate;
+    X.over = B.over + (dust ? G.ncells : 0u);
+    X.any = B.any;
+    for (int k = 0; k < 3; ++k) {
+        X.tile[k] = C.T[k];
+        X.tiles[k] = C.nt[k];
+    }
+    k_xsum_tile<KIND><<<(unsigned)(C.nt[0] * C.nt[1] * C.nt[2]), kXTileThreads, smem + kXQueueBytes, L.stream>>>(G, Ph, C, X);
+    return true;
+}
+
+// Both kinds of sums of a scheme.
+template <class T, int DIM, int AT_GAS, int AT_DUST>
+cudaError_t launch_xsums(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, XArgs<T> Xg, XArgs<T> Xd, double mean_g,
+                         double mean_d, const XDragBufs &B)
+{
+    bool gas = false, dust = false;
+    cudaError_t e = cudaSuccess;
     if constexpr (sizeof(T) == 4 && DIM == 3) {
-        TileCfg C{};
-        size_t smem = 0;
-        if (!X.has_frozen && Ph.eos == TFSPH_EOS_ISOTHERMAL &&
-            plan_tiles(G, 3, mean, 32, kXTileSmem - kXQueueBytes, kXTileThreads, C, smem) && C.cap <= 0xFFFF &&
-            (int64_t)C.nt[0] * C.nt[1] * C.nt[2] >= kSmCount) {
-            // (per call: the attribute belongs to the device's copy of the kernel)
-            cudaError_t e = cudaFuncSetAttribute(k_xsum_tile<KIND>, cudaFuncAttributeMaxDynamicSharedMemorySize, kXTileSmem);
-            if (e != cudaSuccess) return e;
-            const bool choose = X.n > kXFill;
-            if (choose) {
-                X.gate = gate;
-                X.run_if = 0;
-                k_xsum<T, DIM, KIND><<<blocks, kXThreads, 0, L.stream>>>(G, Ph, X);
-                X.run_if = 1;
-            }
-            k_xsum_tile<KIND><<<(unsigned)(C.nt[0] * C.nt[1] * C.nt[2]), kXTileThreads, smem + kXQueueBytes, L.stream>>>(
-                G, Ph, C, X);
-            return cudaGetLastError();
+        if (std::max(Xg.n, Xd.n) > kXFill)
+            k_scattered<<<2, 512, 0, L.stream>>>(G, Xg.tpos, (uint32_t)Xg.n, Xd.tpos, (uint32_t)Xd.n, B.gate);
+        gas = launch_xsum_tile<AT_GAS>(L, G, Ph, Xg, mean_d, B, false, e);
+        if (e == cudaSuccess) dust = launch_xsum_tile<AT_DUST>(L, G, Ph, Xd, mean_g, B, true, e);
+        if (e != cudaSuccess) return e;
+    }
+    auto blocks = [](int n) { return (unsigned)((n + kXThreads - 1) / kXThreads); };
+    if (Xg.n > 0 && !gas) k_xsum<T, DIM, AT_GAS><<<blocks(Xg.n), kXThreads, 0, L.stream>>>(G, Ph, Xg);
+    if (Xd.n > 0 && !dust) k_xsum<T, DIM, AT_DUST><<<blocks(Xd.n), kXThreads, 0, L.stream>>>(G, Ph, Xd);
+    if constexpr (sizeof(T) == 4 && DIM == 3) {
+        if (gas || dust) {
+            const unsigned bg = gas ? blocks(Xg.n) : 0u, bd = dust ? blocks(Xd.n) : 0u;
+            k_xsum_rest<AT_GAS, AT_DUST><<<bg + bd, kXThreads, 0, L.stream>>>(G, Ph, Xg, Xd, bg);
         }
     }
-    k_xsum<T, DIM, KIND><<<blocks, kXThreads, 0, L.stream>>>(G, Ph, X);
     return cudaGetLastError();
 }
 
@@ -561,9 +616,10 @@ __global__ void __launch_bounds__(256)
 k_xupdate_gas(Geo<T> G, Phys<T> Ph, T tau, T g0, T g1, T g2, int has_frozen, V4<T> *__restrict__ pos,
               V4<T> *__restrict__ vel, const uint32_t *__restrict__ id, uint32_t *__restrict__ key,
               const T *__restrict__ rho, const V4<T> *__restrict__ acc, const V4<T> *__restrict__ x4,
-              const T *__restrict__ x1, int n)
+              const T *__restrict__ x1, int n, int *__restrict__ any)
 {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a == 0 && any) *any = 0;  // k_xsum_rest is done with it
     if (a >= n) return;
     V4<T> p = pos[a];
     if (has_frozen && (id[a] & kFrozenBit)) {
@@ -688,27 +744,20 @@ cudaError_t xdrag_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
                      static_cast<V4<T> *>(B.d4), static_cast<V4<T> *>(B.d4b), nullptr};
     const bool isph = scheme == TFSPH_DRAG_ISPH;
     const double mean_g = (double)ng / (double)G.ncells, mean_d = (double)nd / (double)G.ncells;
-    cudaError_t e = cudaSuccess;
-    if constexpr (sizeof(T) == 4 && DIM == 3)
-        if (std::max(ng, nd) > kXFill)
-            k_scattered<<<1, 512, 0, L.stream>>>(G, ng > 0 ? gpos : dpos, (uint32_t)(ng > 0 ? ng : nd), B.gate);
-    if (ng > 0)
-        e = isph ? launch_xsum<T, DIM, kIsphAtGas>(L, G, Ph, at_gas, mean_d, B.gate)
-                 : launch_xsum<T, DIM, kMkAtGas>(L, G, Ph, at_gas, mean_d, B.gate);
-    if (e == cudaSuccess && nd > 0)
-        e = isph ? launch_xsum<T, DIM, kIsphAtDust>(L, G, Ph, at_dust, mean_g, B.gate)
-                 : launch_xsum<T, DIM, kMkAtDust>(L, G, Ph, at_dust, mean_g, B.gate);
+    const cudaError_t e =
+        isph ? launch_xsums<T, DIM, kIsphAtGas, kIsphAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B)
+             : launch_xsums<T, DIM, kMkAtGas, kMkAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B);
     if (e != cudaSuccess) return e;
     const T tau = T(S.tau), g0 = T(S.g[0]), g1 = T(S.g[1]), g2 = T(S.g[2]);
     if (ng > 0) {
         if (isph)
             k_xupdate_gas<T, DIM, TFSPH_DRAG_ISPH><<<blocks_for(ng, 256), 256, 0, L.stream>>>(
                 G, Ph, tau, g0, g1, g2, S.has_frozen, gpos, gvel, Gp.id[Gp.cur], Gp.key, rg,
-                static_cast<const V4<T> *>(acc), static_cast<const V4<T> *>(B.g4), static_cast<const T *>(B.g1), ng);
+                static_cast<const V4<T> *>(acc), static_cast<const V4<T> *>(B.g4), static_cast<const T *>(B.g1), ng, B.any);
         else
             k_xupdate_gas<T, DIM, TFSPH_DRAG_MK><<<blocks_for(ng, 256), 256, 0, L.stream>>>(
                 G, Ph, tau, g0, g1, g2, S.has_frozen, gpos, gvel, Gp.id[Gp.cur], Gp.key, rg,
-                static_cast<const V4<T> *>(acc), static_cast<const V4<T> *>(B.g4), static_cast<const T *>(B.g1), ng);
+                static_cast<const V4<T> *>(acc), static_cast<const V4<T> *>(B.g4), static_cast<const T *>(B.g1), ng, B.any);
     }
     if (nd > 0) {
         if (isph)
