@@ -638,8 +638,8 @@ int tfsph_step(tfsph_ctx *c, double tau, const void *t_stop, int mem_kind, const
             TF_CUDA(c, launch_density(L, c->geo, c->phys, c->D, c->rho_d, false, nullptr, nullptr));
             c->launches += 1;
         }
-        TF_CUDA(c, launch_xdrag(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->rho_d, c->acc, c->xb, S, c->p.drag));
-        c->launches += 2 * ((c->G.n > 0 ? 1 : 0) + (c->D.n > 0 ? 1 : 0));
+        TF_CUDA(c, launch_xdrag(L, c->geo, c->phys, c->G, c->D, c->rho_g, c->rho_d, c->acc, c->xb, S, c->p.drag,
+                                &c->launches));
     }
     if (ev) {
         TF_CUDA(c, cudaEventRecord(ev[TFSPH_PROF_DRAG + 1], c->stream));
@@ -817,9 +817,12 @@ struct SnapPart {
 // One launch copies every part of a device snapshot and, when saving, writes
 // the header, instead of one copy call per array. Every part size and offset
 // is a multiple of 4 bytes. The parts are cut into pieces of four words, shared
-// out over the whole grid at once with two in flight per thread; a part whose
-// two ends are 16-byte aligned moves its pieces as 16-byte words (512^2 column,
-// 25 MB: 14 us against 19 part after part in single words).
+// out over the whole grid at once with two in flight per thread (512^2 column,
+// 25 MB: 16 us against 19 part after part); a part whose two ends are 16-byte
+// aligned moves its pieces as 16-byte words. The header's 72 bytes put the
+// large parts of an aligned buffer 8 bytes past such a boundary, so that form
+// is taken by a buffer that starts at 8 mod 16 (10 us), or by a part whose
+// offset makes up for it.
 constexpr int kCopyParts = 12;
 constexpr int kHeaderWords = (int)(sizeof(SnapHeader) / 4);
 static_assert(sizeof(SnapHeader) % 4 == 0, "snapshot header is copied in words");

@@ -8,7 +8,9 @@
 //   id[2]   : uint32 particle id; bit 31 marks a frozen (wall) gas particle.
 //   key     : uint32 cell key of the particle in each storage slot, written by
 //             the update of the previous step (or at set-up).
-//   count   : uint32 per cell, zero between steps (the scatter counts it down).
+//   count   : uint32 per cell, zero between steps (the scatter counts it down),
+//             but for contexts of the one-launch step, whose update leaves the
+//             counts of the next keys and sets the word behind them.
 //   start   : uint32 per cell + 1, first storage slot of each cell.
 // Gas only: rho (T) and acc (V4<T>: ax, ay, az, de/dt).
 #pragma once
@@ -334,7 +336,7 @@ struct XDragBufs {
 };
 cudaError_t launch_xdrag(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
                          const void *rho_g, const void *rho_d, const void *acc, const XDragBufs &B,
-                         const StepArgs &S, int scheme);
+                         const StepArgs &S, int scheme, int64_t *launches);  // launches: kernels, added
 cudaError_t launch_cell_adjoint(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
                                 const void *acc, const StepArgs &S, const void *lgx, void *lgv, const void *ldx,
                                 void *ldu, void *lA, void *lts);

@@ -587,13 +587,15 @@ bool launch_xsum_tile(const LaunchCtx &L, const Geo<float> &G, const Phys<float>
 // Both kinds of sums of a scheme.
 template <class T, int DIM, int AT_GAS, int AT_DUST>
 cudaError_t launch_xsums(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph, XArgs<T> Xg, XArgs<T> Xd, double mean_g,
-                         double mean_d, const XDragBufs &B)
+                         double mean_d, const XDragBufs &B, int64_t *launches)
 {
     bool gas = false, dust = false;
     cudaError_t e = cudaSuccess;
     if constexpr (sizeof(T) == 4 && DIM == 3) {
-        if (std::max(Xg.n, Xd.n) > kXFill)
+        if (std::max(Xg.n, Xd.n) > kXFill) {
             k_scattered<<<2, 512, 0, L.stream>>>(G, Xg.tpos, (uint32_t)Xg.n, Xd.tpos, (uint32_t)Xd.n, B.gate);
+            ++*launches;
+        }
         gas = launch_xsum_tile<AT_GAS>(L, G, Ph, Xg, mean_d, B, false, e);
         if (e == cudaSuccess) dust = launch_xsum_tile<AT_DUST>(L, G, Ph, Xd, mean_g, B, true, e);
         if (e != cudaSuccess) return e;
@@ -605,8 +607,10 @@ cudaError_t launch_xsums(const LaunchCtx &L, const Geo<T> &G, const Phys<T> &Ph,
         if (gas || dust) {
             const unsigned bg = gas ? blocks(Xg.n) : 0u, bd = dust ? blocks(Xd.n) : 0u;
             k_xsum_rest<AT_GAS, AT_DUST><<<bg + bd, kXThreads, 0, L.stream>>>(G, Ph, Xg, Xd, bg);
+            ++*launches;
         }
     }
+    *launches += (Xg.n > 0) + (Xd.n > 0);  // (a sum of each, tiled or not)
     return cudaGetLastError();
 }
 
@@ -725,7 +729,7 @@ unsigned blocks_for(int64_t n, int threads) { return (unsigned)((n + threads - 1
 template <class T, int DIM>
 cudaError_t xdrag_t(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &Gp, PhaseBufs &Dp,
                     const void *rho_g, const void *rho_d, const void *acc, const XDragBufs &B, const StepArgs &S,
-                    int scheme)
+                    int scheme, int64_t *launches)
 {
     const Geo<T> &G = *static_cast<const Geo<T> *>(geo);
     const Phys<T> &Ph = *static_cast<const Phys<T> *>(phys);
@@ -745,10 +749,11 @@ cudaError_t xdrag_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
     const bool isph = scheme == TFSPH_DRAG_ISPH;
     const double mean_g = (double)ng / (double)G.ncells, mean_d = (double)nd / (double)G.ncells;
     const cudaError_t e =
-        isph ? launch_xsums<T, DIM, kIsphAtGas, kIsphAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B)
-             : launch_xsums<T, DIM, kMkAtGas, kMkAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B);
+        isph ? launch_xsums<T, DIM, kIsphAtGas, kIsphAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B, launches)
+             : launch_xsums<T, DIM, kMkAtGas, kMkAtDust>(L, G, Ph, at_gas, at_dust, mean_g, mean_d, B, launches);
     if (e != cudaSuccess) return e;
     const T tau = T(S.tau), g0 = T(S.g[0]), g1 = T(S.g[1]), g2 = T(S.g[2]);
+    *launches += (ng > 0) + (nd > 0);
     if (ng > 0) {
         if (isph)
             k_xupdate_gas<T, DIM, TFSPH_DRAG_ISPH><<<blocks_for(ng, 256), 256, 0, L.stream>>>(
@@ -776,19 +781,19 @@ cudaError_t xdrag_t(const LaunchCtx &L, const void *geo, const void *phys, Phase
 
 cudaError_t launch_xdrag(const LaunchCtx &L, const void *geo, const void *phys, PhaseBufs &G, PhaseBufs &D,
                          const void *rho_g, const void *rho_d, const void *acc, const XDragBufs &B,
-                         const StepArgs &S, int scheme)
+                         const StepArgs &S, int scheme, int64_t *launches)
 {
     if (L.precision == TFSPH_FP64) {
         switch (L.dim) {
-            case 1: return xdrag_t<double, 1>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
-            case 2: return xdrag_t<double, 2>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
-            default: return xdrag_t<double, 3>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
+            case 1: return xdrag_t<double, 1>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
+            case 2: return xdrag_t<double, 2>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
+            default: return xdrag_t<double, 3>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
         }
     }
     switch (L.dim) {
-        case 1: return xdrag_t<float, 1>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
-        case 2: return xdrag_t<float, 2>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
-        default: return xdrag_t<float, 3>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme);
+        case 1: return xdrag_t<float, 1>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
+        case 2: return xdrag_t<float, 2>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
+        default: return xdrag_t<float, 3>(L, geo, phys, G, D, rho_g, rho_d, acc, B, S, scheme, launches);
     }
 }
 
