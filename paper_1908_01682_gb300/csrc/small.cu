@@ -268,17 +268,20 @@ __global__ void __launch_bounds__(kSmallThreads, 1) k_step_small(const SmallArgs
     const uint32_t rank = blockIdx.x * blockDim.x + threadIdx.x, count = gridDim.x * blockDim.x;
     const uint32_t n = B.ng + B.nd;
 
-    // a step behind one whose barrier gave up does nothing (it finds its
-    // counts and its barrier half done)
+    // The scan runs on the counts that the last step left while the words that
+    // tell whether it did are on their way (0.9 us a step at 2 x 20011); else it
+    // runs again behind a count. A step behind one whose barrier gave up does
+    // nothing (it finds its counts and its barrier half done).
     const int err = *reinterpret_cast<volatile int *>(B.err);
     const int counted = *reinterpret_cast<volatile int *>(B.counted);
+    small_scan(B, wtot);
     if (err & kErrTimeout) return;
     if (!counted) {
         for (uint32_t i = rank; i < n; i += count)
             count_add_agg(i < B.ng ? &B.gcnt[B.gkey[i]] : &B.dcnt[B.dkey[i - B.ng]]);
         if (!barrier()) return;
+        small_scan(B, wtot);
     }
-    small_scan(B, wtot);
     if (!barrier()) return;
     for (uint32_t i = rank; i < n; i += count) {
         if (i < B.ng) scatter_one_agg(i, B.gkey, B.gia, B.gcnt, B.gstart, B.gsrc, B.gtid, B.ng, B.err);

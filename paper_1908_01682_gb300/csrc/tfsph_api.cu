@@ -222,7 +222,9 @@ int stage_inputs(tfsph_ctx *c, const void *const *arrs, int narr, int64_t n, con
 cudaError_t clear_counts(tfsph_ctx *c) { return cudaMemsetAsync(c->counts, 0, c->counts_bytes, c->stream); }
 
 // Loads a full particle state, computes keys and checks it (synchronises).
-int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, const uint8_t *frozen, int mem_kind)
+// replaced: arrays of the context have been written, refused or not.
+int load_arrays(tfsph_ctx *c, const void *const *gas, const void *const *dust, const uint8_t *frozen, int mem_kind,
+                bool *replaced)
 {
     if (mem_kind != TFSPH_MEM_HOST && mem_kind != TFSPH_MEM_DEVICE) return fail(c, TFSPH_E_INVALID_ARG, "bad mem_kind");
     if ((c->G.n > 0 && !gas) || (c->D.n > 0 && !dust)) return fail(c, TFSPH_E_INVALID_ARG, "NULL array list");
@@ -240,6 +242,7 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     if (rc) return rc;
     // from here on the state is replaced, whether its check accepts it or not:
     // nothing of the one before it may be taken for its own
+    *replaced = true;
     c->G.cur = 0;
     c->D.cur = 0;
     c->prepared = false;
@@ -256,7 +259,6 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     }
     c->has_frozen = any_frozen;
     PhaseBufs G = c->G;
-    if (c->counted) TF_CUDA(c, clear_counts(c));
     // the flags are zero between loads, unless one failed before they were read
     if (c->flags_dirty) TF_CUDA(c, cudaMemsetAsync(c->d_flags, 0, sizeof(int), c->stream));
     c->flags_dirty = true;
@@ -281,6 +283,15 @@ int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, co
     c->lost = false;
     c->steps = 0;
     return TFSPH_OK;
+}
+
+int load_state(tfsph_ctx *c, const void *const *gas, const void *const *dust, const uint8_t *frozen, int mem_kind)
+{
+    bool replaced = false;
+    const int rc = load_arrays(c, gas, dust, frozen, mem_kind, &replaced);
+    // (behind the load's synchronisation, where the host does not wait for it)
+    if (replaced && c->counted) TF_CUDA(c, clear_counts(c));
+    return rc;
 }
 
 int fold_profile(tfsph_ctx *c)
