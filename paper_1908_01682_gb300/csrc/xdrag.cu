@@ -512,7 +512,7 @@ k_scattered(Geo<float> G, const float4 *__restrict__ gpos, uint32_t ng, const fl
     float s[kSums] = {};
     for (uint32_t i = threadIdx.x; i < m; i += blockDim.x) {
         // in scattered order (evenly spaced slots may all be the first of their cell)
-        const float4 p = pos[(uint32_t)((uint64_t)i * 2654435761ull % n)];
+        const float4 p = pos[__umulhi(i * 2654435761u, n)];
         const float x[3] = {p.x, p.y, p.z};
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
