@@ -4,13 +4,9 @@ gives (one off the stored one included) and however close 2h is to a whole
 number of cells; no neighbour is left out; and a particle far outside the box
 is told from those the margins hold for."""
 import ctypes as C
-import os
 import subprocess
 
 import pytest
-
-ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-CSRC = os.path.join(ROOT, "paper_1908_01682_gb300", "csrc")
 
 SRC = r"""
 #include <string>
