@@ -94,3 +94,20 @@ def test_order_of_the_sums(case, viscous, prec):
         w.params.update(av_alpha=1.0, av_beta=2.0)
     w.tau = 1e-5
     _same(_states(b, _stir(w, 0.5)))
+
+
+@pytest.mark.parametrize("cell_acc", [0, 1])
+@pytest.mark.parametrize("harmonic", [0, 1])
+@pytest.mark.parametrize("case,size,cell,prec", [
+    ("wave", 1000, 0.9, 0), ("wave", 1000, 0.9, 1), ("wave", 9000, 1.0, 0), ("wave", 9000, 1.0, 1), ("wave", 60, 1.0, 1),
+    ("wave", 4000, 0.4, 0), ("column", 40, 0.8, 0), ("column", 40, 0.8, 1), ("column", 100, 1.0, 0), ("column", 24, 3.0, 1),
+    ("wave", 12000, 12.0, 1)])
+def test_cells_of_few_and_many_particles(case, size, cell, prec, harmonic, cell_acc):
+    """One lane per cell and four give the cell's sums and solve in the same roundings."""
+    b = gpu_lib()
+    w = workloads.dustywave(n=size, precision=prec, amp=1e-2, cell_factor=cell) if case == "wave" else \
+        workloads.column2d(nside=size, precision=prec, cell_factor=cell)
+    w.params.update(tstar_mode=harmonic, cell_acc=cell_acc)
+    rng = np.random.default_rng(3)
+    w.tstop = (w.tstop * np.exp(rng.uniform(-2, 2, w.n_dust))).astype(np.float32).astype(np.float64)
+    _same(_states(b, _stir(w, 0.3)))
